@@ -297,7 +297,7 @@ int chebfi_apply_H_noalloc(chebfi_ctx* ctx, const void* Y, void* HY, int64_t nb,
  * 2^-E ||row of op(A)|| ||column of op(B)|| per entry, E = 53 with the default 14 moduli:
  * no larger than an FP64 dot product's.  The paper (FP64 BLAS on CPUs) has no counterpart. */
 enum {
-  CHEBFI_GEMM_AUTO = 0,        /* tensor cores when K >= 64 and 8 M N K >= 1e9, else CUDA cores */
+  CHEBFI_GEMM_AUTO = 0,        /* tensor cores when K >= 64 and 8 M N K >= 6e7, else CUDA cores */
   CHEBFI_GEMM_CUDA_CORES = 1,  /* FP64 FMA on the CUDA cores only */
   CHEBFI_GEMM_TENSOR = 2       /* the modular emulation for every product */
 };

@@ -167,11 +167,15 @@ template <> struct Ops<float> {
 // ------------------------------------------------------------------ FP64 GEMM routing
 // FP64 complex GEMMs large enough to amortise the operand preparation run on the tensor
 // cores through the modular emulation (ozaki.cu), the others on the CUDA cores; the context
-// can force either engine (chebfi_set_fp64_gemm).
+// can force either engine (chebfi_set_fp64_gemm).  The line: the CUDA cores need 12 us +
+// 8 M N K / 1.1 TFLOP/s, the emulation 45 us of launches plus its operands, and they meet
+// between 3e7 and 6e7 flops (128 x 256 x 128: 42 against 50 us; 192^3: 58 / 52; 256 x 128 x
+// 256: 73 / 50; 256^3: 138 / 54; 256 x 16 x 8000: 235 / 165; 512^3: 903 / 90).  Below
+// K = 64 the reconstruction of the output outweighs the product.
 bool use_tensor_fp64(const chebfi_ctx* ctx, int64_t M, int64_t N, int64_t K) {
   if (M <= 0 || N <= 0 || K <= 0 || ctx->fp64_gemm == CHEBFI_GEMM_CUDA_CORES) return false;
   if (ctx->fp64_gemm == CHEBFI_GEMM_TENSOR) return true;
-  return K >= 64 && 8.0 * (double)M * (double)N * (double)K >= 1e9;
+  return K >= 64 && 8.0 * (double)M * (double)N * (double)K >= 6e7;
 }
 
 // residues of P^H (conj) or P as the A operand, kept while the modulus count is unchanged

@@ -2,9 +2,9 @@
 //
 // Used for the FP64 and FP32 forms of the projector products P^H psi and P W
 // (Algorithm 1, Section 5.1), the Woodbury core products, and the subspace matrices and
-// rotations of Algorithm 2.  64 x 64 output tiles, 256 threads, 4 x 4 complex outputs per
-// thread; split-K with a deterministic second pass when the output has too few tiles to
-// fill the 152 SMs.
+// rotations of Algorithm 2.  FP32: 64 x 64 output tiles, 256 threads, 4 x 4 complex outputs
+// per thread.  FP64: 256 outputs per tile, one per thread (k_gemm_d).  Both split K, with a
+// deterministic second pass, when the output has too few tiles to fill the 152 SMs.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -110,18 +110,103 @@ __global__ void __launch_bounds__(256) k_gemm(int64_t M, int64_t N, int64_t K, R
   }
 }
 
-template <typename R>
-__global__ void k_splitk_reduce(int64_t M, int64_t N, int splits, const cplx<R>* __restrict__ ws, R beta,
-                                cplx<R>* __restrict__ Cm, int64_t ldc) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= M * N) return;
-  const int64_t i = idx % M, j = idx / M;
-  cplx<R> r = cmake<cplx<R>>(0.0, 0.0);
-  for (int z = 0; z < splits; ++z) {
-    const cplx<R> v = ws[(int64_t)z * M * N + idx];
-    r.x += v.x;
-    r.y += v.y;
+// FP64: one output per thread, TM x TN = 256 outputs per block.  GB300 issues about two FP64
+// FMAs per clock and SM, so a block's 16-step k tile keeps the unit busy for 8192 clocks on
+// 8 KB of operands: reuse in registers gains nothing, and what counts is that no work is
+// spent on padding and that every SM has blocks.  Small tiles (8 x 32, 16 x 16 or 32 x 8,
+// whichever pads the output least) and a split of K down to 16 products do that; 64 x 64
+// tiles spent 16 times the needed FMAs on an 8 x 32 product and ran it on one SM
+// (8 x 32 x 1021: 4.13 ms, now 0.010 ms and 0.008 ms for its reduction; 256 x 256 x 256:
+// 1.04 ms on 16 SMs, now 0.14 ms).
+constexpr int KD = 16;
+template <int TM, int TN, bool CA, bool CB>
+__global__ void __launch_bounds__(256) k_gemm_d(int64_t M, int64_t N, int64_t K, double alpha,
+                                                const double2* __restrict__ A, int64_t lda,
+                                                const double2* __restrict__ B, int64_t ldb, double beta,
+                                                double2* __restrict__ Cm, int64_t ldc, int64_t kchunk,
+                                                double2* __restrict__ ws, int lower, int tiles_m, int tiles_n,
+                                                int n_fastest) {
+  static_assert(TM * TN == 256, "one output per thread");
+  const int64_t tile_i = n_fastest ? blockIdx.x / tiles_n : blockIdx.x % tiles_m;
+  const int64_t tile_j = n_fastest ? blockIdx.x % tiles_n : blockIdx.x / tiles_m;
+  const int64_t i0 = tile_i * TM, j0 = tile_j * TN;
+  if (lower && i0 + TM - 1 < j0) return;  // tile strictly above the diagonal
+  __shared__ double2 As[KD][TM + 1];
+  __shared__ double2 Bs[KD][TN + 1];
+  const int tid = threadIdx.x, tx = tid % TM, ty = tid / TM;
+  const int64_t kbeg = (int64_t)blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
+  const double2 zero = make_double2(0.0, 0.0);
+  double re = 0.0, im = 0.0;
+  for (int64_t k0 = kbeg; k0 < kend; k0 += KD) {
+#pragma unroll
+    for (int e = tid; e < TM * KD; e += 256) {
+      const int i = CA ? e / KD : e % TM, k = CA ? e % KD : e / TM;
+      const int64_t gi = i0 + i, gk = k0 + k;
+      double2 v = zero;
+      if (gi < M && gk < kend) v = CA ? ld_op(A + gk + gi * lda, true) : A[gi + gk * lda];
+      As[k][i] = v;
+    }
+#pragma unroll
+    for (int e = tid; e < TN * KD; e += 256) {
+      const int j = CB ? e % TN : e / KD, k = CB ? e / TN : e % KD;
+      const int64_t gj = j0 + j, gk = k0 + k;
+      double2 v = zero;
+      if (gj < N && gk < kend) v = CB ? ld_op(B + gj + gk * ldb, true) : B[gk + gj * ldb];
+      Bs[k][j] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {
+      const double2 a = As[k][tx], b = Bs[k][ty];
+      re = fma(a.x, b.x, re);
+      im = fma(a.x, b.y, im);
+      re = fma(-a.y, b.y, re);
+      im = fma(a.y, b.x, im);
+    }
+    __syncthreads();
   }
+  const int64_t gi = i0 + tx, gj = j0 + ty;
+  if (gi >= M || gj >= N) return;
+  double2 r = make_double2(alpha * re, alpha * im);
+  if (ws) {
+    ws[(int64_t)blockIdx.z * M * N + gi + gj * M] = r;
+    return;
+  }
+  if (beta != 0.0) {
+    const double2 c = Cm[gi + gj * ldc];
+    r.x = fma(beta, c.x, r.x);
+    r.y = fma(beta, c.y, r.y);
+  }
+  Cm[gi + gj * ldc] = r;
+}
+
+// C = sum_z ws[z] + beta C.  32 outputs per block; eight threads per output each add every
+// eighth split, their partial sums are added in a fixed order: one thread per output is a
+// chain of up to 64 dependent loads and slow FP64 additions (16 us at 64 splits of 8 x 32, now 8 us).
+template <typename R>
+__global__ void __launch_bounds__(256) k_splitk_reduce(int64_t M, int64_t N, int splits, const cplx<R>* __restrict__ ws,
+                                                       R beta, cplx<R>* __restrict__ Cm, int64_t ldc) {
+  __shared__ cplx<R> part[8][33];
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const int64_t idx = (int64_t)blockIdx.x * 32 + tx;
+  cplx<R> r = cmake<cplx<R>>(0.0, 0.0);
+  if (idx < M * N) {
+#pragma unroll 4
+    for (int z = ty; z < splits; z += 8) {
+      const cplx<R> v = ws[(int64_t)z * M * N + idx];
+      r.x += v.x;
+      r.y += v.y;
+    }
+  }
+  part[ty][tx] = r;
+  __syncthreads();
+  if (ty != 0 || idx >= M * N) return;
+#pragma unroll
+  for (int z = 1; z < 8; ++z) {
+    r.x += part[z][tx].x;
+    r.y += part[z][tx].y;
+  }
+  const int64_t i = idx % M, j = idx / M;
   if (beta != (R)0) {
     const cplx<R> c = Cm[i + j * ldc];
     r.x = fma(beta, c.x, r.x);
@@ -160,8 +245,52 @@ void launch(int64_t M, int64_t N, int64_t K, double alpha, const cplx<R>* A, int
                                                           wsp, lower ? 1 : 0, n_fastest ? 1 : 0));
   if (splits > 1) {
     const int64_t tot = M * N;
-    CHEBFI_LAUNCH("k_splitk_reduce", st, k_splitk_reduce<R><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(M, N, splits, wsp, (R)beta, Cm, ldc));
+    CHEBFI_LAUNCH("k_splitk_reduce", st, k_splitk_reduce<R><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, splits, wsp, (R)beta, Cm, ldc));
   }
+}
+
+// the FP64 tile shape with the least padded output: 16 x 16, 8 x 32 (few rows), 32 x 8
+template <bool CA, bool CB>
+void launch_d(int64_t M, int64_t N, int64_t K, double alpha, const double2* A, int64_t lda, const double2* B,
+              int64_t ldb, double beta, double2* Cm, int64_t ldc, cudaStream_t st, DevBuf<double2>* ws,
+              const char* tag, bool lower) {
+  auto padded = [&](int64_t tm, int64_t tn) { return (M + tm - 1) / tm * ((N + tn - 1) / tn); };
+  int64_t TM = 16, TN = 16;
+  if (padded(8, 32) < padded(TM, TN)) { TM = 8; TN = 32; }
+  if (padded(32, 8) < padded(TM, TN)) { TM = 32; TN = 8; }
+  const int64_t tm = (M + TM - 1) / TM, tn = (N + TN - 1) / TN, tiles = tm * tn;
+  // two blocks per SM; a split is at least one k tile
+  int64_t splits = 1;
+  if (ws && tiles < 304) splits = std::max<int64_t>(1, std::min<int64_t>((304 + tiles - 1) / tiles, (K + KD - 1) / KD));
+  int64_t kchunk = std::max<int64_t>(KD, ((K + splits - 1) / splits + KD - 1) / KD * KD);
+  splits = std::max<int64_t>(1, (K + kchunk - 1) / kchunk);
+  double2* wsp = nullptr;
+  if (splits > 1) {
+    ws->alloc((size_t)(splits * M * N));
+    wsp = ws->p;
+  }
+  const bool n_fastest = tm > 4 * tn;
+  CHEBFI_REQUIRE(tiles < (1ll << 31), CHEBFI_ERR_ARG, "GEMM too large");
+  const dim3 grid((unsigned)tiles, 1, (unsigned)splits);
+  const double tiles_done = lower ? 0.5 * (1.0 + 1.0 / (double)tm) : 1.0;
+  auto go = [&](auto kernel) {
+    CHEBFI_LAUNCH_W(tag, st, 8.0 * (double)M * (double)N * (double)K * tiles_done,
+                    kernel<<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, Cm, ldc, kchunk, wsp,
+                                                 lower ? 1 : 0, (int)tm, (int)tn, n_fastest ? 1 : 0));
+  };
+  if (TM == 8) go(k_gemm_d<8, 32, CA, CB>);
+  else if (TM == 32) go(k_gemm_d<32, 8, CA, CB>);
+  else go(k_gemm_d<16, 16, CA, CB>);
+  if (splits > 1) {
+    const int64_t tot = M * N;
+    CHEBFI_LAUNCH("k_splitk_reduce", st,
+                  k_splitk_reduce<double><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, (int)splits, wsp, beta, Cm, ldc));
+  }
+}
+
+template <typename R, bool CA, bool CB, typename... Args> void route(Args... args) {
+  if constexpr (sizeof(R) == 8) launch_d<CA, CB>(args...);
+  else launch<R, CA, CB>(args...);
 }
 
 }  // namespace
@@ -172,10 +301,10 @@ void gemm(bool conjA, bool conjB, int64_t M, int64_t N, int64_t K, double alpha,
           DevBuf<cplx<R>>* ws, const char* tag, bool lower) {
   if (M <= 0 || N <= 0) return;
   CHEBFI_REQUIRE(!lower || M == N, CHEBFI_ERR_ARG, "lower-triangle GEMM needs a square result");
-  if (conjA && conjB) launch<R, true, true>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
-  else if (conjA) launch<R, true, false>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
-  else if (conjB) launch<R, false, true>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
-  else launch<R, false, false>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
+  if (conjA && conjB) route<R, true, true>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
+  else if (conjA) route<R, true, false>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
+  else if (conjB) route<R, false, true>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
+  else route<R, false, false>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, ws, tag, lower);
 }
 
 template void gemm<double>(bool, bool, int64_t, int64_t, int64_t, double, const double2*, int64_t, const double2*,
