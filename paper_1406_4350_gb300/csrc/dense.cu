@@ -27,9 +27,14 @@ __device__ __forceinline__ void flag_error(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
 }
 
-// Unblocked Cholesky of one nb x nb diagonal block (nb <= NB) in shared memory.
-__global__ void k_chol_diag(double2* A, int64_t lda, int nb, int* status) {
+// Unblocked Cholesky of one nb x nb diagonal block (nb <= NB) in shared memory.  One block:
+// the pivots are a serial chain, and GB300's FP64 unit (about two FMAs per clock) makes each
+// square root and division ~10 dependent slow instructions.  Only 1 / sqrt(d) is on the
+// chain (the column is scaled by it); the diagonal's sqrt(d) is another warp's work
+// (32 x 32: 66 us with sqrt and a division per entry on the chain, now 39 us).
+__global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int nb, int* status) {
   __shared__ double2 a[NB][NB + 1];
+  __shared__ double rpiv;
   const int tid = threadIdx.x;
   for (int e = tid; e < nb * nb; e += blockDim.x) {
     const int i = e % nb, j = e / nb;
@@ -37,31 +42,36 @@ __global__ void k_chol_diag(double2* A, int64_t lda, int nb, int* status) {
   }
   __syncthreads();
   for (int j = 0; j < nb; ++j) {
-    __shared__ double piv;
+    const double d0 = a[j][j].x;
+    const double d = d0 > 0.0 ? d0 : 1.0;  // also catches NaN
     if (tid == 0) {
-      double d = a[j][j].x;
-      if (!(d > 0.0)) {  // also catches NaN
-        flag_error(status, CHEBFI_ERR_NOT_SPD);
-        d = 1.0;
-      }
-      piv = sqrt(d);
-      a[j][j] = make_double2(piv, 0.0);
+      if (!(d0 > 0.0)) flag_error(status, CHEBFI_ERR_NOT_SPD);
+      rpiv = rsqrt(d);
     }
+    const double piv = tid == 32 ? sqrt(d) : 0.0;
     __syncthreads();
+    if (tid == 32) a[j][j] = make_double2(piv, 0.0);
     for (int i = j + 1 + tid; i < nb; i += blockDim.x) {
-      a[i][j].x /= piv;
-      a[i][j].y /= piv;
+      a[i][j].x *= rpiv;
+      a[i][j].y *= rpiv;
     }
     __syncthreads();
-    // trailing update of the lower triangle: a[i][k] -= L[i][j] conj(L[k][j]) for i >= k > j
+    // trailing update of the lower triangle: a[i][k] -= L[i][j] conj(L[k][j]) for i >= k > j.
+    // Its m columns are folded in pairs (q, m - 1 - q) of m + 1 entries together, so that no
+    // lane of the slow FP64 instructions is spent above the diagonal.
     const int m = nb - j - 1;
-    for (int e = tid; e < m * m; e += blockDim.x) {
-      const int i = j + 1 + e % m, k = j + 1 + e / m;
-      if (i >= k) {
-        const double2 li = a[i][j], lk = a[k][j];
-        a[i][k].x -= li.x * lk.x + li.y * lk.y;
-        a[i][k].y -= li.y * lk.x - li.x * lk.y;
-      }
+    for (int e = tid; e < (m + 1) * ((m + 1) / 2); e += blockDim.x) {
+      const int q = e / (m + 1), c = e - q * (m + 1);
+      const bool first = c < m - q;
+      if (!first && m - 1 - q == q) continue;  // the middle column of an odd m has no partner
+      const int k = j + 1 + (first ? q : m - 1 - q), i = first ? k + c : k + c - (m - q);
+      const double2 li = a[i][j], lk = a[k][j];
+      double2 v = a[i][k];
+      v.x = fma(-li.x, lk.x, v.x);
+      v.y = fma(-li.y, lk.x, v.y);
+      v.x = fma(-li.y, lk.y, v.x);
+      v.y = fma(li.x, lk.y, v.y);
+      a[i][k] = v;
     }
     __syncthreads();
   }
@@ -71,75 +81,65 @@ __global__ void k_chol_diag(double2* A, int64_t lda, int nb, int* status) {
   }
 }
 
-// Panel: rows of B (m x nb) <- B L^{-H}, L = nb x nb lower (diagonal real).
-__global__ void k_trsm_right_lh(const double2* __restrict__ L, int64_t ldl, double2* B, int64_t ldb, int64_t m, int nb) {
-  __shared__ double2 l[NB][NB + 1];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e % nb, j = e / nb;
-    l[i][j] = L[i + j * ldl];
-  }
-  __syncthreads();
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= m) return;
-  double2 x[NB];
-#pragma unroll
-  for (int j = 0; j < NB; ++j)
-    if (j < nb) x[j] = B[r + j * ldb];
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    if (j < nb) {
-      double2 s = x[j];
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-        if (k < j) {  // s -= x_k conj(L[j][k])
-          const double2 lj = l[j][k];
-          s.x -= x[k].x * lj.x + x[k].y * lj.y;
-          s.y -= x[k].y * lj.x - x[k].x * lj.y;
-        }
-      }
-      const double d = l[j][j].x;
-      x[j] = make_double2(s.x / d, s.y / d);
+// The two triangular solves with an nb x nb lower L (diagonal real), one system per warp: the
+// lanes hold its unknowns, and step k broadcasts x_k = s_k / L_kk to the lanes that still
+// need it.  A system is a serial chain of nb slow FP64 steps, so systems are spread over the
+// SMs (four warps a block) instead of one per thread, which kept 128 of them on one SM
+// (224 x 32: 131 and 172 us with a thread per system, now 18 us).
+constexpr int kTrsmWarps = 4;
+// x_l <- x_l - sum_{k < l} c_lk x_k solved forward; c_lk = L[l][k], or its conjugate
+template <bool CONJ>
+__device__ __forceinline__ double2 warp_forward(const double2 (*l)[NB + 1], const double* rd, double2 x, int nb) {
+  const int lane = threadIdx.x % 32;
+  for (int k = 0; k < nb; ++k) {
+    const double r = rd[k];
+    const double2 xk = make_double2(__shfl_sync(0xffffffffu, x.x, k) * r, __shfl_sync(0xffffffffu, x.y, k) * r);
+    double2 c = l[lane][k];  // L is lower triangular: zero above, and rows >= nb are zero
+    if (CONJ) c.y = -c.y;
+    if (lane == k) x = xk;
+    else if (lane > k) {
+      x.x = fma(-c.x, xk.x, fma(c.y, xk.y, x.x));
+      x.y = fma(-c.x, xk.y, fma(-c.y, xk.x, x.y));
     }
   }
-#pragma unroll
-  for (int j = 0; j < NB; ++j)
-    if (j < nb) B[r + j * ldb] = x[j];
+  return x;
+}
+__device__ __forceinline__ void load_tri(const double2* __restrict__ L, int64_t ldl, int nb, double2 (*l)[NB + 1],
+                                         double* rd) {
+  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
+    const int i = e % NB, j = e / NB;
+    l[i][j] = i < nb && j < nb ? L[i + j * ldl] : make_double2(0.0, 0.0);
+    if (i == j) rd[i] = i < nb ? 1.0 / L[i + j * ldl].x : 0.0;
+  }
+  __syncthreads();
 }
 
-// Columns of B (nb x m) <- L^{-1} B, L = nb x nb lower.
-__global__ void k_trsm_left_l(const double2* __restrict__ L, int64_t ldl, double2* B, int64_t ldb, int64_t m, int nb) {
+// Panel: rows of B (m x nb) <- B L^{-H}; row r of X solves conj(L) x = b.
+__global__ void __launch_bounds__(32 * kTrsmWarps) k_trsm_right_lh(const double2* __restrict__ L, int64_t ldl, double2* B, int64_t ldb, int64_t m,
+                                                                  int nb) {
   __shared__ double2 l[NB][NB + 1];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e % nb, j = e / nb;
-    l[i][j] = L[i + j * ldl];
-  }
-  __syncthreads();
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ double rd[NB];
+  load_tri(L, ldl, nb, l, rd);
+  const int lane = threadIdx.x % 32;
+  const int64_t r = (int64_t)blockIdx.x * kTrsmWarps + threadIdx.x / 32;
+  if (r >= m) return;
+  double2 x = lane < nb ? B[r + lane * ldb] : make_double2(0.0, 0.0);
+  x = warp_forward<true>(l, rd, x, nb);
+  if (lane < nb) B[r + lane * ldb] = x;
+}
+
+// Columns of B (nb x m) <- L^{-1} B.
+__global__ void __launch_bounds__(32 * kTrsmWarps) k_trsm_left_l(const double2* __restrict__ L, int64_t ldl, double2* B, int64_t ldb, int64_t m,
+                                                                int nb) {
+  __shared__ double2 l[NB][NB + 1];
+  __shared__ double rd[NB];
+  load_tri(L, ldl, nb, l, rd);
+  const int lane = threadIdx.x % 32;
+  const int64_t c = (int64_t)blockIdx.x * kTrsmWarps + threadIdx.x / 32;
   if (c >= m) return;
-  double2 x[NB];
-  double2* b = B + c * ldb;
-#pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < nb) x[i] = b[i];
-#pragma unroll
-  for (int i = 0; i < NB; ++i) {
-    if (i < nb) {
-      double2 s = x[i];
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-        if (k < i) {  // s -= L[i][k] x_k
-          const double2 li = l[i][k];
-          s.x -= li.x * x[k].x - li.y * x[k].y;
-          s.y -= li.x * x[k].y + li.y * x[k].x;
-        }
-      }
-      const double d = l[i][i].x;
-      x[i] = make_double2(s.x / d, s.y / d);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < nb) b[i] = x[i];
+  double2 x = lane < nb ? B[lane + c * ldb] : make_double2(0.0, 0.0);
+  x = warp_forward<false>(l, rd, x, nb);
+  if (lane < nb) B[lane + c * ldb] = x;
 }
 
 __global__ void k_zero_upper(int64_t n, double2* A, int64_t lda) {
@@ -921,9 +921,9 @@ void cholesky(int64_t n, double2* A, int64_t lda, int* status, cudaStream_t st, 
     const int64_t m2 = n - k0 - nb;
     if (m2 > 0) {
       double2* L21 = A + (k0 + nb) + k0 * lda;
-      CHEBFI_LAUNCH("k_trsm_right_lh", st, k_trsm_right_lh<<<nblk(m2, 128), 128, 0, st>>>(A + k0 + k0 * lda, lda, L21, lda, m2, nb));
+      CHEBFI_LAUNCH("k_trsm_right_lh", st, k_trsm_right_lh<<<nblk(m2, kTrsmWarps), 32 * kTrsmWarps, 0, st>>>(A + k0 + k0 * lda, lda, L21, lda, m2, nb));
       gemm<double>(false, true, m2, m2, nb, -1.0, L21, lda, L21, lda, 1.0, A + (k0 + nb) + (k0 + nb) * lda, lda, st,
-                   ws);
+                   ws, "k_gemm", true);
     }
   }
   CHEBFI_LAUNCH("k_zero_upper", st, k_zero_upper<<<nblk(n * n), 256, 0, st>>>(n, A, lda));
@@ -933,7 +933,7 @@ void trsm_lower(int64_t n, int64_t m, const double2* L, int64_t ldl, double2* B,
                 DevBuf<double2>* ws) {
   for (int64_t k0 = 0; k0 < n; k0 += NB) {
     const int nb = (int)std::min<int64_t>(NB, n - k0);
-    CHEBFI_LAUNCH("k_trsm_left_l", st, k_trsm_left_l<<<nblk(m, 128), 128, 0, st>>>(L + k0 + k0 * ldl, ldl, B + k0, ldb, m, nb));
+    CHEBFI_LAUNCH("k_trsm_left_l", st, k_trsm_left_l<<<nblk(m, kTrsmWarps), 32 * kTrsmWarps, 0, st>>>(L + k0 + k0 * ldl, ldl, B + k0, ldb, m, nb));
     const int64_t m2 = n - k0 - nb;
     if (m2 > 0)
       gemm<double>(false, false, m2, m, nb, -1.0, L + (k0 + nb) + k0 * ldl, ldl, B + k0, ldb, 1.0, B + k0 + nb, ldb, st,
