@@ -182,7 +182,7 @@ bool use_tensor_fp64(const chebfi_ctx* ctx, int64_t M, int64_t N, int64_t K) {
 const OzOperand& oz_P(chebfi_ctx* ctx, bool conj, cudaStream_t st) {
   OzOperand& o = conj ? ctx->ozPh : ctx->ozP;
   if (o.nmod != ctx->oz_nmod)
-    oz_prepare(ctx->d_P.p, ctx->npw, conj ? ctx->nproj : ctx->npw, conj ? ctx->npw : ctx->nproj, conj, conj, true,
+    oz_prepare(ctx->d_P.p, ctx->npw, conj ? ctx->nproj : ctx->npw, conj ? ctx->npw : ctx->nproj, conj, conj,
                ctx->oz_nmod, o, st);
   return o;
 }
@@ -200,8 +200,8 @@ void gemm64(chebfi_ctx* ctx, bool conjA, bool conjB, int64_t M, int64_t N, int64
   const bool is_P = ctx->has_proj && A == ctx->d_P.p && lda == ctx->npw &&
                     (conjA ? (M == ctx->nproj && K == ctx->npw) : (M == ctx->npw && K == ctx->nproj));
   if (is_P) a = &oz_P(ctx, conjA, st);
-  else oz_prepare(A, lda, M, K, conjA, conjA, true, ctx->oz_nmod, z.A, st);
-  oz_prepare(B, ldb, N, K, !conjB, conjB, false, ctx->oz_nmod, z.B, st);
+  else oz_prepare(A, lda, M, K, conjA, conjA, ctx->oz_nmod, z.A, st);
+  oz_prepare(B, ldb, N, K, !conjB, conjB, ctx->oz_nmod, z.B, st);
   oz_gemm(*a, z.B, alpha, beta, C, ldc, lower, z.R, ctx->d_status.p, st, tag);
 }
 

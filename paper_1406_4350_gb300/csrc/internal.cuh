@@ -166,18 +166,17 @@ struct TcGroupProb {
   int64_t ldc;
 };
 
-// Residues of a real-embedded complex operand for the modular tensor-core GEMM (ozaki.cu):
-// one K-major bf16 matrix per modulus, res[mod * mstride + row * ld + k], and per complex
-// row the power of two s applied before rounding to integers.
+// Residues of a complex operand for the modular tensor-core GEMM (ozaki.cu): three K-major
+// bf16 matrices per modulus (the residues of Re, Im and Re + Im), plane 3 mod + part at
+// res[(3 mod + part) * pstride + row * ld + k], and per row the power of two s applied before
+// rounding to integers.
 constexpr int kOzMinMod = 8, kOzMaxMod = 15;
 constexpr int kOzBadShift = -0x40000000;  // shift of a row holding Inf or NaN
 struct OzOperand {
   DevBuf<__nv_bfloat16> res;
   DevBuf<int32_t> shift;
-  int64_t crows = 0;   // complex rows
-  int64_t rows = 0;    // real rows (2 crows for the doubled A operand)
-  int64_t kreal = 0;   // reals per row (2 K)
-  int64_t ld = 0, mstride = 0;
+  int64_t rows = 0, K = 0;
+  int64_t ld = 0, pstride = 0;
   int nmod = 0;
 };
 struct OzWork {

@@ -122,11 +122,11 @@ void tc_cgemm3(const SplitBF16x3& A, const SplitBF16x3& B, bool conjA, int64_t M
 
 // ---------------------------------------------------------------- FP64-accurate GEMM on tensor cores (ozaki.cu)
 // Residues of op(X) (nrows x K complex; row r is column r of X when rows_are_columns, else
-// row r of X; conjugated if conj) for the modular GEMM; doubled: the A operand's two real
-// rows per complex row.  The scale makes every row's 2-norm 2^(E-1)..2^E, E = oz_precision_bits.
-void oz_prepare(const double2* X, int64_t ldx, int64_t nrows, int64_t K, bool rows_are_columns, bool conj,
-                bool doubled, int nmod, OzOperand& out, cudaStream_t st);
-// C = alpha op(A) op(B) + beta C (complex, M = A.crows, N = B.crows; lower: only the complex
+// row r of X; conjugated if conj) for the modular GEMM.  The scale makes every row's 2-norm
+// 2^(E-1)..2^E, E = oz_precision_bits.
+void oz_prepare(const double2* X, int64_t ldx, int64_t nrows, int64_t K, bool rows_are_columns, bool conj, int nmod,
+                OzOperand& out, cudaStream_t st);
+// C = alpha op(A) op(B) + beta C (complex, M = A.rows, N = B.rows; lower: only the complex
 // lower triangle of a square C is written) from prepared operands; R: residue workspace.
 void oz_gemm(const OzOperand& A, const OzOperand& B, double alpha, double beta, double2* C, int64_t ldc, bool lower,
              DevBuf<signed char>& R, int* status, cudaStream_t st, const char* tag);

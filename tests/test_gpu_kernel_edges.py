@@ -1,0 +1,99 @@
+"""Kernels at the edges of their tiles, blocks and dispatch ranges, against the oracle or a
+numpy product in extended precision.  Tolerances are the a-priori rounding bounds."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import chebyshev as ch
+from oracle.planewave import PWOperator
+from synth import make_cell
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1406_4350_gb300 import build
+    build.build()
+
+
+def _F(x):
+    from paper_1406_4350_gb300.chebfi import fortran
+    return fortran(x)
+
+
+def _np(t):
+    torch.cuda.synchronize()
+    return t.cpu().numpy()
+
+
+def _ctx(cell=None):
+    from paper_1406_4350_gb300.chebfi import ChebFI
+    return ChebFI.from_cell(cell) if cell is not None else ChebFI(0)
+
+
+def _rand(rng, m, n):
+    return rng.standard_normal((m, n)) + 1j * rng.standard_normal((m, n))
+
+
+# one entry; one short of, at and past the 8 x 32, 16 x 16 and 32 x 8 tiles; K below one k
+# tile, at it, past it, and long enough to be split to the last tile
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (8, 32, 1021), (9, 33, 16), (7, 31, 17), (32, 8, 300), (33, 7, 15),
+                                   (15, 17, 2049), (16, 16, 64), (1021, 32, 8), (300, 3, 40)])
+@pytest.mark.parametrize("conjA,conjB", [(False, False), (True, False), (False, True), (True, True)])
+def test_cuda_core_fp64_gemm(m, n, k, conjA, conjB):
+    from paper_1406_4350_gb300._lib import GEMM_CUDA_CORES
+    rng = np.random.default_rng(100 * m + 10 * n + k)
+    A = _rand(rng, k, m) if conjA else _rand(rng, m, k)
+    B = _rand(rng, n, k) if conjB else _rand(rng, k, n)
+    C0 = _rand(rng, m, n)
+    a = A.conj().T if conjA else A
+    b = B.conj().T if conjB else B
+    ref = 0.5 * (a.astype(np.clongdouble) @ b.astype(np.clongdouble)) + 2.0 * C0
+    g = _ctx()
+    g.set_fp64_gemm(GEMM_CUDA_CORES)
+    C = _np(g.gemm_fp64(_F(A), _F(B), conjA, conjB, alpha=0.5, beta=2.0, C=_F(C0)))
+    bound = (2 * k + 8) * U * (np.abs(a) @ np.abs(b) + 2.0 * np.abs(C0))
+    assert np.all(np.abs((C - ref).astype(complex)) <= 2.0 * bound)
+
+
+# one 32 x 32 diagonal block, its edges, two blocks, and the recursive factor's 256-leaf edge
+@pytest.mark.parametrize("nb", [1, 2, 31, 32, 33, 64, 95, 257])
+def test_cholesky_qr_block_edges(nb):
+    cell = make_cell(8.0, 20, 6.0, 2, 8, nb, True, 31)
+    op = PWOperator.from_cell(cell)
+    g = _ctx(cell)
+    Y = _F(cell.Y0)
+    g.orthonormalise(Y)
+    Yg = _np(Y)
+    # Y = Y0 L^-H with S-Gram L L^H: S-orthonormal, and Y^H S Y0 = L^H is upper triangular
+    # with a positive real diagonal
+    SY0 = op.apply_S(cell.Y0)
+    gram = cell.Y0.conj().T @ SY0
+    tol = 50.0 * nb * U * np.linalg.cond(gram)
+    np.testing.assert_allclose(Yg.conj().T @ op.apply_S(Yg), np.eye(nb), atol=tol)
+    LH = Yg.conj().T @ SY0
+    scale = np.sqrt(np.abs(np.diag(gram)).max())
+    assert np.abs(np.tril(LH, -1)).max(initial=0.0) <= tol * scale
+    assert np.all(np.diag(LH).real > 0) and np.abs(np.diag(LH).imag).max() <= tol * scale
+
+
+# the modular GEMM: one entry; one short of, at and past its 256-row tile, the 128-row halves
+# of a CTA pair, the 128- and 256-column forms; K below and past a k-tile and a 512-product
+# chunk, and long with few tiles (split over K); rows past M inside a group of four
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (127, 128, 63), (129, 129, 65), (256, 256, 512), (255, 257, 513),
+                                   (258, 300, 1030), (30, 7, 20001), (511, 127, 9000)])
+def test_modular_gemm_is_exact_on_integers(m, n, k):
+    from paper_1406_4350_gb300._lib import GEMM_TENSOR
+    rng = np.random.default_rng(m + n + k)
+    A = rng.integers(-1000, 1001, (k, m)) + 1j * rng.integers(-1000, 1001, (k, m))
+    B = rng.integers(-1000, 1001, (k, n)) + 1j * rng.integers(-1000, 1001, (k, n))
+    ar, ai = A.real.astype(np.int64).T, -A.imag.astype(np.int64).T
+    br, bi = B.real.astype(np.int64), B.imag.astype(np.int64)
+    g = _ctx()
+    g.set_fp64_gemm(GEMM_TENSOR, 14)
+    C = _np(g.gemm_fp64(_F(A), _F(B), conjA=True))
+    assert np.array_equal(C.real, (ar @ br - ai @ bi).astype(np.float64))
+    assert np.array_equal(C.imag, (ar @ bi + ai @ br).astype(np.float64))
