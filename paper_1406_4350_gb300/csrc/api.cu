@@ -573,15 +573,18 @@ void rq_sorted(chebfi_ctx* ctx, const double2* Y, int64_t nb, double* rq, cudaSt
 
 // Dense Hermitian eigenproblem of the Rayleigh-Ritz step (Algorithm 2; the paper calls
 // ELPA): A (n x n, ld n) -> ascending eigenvalues w and orthonormal eigenvectors X (ld n).
-// FP64 cyclic Jacobi for small n; from n = 512 up (or when selected) the FP32 Jacobi gives
+// FP64 cyclic Jacobi for n < 8; from there up (or when selected) the FP32 Jacobi gives
 // approximate vectors, which the iterative refinement of Ogita & Aishima (2018) brings to
 // FP64 accuracy with FP64 GEMMs (quadratic convergence, 2-4 steps), or, for a nearly
 // diagonal A, the refinement starts from the identity; pairs too close for its formula end
-// in a dense FP64 Jacobi of their cluster's block.  A is destroyed.
+// in a dense FP64 Jacobi of their cluster's block.  A is destroyed.  Rayleigh-Ritz with the
+// FP64 Jacobi / refined: n = 8 0.96 / 0.75 ms, 32 3.1 / 1.0, 128 24 / 5.0, 256 54 / 9.9,
+// 400 96 / 19 (the FP64 sweeps are n - 1 grid-wide rounds each on the slow FP64 unit).
+constexpr int64_t kRefineMin = 8;
 void eigh_rr(chebfi_ctx* ctx, int64_t n, double2* A, double* w, double2* X, cudaStream_t st) {
   Work& wk = ctx->w;
   int* status = ctx->d_status.p;
-  const bool refined = ctx->eig_mode == CHEBFI_EIG_REFINED || (ctx->eig_mode == CHEBFI_EIG_AUTO && n >= 512);
+  const bool refined = ctx->eig_mode == CHEBFI_EIG_REFINED || (ctx->eig_mode == CHEBFI_EIG_AUTO && n >= kRefineMin);
   ctx->eig_iters = 0;
   if (!refined || n < 2) {
     jacobi_eigh(n, A, n, w, X, n, status, st, &wk.small5);
@@ -592,7 +595,6 @@ void eigh_rr(chebfi_ctx* ctx, int64_t n, double2* A, double* w, double2* X, cuda
   constexpr int kCap = 1 << 16;
   wk.e32a.alloc(nn);
   wk.e32b.alloc(nn);
-  wk.e32w.alloc(n);
   wk.eG.alloc(nn);
   wk.eS.alloc(nn);
   wk.eAX.alloc(nn);
@@ -602,6 +604,45 @@ void eigh_rr(chebfi_ctx* ctx, int64_t n, double2* A, double* w, double2* X, cuda
   wk.estats.alloc(2);
   wk.enp.alloc(1);
   wk.epairs.alloc(kCap);
+  // the listed pairs' connected components as (offsets, columns) of those that one launch of
+  // small dense solves takes; the larger ones stay in `big`
+  std::vector<int> clusters;
+  int ncl = 0;
+  std::map<int, std::vector<int>> big;
+  auto find_clusters = [&](int npairs) {
+    std::vector<int2> hp(npairs);
+    CHEBFI_CUDA(cudaMemcpyAsync(hp.data(), wk.epairs.p, sizeof(int2) * npairs, cudaMemcpyDeviceToHost, st));
+    CHEBFI_CUDA(cudaStreamSynchronize(st));
+    std::vector<int> parent(n);
+    std::iota(parent.begin(), parent.end(), 0);
+    std::function<int(int)> find = [&](int v) { return parent[v] == v ? v : parent[v] = find(parent[v]); };
+    for (const int2& pr : hp) parent[find(pr.x)] = find(pr.y);
+    big.clear();
+    for (const int2& pr : hp) big[find(pr.x)];
+    for (int v = 0; v < (int)n; ++v) {
+      auto it = big.find(find(v));
+      if (it != big.end()) it->second.push_back(v);
+    }
+    clusters.assign(1, 0);
+    std::vector<int> list;
+    for (auto it = big.begin(); it != big.end();) {
+      if ((int)it->second.size() > max_cluster()) {
+        ++it;
+        continue;
+      }
+      list.insert(list.end(), it->second.begin(), it->second.end());
+      clusters.push_back((int)list.size());
+      it = big.erase(it);
+    }
+    ncl = (int)clusters.size() - 1;
+    clusters.insert(clusters.end(), list.begin(), list.end());
+  };
+  auto solve_clusters = [&](double2* X_, const double2* G) {
+    if (ncl == 0) return;
+    wk.eidx.upload(clusters.data(), clusters.size(), st);
+    cluster_solve(n, ncl, wk.eidx.p, wk.eidx.p + ncl + 1, wk.eS.p, G, X_, wk.elam.p, status, st);
+    CHEBFI_CUDA(cudaStreamSynchronize(st));  // the host list is reused
+  };
   DevBuf<double2>* ws = &wk.splitk;
   double2 *Xc = X, *Xn = wk.eX.p;
   bool conv = false;
@@ -627,6 +668,14 @@ void eigh_rr(chebfi_ctx* ctx, int64_t n, double2* A, double* w, double2* X, cuda
       ++ctx->eig_iters;
       // after an update of size emax the vectors are accurate to O(emax^2): below rounding
       conv = std::isfinite(emax) && emax <= 1e-10;
+      // A close pair that the step left unturned couples to its neighbours and would make the
+      // other entries converge linearly: turn it now (its block of this step's S is right to
+      // first order), so that the next step sees it diagonal.  2048 bands: 5-8 steps, or none
+      // and the FP64 Jacobi, become 4.
+      if (!conv && std::isfinite(emax) && npairs > 0 && npairs <= kCap) {
+        find_clusters(npairs);
+        solve_clusters(Xc, wk.eG.p);
+      }
     }
   };
   // Fast path: when A is already nearly diagonal (the later sweeps of a converging solve,
@@ -652,12 +701,13 @@ void eigh_rr(chebfi_ctx* ctx, int64_t n, double2* A, double* w, double2* X, cuda
   if (!conv) {
     // stage 1: FP32 Jacobi on a copy; stage 2: refinement from its vectors
     convert(n, n, A, n, wk.e32a.p, n, st);
-    jacobi_eigh_f32(n, wk.e32a.p, n, wk.e32w.p, wk.e32b.p, n, status, st, &wk.small5);
-    convert(n, n, wk.e32b.p, n, X, n, st);
-    Xc = X;
-    Xn = wk.eX.p;
-    ctx->eig_iters = 0;
-    refine(8);
+    if (jacobi_eigh_f32(n, wk.e32a.p, n, wk.e32b.p, n, st, &wk.small5)) {
+      convert(n, n, wk.e32b.p, n, X, n, st);
+      Xc = X;
+      Xn = wk.eX.p;
+      ctx->eig_iters = 0;
+      refine(8);
+    }
   }
   if (!conv || npairs > kCap) {
     // not converged (or too many near-equal pairs): the FP64 Jacobi of the original matrix
@@ -669,22 +719,11 @@ void eigh_rr(chebfi_ctx* ctx, int64_t n, double2* A, double* w, double2* X, cuda
   if (npairs > 0) {
     // clusters: connected components of the listed pairs; each block of X^H A X on a
     // component is diagonalised by FP64 Jacobi and its columns rotated
-    std::vector<int2> hp(npairs);
-    CHEBFI_CUDA(cudaMemcpyAsync(hp.data(), wk.epairs.p, sizeof(int2) * npairs, cudaMemcpyDeviceToHost, st));
     gemm64(ctx, false, false, n, n, n, 1.0, A, n, Xc, n, 0.0, wk.eAX.p, n, st, ws, "gemm_eig");
     gemm64(ctx, true, false, n, n, n, 1.0, Xc, n, wk.eAX.p, n, 0.0, wk.eS.p, n, st, ws, "gemm_eig");
-    CHEBFI_CUDA(cudaStreamSynchronize(st));
-    std::vector<int> parent(n);
-    std::iota(parent.begin(), parent.end(), 0);
-    std::function<int(int)> find = [&](int v) { return parent[v] == v ? v : parent[v] = find(parent[v]); };
-    for (const int2& pr : hp) parent[find(pr.x)] = find(pr.y);
-    std::map<int, std::vector<int>> comp;
-    for (const int2& pr : hp) {
-      comp[find(pr.x)];
-    }
-    for (int v = 0; v < (int)n; ++v)
-      if (comp.count(find(v))) comp[find(v)].push_back(v);
-    for (auto& kv : comp) {
+    find_clusters(npairs);
+    solve_clusters(Xc, nullptr);
+    for (auto& kv : big) {
       const std::vector<int>& idx = kv.second;
       const int k = (int)idx.size();
       wk.eidx.upload(idx.data(), k, st);

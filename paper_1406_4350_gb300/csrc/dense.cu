@@ -482,8 +482,9 @@ void jacobi_eigh_t(int64_t n0, cplx<R>* A, int64_t lda, R* w, cplx<R>* V, int64_
 //   E_ij = (S_ij - lambda_j G_ij) / (lambda_j - lambda_i)   (i != j; = (s_ij + lambda_j r_ij)/(...)),
 //   E_ii = (1 - G_ii) / 2,
 // and X <- X (I + E).  A pair whose gap is not large against its numerator (|gap| <=
-// 4 |num|, or below 1e-13 |A|) is treated as a cluster: E_ij = -G_ij / 2 only restores
-// orthogonality, and the pair is listed for a final dense solve of the cluster.
+// 16 |num|, below 1e-13 |A|, or a numerator at rounding level that still turns the pair by more
+// than 1e-8) is treated as a cluster: E_ij = -G_ij / 2 only restores orthogonality, and the
+// pair is listed for a dense solve of the cluster.
 __global__ void k_oa_lambda(int64_t n, const double2* __restrict__ G, int64_t ldg, const double2* __restrict__ S,
                             int64_t lds, double* __restrict__ lam, unsigned long long* __restrict__ amax) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -503,6 +504,7 @@ __global__ void k_oa_update(int64_t n, const double2* __restrict__ G, int64_t ld
   const double2 g = in ? G[i + j * ldg] : make_double2(1.0, 0.0);
   double2 e;
   double mag = 0.0;
+  bool quiet = false;
   if (!in) {
     e = make_double2(0.0, 0.0);
   } else if (i == j) {
@@ -513,9 +515,13 @@ __global__ void k_oa_update(int64_t n, const double2* __restrict__ G, int64_t ld
     const double lj = lam[j], gap = lj - lam[i];
     const double2 num = make_double2(s.x - lj * g.x, s.y - lj * g.y);
     const double anum = hypot(num.x, num.y);
-    const double tiny = 1e-13 * __longlong_as_double((long long)*amax);
-    if (fabs(gap) > 4.0 * anum && fabs(gap) > tiny) {
+    const double top = __longlong_as_double((long long)*amax);
+    // the numerator of exact eigenvectors is rounding noise of S (about 2^-53 |A| times a small
+    // constant); an update of that size is no sign of missing convergence
+    const bool noise = anum <= 2e-15 * top;
+    if (fabs(gap) > 16.0 * anum && fabs(gap) > 1e-13 * top && !(noise && anum > 1e-8 * fabs(gap))) {
       e = make_double2(num.x / gap, num.y / gap);
+      quiet = noise;
     } else {
       e = make_double2(-0.5 * g.x, -0.5 * g.y);
       if (i < j) {
@@ -523,7 +529,7 @@ __global__ void k_oa_update(int64_t n, const double2* __restrict__ G, int64_t ld
         if (k < cap) pairs[k] = make_int2((int)i, (int)j);
       }
     }
-    mag = hypot(e.x, e.y);
+    if (!quiet) mag = hypot(e.x, e.y);
   }
   // max |E| over the warp first (the bits of non-negative doubles order like their values,
   // a NaN above all), then one atomic per warp: one per element serialises on the word
@@ -579,19 +585,120 @@ __global__ void k_scatter_vals(int k, const int* __restrict__ idx, const double*
   if (b < k) dst[idx[b]] = src[b];
 }
 
+// ------------------------------------------------------------------ clusters (FP64)
+// Small dense problems of the refinement's clusters: one block per cluster c of k <= kMaxCluster
+// listed columns idx[off[c]..off[c + 1]).  The block S[idx, idx] is diagonalised in shared
+// memory by the cyclic Jacobi method above; lam[idx] gets its eigenvalues and
+// X[:, idx] <- X[:, idx] Z.  With G (inside the refinement, X^H X not yet the identity, lam the
+// step's values): the block of the basis that the step's -G / 2 orthogonalises, to first order
+// S_ij - (lam_i + lam_j) G_ij / 2 beside lam on the diagonal.  A symmetric crystal has dozens of 2- and 3-fold shells: one
+// launch for all of them instead of a cooperative eigensolve, three copies and a host
+// synchronisation each (about 0.2 ms apiece).
+constexpr int kMaxCluster = 32;
+__global__ void __launch_bounds__(256) k_cluster_solve(int64_t n, const int* __restrict__ off, const int* __restrict__ idx,
+                                                       const double2* __restrict__ S, const double2* __restrict__ G,
+                                                       double2* X, double* __restrict__ lam, int* status) {
+  constexpr int P = kMaxCluster + 1;
+  __shared__ double2 A[kMaxCluster * P], Z[kMaxCluster * P];
+  __shared__ RotT<double> rot[kMaxCluster / 2];
+  __shared__ int pairs[kMaxCluster];
+  __shared__ double norms[2];
+  const int* id = idx + off[blockIdx.x];
+  const int k = off[blockIdx.x + 1] - off[blockIdx.x], kp = k + (k & 1), tid = threadIdx.x;
+  for (int e = tid; e < k * k; e += blockDim.x) {
+    const int i = e % k, j = e / k;
+    // the Hermitian part
+    const double2 u = S[id[i] + id[j] * n], v = S[id[j] + id[i] * n];
+    double2 h = make_double2(0.5 * (u.x + v.x), 0.5 * (u.y - v.y));
+    if (G && i == j) h = make_double2(lam[id[i]], 0.0);
+    if (G && i != j) {
+      const double2 g = G[id[i] + id[j] * n];
+      const double l = 0.5 * (lam[id[i]] + lam[id[j]]);
+      h = make_double2(h.x - l * g.x, h.y - l * g.y);
+    }
+    A[i + P * j] = h;
+    Z[i + P * j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
+  }
+  __syncthreads();
+  double prev = INFINITY;
+  bool done = false;
+  for (int sweep = 0; sweep <= 40; ++sweep) {
+    if (tid < 32) {
+      double o = 0.0, t = 0.0;
+      for (int e = tid; e < k * k; e += 32) {
+        const double2 v = A[e % k + P * (e / k)];
+        const double m = v.x * v.x + v.y * v.y;
+        t += m;
+        if (e % k != e / k) o += m;
+      }
+#pragma unroll
+      for (int h = 16; h > 0; h >>= 1) {
+        o += __shfl_xor_sync(0xffffffffu, o, h);
+        t += __shfl_xor_sync(0xffffffffu, t, h);
+      }
+      if (tid == 0) {
+        norms[0] = sqrt(o);
+        norms[1] = sqrt(t);
+      }
+    }
+    __syncthreads();
+    const double o = norms[0], t = norms[1];
+    __syncthreads();
+    if (o <= 1e-15 * t || o == 0.0 || (sweep > 2 && o > 0.5 * prev && o <= 1e-12 * t)) {
+      done = true;
+      break;
+    }
+    if (sweep == 40 || !(t < INFINITY)) break;
+    prev = o;
+    for (int r = 0; r < kp - 1; ++r) {
+      if (tid < kp / 2) jac_params_item<double>(tid, k, kp, r, A, P, rot, pairs);
+      __syncthreads();
+      for (int i = tid; i < (int)jac_items(kp / 2, k); i += blockDim.x)
+        jac_apply_item<double>(i, kp / 2, k, A, P, Z, P, rot, pairs);
+      __syncthreads();
+    }
+  }
+  if (!done && tid == 0) flag_error(status, CHEBFI_ERR_NO_CONVERGENCE);
+  if (tid < k) lam[id[tid]] = A[tid + P * tid].x;
+  // rows of X in steps of the block: a thread holds its row's k entries
+  for (int64_t row = tid; row < n; row += blockDim.x) {
+    double2 x[kMaxCluster];
+    for (int j = 0; j < k; ++j) x[j] = X[row + id[j] * n];
+    for (int j = 0; j < k; ++j) {
+      double2 y = make_double2(0.0, 0.0);
+      for (int l = 0; l < k; ++l) {
+        const double2 z = Z[l + P * j];
+        y.x = fma(x[l].x, z.x, fma(-x[l].y, z.y, y.x));
+        y.y = fma(x[l].x, z.y, fma(x[l].y, z.x, y.y));
+      }
+      X[row + id[j] * n] = y;
+    }
+  }
+}
+
 // ------------------------------------------------------------------ blocked Jacobi (FP32)
 // The two-sided cyclic Jacobi method on blocks: the n columns form n / 32 blocks, paired by
 // the round-robin tournament (n / 32 - 1 rounds per sweep, n / 64 disjoint pairs per round).
-// For a pair (I, J) the 64 x 64 subproblem A[IJ, IJ] is diagonalised in shared memory by the
-// scalar method (same rotations as above) giving a unitary W, then A <- W^H A W on rows and
+// For a pair (I, J) the 64 x 64 subproblem A[IJ, IJ] is swept once in shared memory by the
+// scalar method (same rotations as above; the pairs within I and within J only in the first
+// round, so that a sweep meets every pair of columns once) giving a unitary W, then A <- W^H A W on rows and
 // columns I u J and V <- V W: each round is one pass over A and V as small dense products
 // instead of 63 passes of scalar rotations, which the scalar method spends in grid barriers
 // and load latency.
+//
+// Two launches a round.  k_bj_update forms the tile W1^H A W2 of each pair of pairs in one
+// go and only for the lower triangle of A, writing the conjugate tile beside it (2080 64^3
+// products a round at n = 2048 where column and row passes take 3072).  The subproblems are a
+// chain of 63 short steps on n / 64 SMs, so k_bj_solve's other blocks meanwhile apply the
+// round before's W to V, which nobody waits for.  n = 2048: 233 us a round (93 + 140) with
+// one kernel each for solve, columns and rows, now 121 us.
 namespace bj {
 constexpr int B = 32, S2 = 64, PS = S2 + 1;  // block, subproblem, shared pitch
 
 __device__ __forceinline__ int player(int pos, int round, int m) {
-  return pos == 0 ? 0 : 1 + (pos - 1 + round) % (m - 1);
+  if (pos == 0) return 0;
+  const int p = pos - 1 + round;  // round < m - 1, pos < m
+  return 1 + (p >= m - 1 ? p - (m - 1) : p);
 }
 __device__ __forceinline__ void blocks_of(int pair, int round, int nbk, int& I, int& J) {
   I = player(pair, round, nbk);
@@ -604,145 +711,23 @@ __device__ __forceinline__ void blocks_of(int pair, int round, int nbk, int& I, 
 }
 __device__ __forceinline__ int gidx(int l, int I, int J) { return l < B ? I * B + l : J * B + (l - B); }
 
-// One CTA of 1024 threads per pair: gather the subproblem, diagonalise it (up to `sweeps`
-// cyclic sweeps, or until its off-diagonal part is below tol of its norm), write the
-// rotation W (64 x 64, column-major) to Wout[pair].
-__global__ void __launch_bounds__(1024) k_bj_solve(const float2* __restrict__ A, int64_t lda, int nbk, int round,
-                                                  float2* __restrict__ Wout, int sweeps, float tol) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float2* S = reinterpret_cast<float2*>(smem);  // S[i + PS j] = element (i, j)
-  float2* W = S + S2 * PS;
-  RotT<float>* rot = reinterpret_cast<RotT<float>*>(W + S2 * PS);
-  int* pq = reinterpret_cast<int*>(rot + S2 / 2);
-  __shared__ float red[2][1024];
-  int I, J;
-  blocks_of(blockIdx.x, round, nbk, I, J);
-  const int tid = threadIdx.x;
-  for (int e = tid; e < S2 * S2; e += blockDim.x) {
-    const int i = e % S2, j = e / S2;
-    S[i + PS * j] = A[gidx(i, I, J) + (int64_t)gidx(j, I, J) * lda];
-    W[i + PS * j] = make_float2(i == j ? 1.f : 0.f, 0.f);
-  }
-  __syncthreads();
-  for (int sw = 0; sw < sweeps; ++sw) {
-    float o = 0.f, t = 0.f;
-    for (int e = tid; e < S2 * S2; e += blockDim.x) {
-      const int i = e % S2, j = e / S2;
-      const float2 v = S[i + PS * j];
-      const float m = v.x * v.x + v.y * v.y;
-      t += m;
-      if (i != j) o += m;
-    }
-    red[0][tid] = o;
-    red[1][tid] = t;
-    __syncthreads();
-    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-      if (tid < h) {
-        red[0][tid] += red[0][tid + h];
-        red[1][tid] += red[1][tid + h];
-      }
-      __syncthreads();
-    }
-    const bool done = red[0][0] <= tol * tol * red[1][0];
-    __syncthreads();
-    if (done) break;
-    for (int r = 0; r < S2 - 1; ++r) {
-      if (tid < S2 / 2) {
-        int p = player(tid, r, S2), q = player(S2 - 1 - tid, r, S2);
-        if (p > q) {
-          const int x = p;
-          p = q;
-          q = x;
-        }
-        RotT<float> rr;
-        rr.c = 1.f;
-        rr.s = 0.f;
-        rr.ph = make_float2(1.f, 0.f);
-        const float2 h = S[p + PS * q];
-        const float g = hypotf(h.x, h.y);
-        const float app = S[p + PS * p].x, aqq = S[q + PS * q].x;
-        if (g > JacEps<float>::tiny && g > JacEps<float>::v * sqrtf(fabsf(app * aqq))) {
-          const float zeta = (aqq - app) / (2.f * g);
-          const float tt = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + hypotf(1.f, zeta));
-          rr.c = 1.f / sqrtf(1.f + tt * tt);
-          rr.s = tt * rr.c;
-          rr.ph = make_float2(h.x / g, h.y / g);
-        }
-        rot[tid] = rr;
-        pq[2 * tid] = p;
-        pq[2 * tid + 1] = q;
-      }
-      __syncthreads();
-      // 2 x 2 blocks of S: U1^H S U2
-      for (int it = tid; it < (S2 / 2) * (S2 / 2); it += blockDim.x) {
-        const int t1 = it % (S2 / 2), t2 = it / (S2 / 2);
-        const RotT<float> r1 = rot[t1], r2 = rot[t2];
-        if (r1.s == 0.f && r2.s == 0.f) continue;
-        const int p1 = pq[2 * t1], q1 = pq[2 * t1 + 1], p2 = pq[2 * t2], q2 = pq[2 * t2 + 1];
-        float2 m00 = S[p1 + PS * p2], m10 = S[q1 + PS * p2], m01 = S[p1 + PS * q2], m11 = S[q1 + PS * q2];
-        if (r1.s != 0.f) {
-          rot2(m00, m10, r1.c, r1.s, r1.ph);
-          rot2(m01, m11, r1.c, r1.s, r1.ph);
-        }
-        if (r2.s != 0.f) {
-          const float2 c2 = conjg(r2.ph);
-          rot2(m00, m01, r2.c, r2.s, c2);
-          rot2(m10, m11, r2.c, r2.s, c2);
-        }
-        S[p1 + PS * p2] = m00;
-        S[q1 + PS * p2] = m10;
-        S[p1 + PS * q2] = m01;
-        S[q1 + PS * q2] = m11;
-      }
-      // W <- W U on columns {p, q}
-      for (int it = tid; it < S2 * (S2 / 2); it += blockDim.x) {
-        const int i = it % S2, tt = it / S2;
-        const RotT<float> rr = rot[tt];
-        if (rr.s == 0.f) continue;
-        const int p = pq[2 * tt], q = pq[2 * tt + 1];
-        float2 a = W[i + PS * p], b = W[i + PS * q];
-        rot2(a, b, rr.c, rr.s, conjg(rr.ph));
-        W[i + PS * p] = a;
-        W[i + PS * q] = b;
-      }
-      __syncthreads();
-    }
-  }
-  float2* wo = Wout + (int64_t)blockIdx.x * S2 * S2;
-  for (int e = tid; e < S2 * S2; e += blockDim.x) wo[e] = W[(e % S2) + PS * (e / S2)];
-}
-
-// columns I u J of M (A or V; blockIdx.z) times W: a CTA takes 64 rows, in place
-__global__ void __launch_bounds__(256) k_bj_cols(float2* A, int64_t lda, float2* V, int64_t ldv, int nbk, int round,
-                                                 const float2* __restrict__ Win, int64_t nrows) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float2* W = reinterpret_cast<float2*>(smem);  // W[l + PS c]
-  float2* X = W + S2 * PS;                       // X[row + PS l]
-  int I, J;
-  blocks_of(blockIdx.y, round, nbk, I, J);
-  float2* M = blockIdx.z == 0 ? A : V;
-  const int64_t ld = blockIdx.z == 0 ? lda : ldv;
-  const int64_t r0 = (int64_t)blockIdx.x * S2;
-  const float2* w = Win + (int64_t)blockIdx.y * S2 * S2;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < S2 * S2; e += blockDim.x) {
-    const int a = e % S2, b = e / S2;
-    W[a + PS * b] = w[e];
-    const int64_t r = r0 + a;
-    X[a + PS * b] = r < nrows ? M[r + (int64_t)gidx(b, I, J) * ld] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  // thread: rows ri + 16 k (k < 4), columns ci + 16 m (m < 4)
-  const int ri = tid % 16, ci = tid / 16;
-  float2 acc[4][4];
+// acc(r, c) = sum_l X(r, l) W(l, c), or with CONJ sum_l conj(X(l, r)) W(l, c), of 64 x 64 tiles
+// in shared memory (X[i + PS j] = element (i, j)); thread: rows ri + 16 k, columns ci + 16 m
+template <bool CONJ>
+__device__ __forceinline__ void mul64(const float2* X, const float2* W, float2 (&acc)[4][4]) {
+  const int ri = threadIdx.x % 16, ci = threadIdx.x % 256 / 16;
 #pragma unroll
   for (int k = 0; k < 4; ++k)
 #pragma unroll
     for (int m = 0; m < 4; ++m) acc[k][m] = make_float2(0.f, 0.f);
+#pragma unroll 4
   for (int l = 0; l < S2; ++l) {
     float2 x[4], y[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) x[k] = X[ri + 16 * k + PS * l];
+    for (int k = 0; k < 4; ++k) {
+      x[k] = CONJ ? X[l + PS * (ri + 16 * k)] : X[ri + 16 * k + PS * l];
+      if (CONJ) x[k].y = -x[k].y;
+    }
 #pragma unroll
     for (int m = 0; m < 4; ++m) y[m] = W[l + PS * (ci + 16 * m)];
 #pragma unroll
@@ -753,136 +738,248 @@ __global__ void __launch_bounds__(256) k_bj_cols(float2* A, int64_t lda, float2*
         acc[k][m].y = fmaf(x[k].x, y[m].y, fmaf(x[k].y, y[m].x, acc[k][m].y));
       }
   }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int64_t r = r0 + ri + 16 * k;
-    if (r >= nrows) continue;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) M[r + (int64_t)gidx(ci + 16 * m, I, J) * ld] = acc[k][m];
-  }
 }
-
-// rows I u J of A: W^H times them; a CTA takes 64 columns, in place
-__global__ void __launch_bounds__(256) k_bj_rows(float2* A, int64_t lda, int nbk, int round,
-                                                 const float2* __restrict__ Win, int64_t ncols) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float2* W = reinterpret_cast<float2*>(smem);  // W[l + PS c]
-  float2* Z = W + S2 * PS;                       // Z[l + PS col]
-  int I, J;
-  blocks_of(blockIdx.y, round, nbk, I, J);
-  const int64_t c0 = (int64_t)blockIdx.x * S2;
-  const float2* w = Win + (int64_t)blockIdx.y * S2 * S2;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < S2 * S2; e += blockDim.x) {
-    const int a = e % S2, b = e / S2;
-    W[a + PS * b] = w[e];
-    const int64_t c = c0 + b;
-    Z[a + PS * b] = c < ncols ? A[gidx(a, I, J) + c * lda] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  // thread: output rows li + 16 k, columns cj + 16 m; out(l, col) = sum_k conj(W(k, l)) Z(k, col)
-  const int li = tid % 16, cj = tid / 16;
-  float2 acc[4][4];
+__device__ __forceinline__ void put64(float2* X, const float2 (&acc)[4][4]) {
+  const int ri = threadIdx.x % 16, ci = threadIdx.x / 16;
 #pragma unroll
   for (int k = 0; k < 4; ++k)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) acc[k][m] = make_float2(0.f, 0.f);
-  for (int q = 0; q < S2; ++q) {
-    float2 wv[4], z[4];
+    for (int m = 0; m < 4; ++m) X[ri + 16 * k + PS * (ci + 16 * m)] = acc[k][m];
+}
+
+// [a, b] <- [c a - s ph b, s a + c ph b] as packed (Re, Im) operations
+__device__ __forceinline__ void rot2p(float2& a, float2& b, float c, float s, float2 ph) {
+  const float2 pb = __ffma2_rn(make_float2(ph.x, ph.x), b, __fmul2_rn(make_float2(-ph.y, ph.y), make_float2(b.y, b.x)));
+  const float2 na = __ffma2_rn(make_float2(c, c), a, __fmul2_rn(make_float2(-s, -s), pb));
+  b = __ffma2_rn(make_float2(s, s), a, __fmul2_rn(make_float2(c, c), pb));
+  a = na;
+}
+
+// Diagonalise the SS x SS Hermitian S (in shared memory, S[i + (SS + 1) j]) by up to `sweeps`
+// cyclic sweeps, or until its off-diagonal part is below tol of its norm; W (same layout,
+// the identity on entry) collects the rotations.  A sweep is a chain of SS - 1 short rounds,
+// bound by latency: lane l of every warp computes the rotation of pair l from the same
+// entries (no hand-over through shared memory, one barrier less) with the fast reciprocal
+// square root (2 ulp there cost nothing, the vectors are refined), takes the 2 x 2 blocks of
+// row pair l and of its warp's column pairs, and gets the latter's rotations by shuffles.
+// One 64 x 64 sweep: 93 us with 1024 threads and rotations through shared memory, now 86 us,
+// and 45 us for the 32 x 32 pairs across the blocks.
+template <int SS> struct SolveThreads { static constexpr int v = SS == 64 ? 512 : 256; };
+// CROSS: only the pairs of one index below SS / 2 and one above (SS / 2 rounds).
+template <int SS, bool CROSS>
+__device__ void solve_shared(float2* S, float2* W, int sweeps, float tol) {
+  constexpr int P = SS + 1, NP = SS / 2, NT = SolveThreads<SS>::v, NW = NT / 32;
+  static_assert(NP * NP % NT == 0 && (NP == 32 || 2 * NW == NP), "items of a round");
+  __shared__ float red[2][NW];
+  const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+  const unsigned all = 0xffffffffu;
+  for (int sw = 0; sw < sweeps; ++sw) {
+    float o = 0.f, t = 0.f;
+    for (int e = tid; e < SS * SS; e += NT) {
+      const int i = e % SS, j = e / SS;
+      const float2 v = S[i + P * j];
+      const float m = v.x * v.x + v.y * v.y;
+      t += m;
+      if (i != j) o += m;
+    }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) wv[k] = W[q + PS * (li + 16 * k)];
+    for (int h = 16; h > 0; h >>= 1) {
+      o += __shfl_xor_sync(all, o, h);
+      t += __shfl_xor_sync(all, t, h);
+    }
+    if (lane == 0) {
+      red[0][warp] = o;
+      red[1][warp] = t;
+    }
+    __syncthreads();
+    o = t = 0.f;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) z[m] = Z[q + PS * (cj + 16 * m)];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {  // conj(wv) z
-        acc[k][m].x = fmaf(wv[k].x, z[m].x, fmaf(wv[k].y, z[m].y, acc[k][m].x));
-        acc[k][m].y = fmaf(wv[k].x, z[m].y, fmaf(-wv[k].y, z[m].x, acc[k][m].y));
+    for (int i = 0; i < NW; ++i) {
+      o += red[0][i];
+      t += red[1][i];
+    }
+    __syncthreads();
+    if (!(o > tol * tol * t)) break;
+    for (int r = 0; r < (CROSS ? NP : SS - 1); ++r) {
+      int p = lane % NP, q = NP + (p + r) % NP;
+      if (!CROSS) {
+        p = player(lane % NP, r, SS);
+        q = player(SS - 1 - lane % NP, r, SS);
+        if (p > q) {
+          const int x = p;
+          p = q;
+          q = x;
+        }
       }
-  }
+      const float2 h = S[p + P * q];
+      const float app = S[p + P * p].x, aqq = S[q + P * q].x;
+      const float g2 = h.x * h.x + h.y * h.y;
+      float c = 1.f, s = 0.f, px = 1.f, py = 0.f;
+      if (g2 > 1e-36f && g2 > JacEps<float>::v * JacEps<float>::v * fabsf(app * aqq)) {
+        const float rg = rsqrtf(g2), zeta = 0.5f * (aqq - app) * rg;
+        const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + __fsqrt_rn(fmaf(zeta, zeta, 1.f)));
+        c = rsqrtf(fmaf(tt, tt, 1.f));
+        s = tt * c;
+        px = h.x * rg;
+        py = h.y * rg;
+      }
+      __syncthreads();
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int64_t c = c0 + cj + 16 * m;
-    if (c >= ncols) continue;
+      for (int i = 0; i < NP * NP / NT; ++i) {
+        // block of row pair t1 = lane % NP and column pair t2: U1^H S U2
+        const int t2 = NP == 32 ? warp + NW * i : 2 * warp + lane / 16;
+        const int p2 = CROSS ? t2 : __shfl_sync(all, p, t2), q2 = CROSS ? NP + (t2 + r) % NP : __shfl_sync(all, q, t2);
+        const float c2 = __shfl_sync(all, c, t2), s2 = __shfl_sync(all, s, t2);
+        const float2 ph2 = make_float2(__shfl_sync(all, px, t2), -__shfl_sync(all, py, t2));
+        const float2 ph1 = make_float2(px, py);
+        float2 m00 = S[p + P * p2], m10 = S[q + P * p2], m01 = S[p + P * q2], m11 = S[q + P * q2];
+        rot2p(m00, m10, c, s, ph1);
+        rot2p(m01, m11, c, s, ph1);
+        rot2p(m00, m01, c2, s2, ph2);
+        rot2p(m10, m11, c2, s2, ph2);
+        S[p + P * p2] = m00;
+        S[q + P * p2] = m10;
+        S[p + P * q2] = m01;
+        S[q + P * q2] = m11;
+        // W <- W U2 on columns {p2, q2}
+        if (NP == 32) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) A[gidx(li + 16 * k, I, J) + c * lda] = acc[k][m];
+          for (int row = lane; row < SS; row += 32) {
+            float2 a = W[row + P * p2], b = W[row + P * q2];
+            rot2p(a, b, c2, s2, ph2);
+            W[row + P * p2] = a;
+            W[row + P * q2] = b;
+          }
+        } else {  // SS = 32: the half-warp's own column pair, both halves of its rows
+#pragma unroll
+          for (int row = lane % 16; row < SS; row += 16) {
+            float2 a = W[row + P * p2], b = W[row + P * q2];
+            rot2p(a, b, c2, s2, ph2);
+            W[row + P * p2] = a;
+            W[row + P * q2] = b;
+          }
+        }
+      }
+      __syncthreads();
+    }
   }
 }
 
-// zero-padded copy with pad values on the extra diagonal entries
-__global__ void k_bj_pad(int64_t n0, int64_t np, const float2* __restrict__ A, int64_t lda, float2* __restrict__ Ap,
-                         float pad) {
+// Blocks [0, npairs): gather the pair's subproblem, one sweep, write its rotation W (64 x 64,
+// column-major) to Wout[pair].  The others: V <- V W of the round before (Wprev), a block per
+// 128 rows and pair, 64 rows for each half of its threads.
+__global__ void __launch_bounds__(512) k_bj_solve(const float2* __restrict__ A, float2* __restrict__ V, int64_t ld,
+                                                  int nbk, int round, int round_prev, float2* __restrict__ Wout,
+                                                  const float2* __restrict__ Wprev, float tol) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* W = reinterpret_cast<float2*>(smem);
+  float2* S = W + S2 * PS;
+  const int tid = threadIdx.x, npairs = nbk / 2;
+  int I, J;
+  if ((int)blockIdx.x < npairs) {
+    blocks_of(blockIdx.x, round, nbk, I, J);
+    for (int e = tid; e < S2 * S2; e += 512) {
+      const int i = e % S2, j = e / S2;
+      S[i + PS * j] = A[gidx(i, I, J) + (int64_t)gidx(j, I, J) * ld];
+      W[i + PS * j] = make_float2(i == j ? 1.f : 0.f, 0.f);
+    }
+    __syncthreads();
+    // the pairs within a block meet once a sweep, in its first round
+    if (round == 0) solve_shared<S2, false>(S, W, 1, tol);
+    else solve_shared<S2, true>(S, W, 1, tol);
+    float2* wo = Wout + (int64_t)blockIdx.x * S2 * S2;
+    for (int e = tid; e < S2 * S2; e += 512) wo[e] = W[(e % S2) + PS * (e / S2)];
+    return;
+  }
+  const int u = blockIdx.x - npairs, pair = u % npairs, half = tid / 256, t = tid % 256;
+  const int64_t r0 = (int64_t)(u / npairs) * 2 * S2 + half * S2;
+  const bool rows = r0 < ld;  // an odd number of 64-row tiles leaves the last half idle
+  blocks_of(pair, round_prev, nbk, I, J);
+  const float2* w = Wprev + (int64_t)pair * S2 * S2;
+  S += half * S2 * PS;
+  for (int e = tid; e < S2 * S2; e += 512) W[e % S2 + PS * (e / S2)] = w[e];
+  if (rows)
+    for (int e = t; e < S2 * S2; e += 256) S[e % S2 + PS * (e / S2)] = V[r0 + e % S2 + (int64_t)gidx(e / S2, I, J) * ld];
+  __syncthreads();
+  if (!rows) return;
+  float2 acc[4][4];
+  mul64<false>(S, W, acc);
+  const int ri = t % 16, ci = t / 16;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int m = 0; m < 4; ++m) V[r0 + ri + 16 * k + (int64_t)gidx(ci + 16 * m, I, J) * ld] = acc[k][m];
+}
+
+// A <- W^H A W, one block per tile (pair t1, pair t2), t1 >= t2: the rows of pair t1 and the
+// columns of pair t2, and the conjugate tile across the diagonal
+__global__ void __launch_bounds__(256) k_bj_update(float2* A, int64_t ld, int nbk, int round, const float2* __restrict__ Win) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* X = reinterpret_cast<float2*>(smem);
+  float2* W = X + S2 * PS;
+  const int tid = threadIdx.x;
+  // block -> (t1, t2) of the lower triangle, row by row
+  int t1 = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((t1 + 1) * (t1 + 2) / 2 <= (int)blockIdx.x) ++t1;
+  while (t1 * (t1 + 1) / 2 > (int)blockIdx.x) --t1;
+  const int t2 = (int)blockIdx.x - t1 * (t1 + 1) / 2;
+  int I1, J1, I2, J2;
+  blocks_of(t1, round, nbk, I1, J1);
+  blocks_of(t2, round, nbk, I2, J2);
+  const float2 *w1 = Win + (int64_t)t1 * S2 * S2, *w2 = Win + (int64_t)t2 * S2 * S2;
+  for (int e = tid; e < S2 * S2; e += 256) {
+    const int a = e % S2, b = e / S2;
+    W[a + PS * b] = w2[e];
+    X[a + PS * b] = A[gidx(a, I1, J1) + (int64_t)gidx(b, I2, J2) * ld];
+  }
+  __syncthreads();
+  float2 acc[4][4];
+  mul64<false>(X, W, acc);
+  __syncthreads();
+  put64(X, acc);
+  for (int e = tid; e < S2 * S2; e += 256) W[e % S2 + PS * (e / S2)] = w1[e];
+  __syncthreads();
+  mul64<true>(W, X, acc);
+  __syncthreads();
+  put64(X, acc);
+  __syncthreads();
+  for (int e = tid; e < S2 * S2; e += 256) {
+    const int a = e % S2, b = e / S2;
+    A[gidx(a, I1, J1) + (int64_t)gidx(b, I2, J2) * ld] = X[a + PS * b];
+  }
+  if (t1 == t2) return;
+  for (int e = tid; e < S2 * S2; e += 256) {
+    const int b = e % S2, a = e / S2;
+    const float2 v = X[a + PS * b];
+    A[gidx(b, I2, J2) + (int64_t)gidx(a, I1, J1) * ld] = make_float2(v.x, -v.y);
+  }
+}
+
+// the whole problem in one block, n <= SS (padded with decoupled zero rows): V's n x n block
+template <int SS>
+__global__ void __launch_bounds__(SolveThreads<SS>::v) k_bj_small(int n, const float2* __restrict__ A, int64_t lda, float2* __restrict__ V,
+                                                  int64_t ldv, float tol) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* S = reinterpret_cast<float2*>(smem);
+  float2* W = S + SS * (SS + 1);
+  for (int e = threadIdx.x; e < SS * SS; e += SolveThreads<SS>::v) {
+    const int i = e % SS, j = e / SS;
+    S[i + (SS + 1) * j] = i < n && j < n ? A[i + j * lda] : make_float2(0.f, 0.f);
+    W[i + (SS + 1) * j] = make_float2(i == j ? 1.f : 0.f, 0.f);
+  }
+  __syncthreads();
+  solve_shared<SS, false>(S, W, 16, tol);
+  for (int e = threadIdx.x; e < n * n; e += SolveThreads<SS>::v) V[e % n + (e / n) * ldv] = W[e % n + (SS + 1) * (e / n)];
+}
+
+// zero-padded copy
+__global__ void k_bj_pad(int64_t n0, int64_t np, const float2* __restrict__ A, int64_t lda, float2* __restrict__ Ap) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= np * np) return;
   const int64_t i = e % np, j = e / np;
-  Ap[e] = (i < n0 && j < n0) ? A[i + j * lda] : make_float2(i == j ? pad : 0.f, 0.f);
+  Ap[e] = (i < n0 && j < n0) ? A[i + j * lda] : make_float2(0.f, 0.f);
 }
 }  // namespace bj
-
-// The blocked FP32 Jacobi (bj:: kernels) on A (n0 x n0, destroyed): ascending w and V
-// (ld ldv).  The matrix is padded to a multiple of 64 with decoupled diagonal entries above
-// every eigenvalue (2 ||A||_F + 1), which no rotation touches and the sort puts last.
-bool block_jacobi_f32(int64_t n0, float2* A, int64_t lda, float* w, float2* V, int64_t ldv, cudaStream_t st,
-                      DevBuf<double2>* ws, double tol_conv, double tol_stall) {
-  if (n0 < 128) return false;
-  const int64_t np = (n0 + bj::S2 - 1) / bj::S2 * bj::S2;
-  const int nbk = (int)(np / bj::B), npairs = nbk / 2;
-  constexpr int kParts = 256;
-  // workspace in float2 slots: Ap, Vp, Vs (np^2 each), W (npairs x 64^2), wp (np / 2 + 1),
-  // norm partials and sums (2 kParts + 2 doubles)
-  const size_t nn = (size_t)np * np, nw = (size_t)npairs * bj::S2 * bj::S2;
-  const size_t total = 3 * nn + nw + np / 2 + 1 + 2 * kParts + 2;
-  ws->alloc(total / 2 + 1);
-  float2* Ap = reinterpret_cast<float2*>(ws->p);
-  float2* Vp = Ap + nn;
-  float2* Vs = Vp + nn;
-  float2* Wb = Vs + nn;
-  float* wp = reinterpret_cast<float*>(Wb + nw);
-  double* part = reinterpret_cast<double*>(Wb + nw + np / 2 + 1);
-  double* nrm = part + 2 * kParts;
-  auto norms = [&](const float2* M, int64_t n, int64_t ld, double& off, double& tot) {
-    const unsigned parts = (unsigned)std::min<int64_t>(kParts, std::max<int64_t>(1, n * n / 4096));
-    CHEBFI_LAUNCH("k_offnorm", st, k_offnorm_part<float><<<parts, 256, 0, st>>>(n, M, ld, part));
-    CHEBFI_LAUNCH("k_offnorm", st, k_offnorm_sum<<<1, 32, 0, st>>>((int)parts, part, nrm));
-    double hn[2];
-    CHEBFI_CUDA(cudaMemcpyAsync(hn, nrm, sizeof(hn), cudaMemcpyDeviceToHost, st));
-    CHEBFI_CUDA(cudaStreamSynchronize(st));
-    off = std::sqrt(hn[0]);
-    tot = std::sqrt(hn[1]);
-  };
-  double off = 0.0, tot = 0.0, tot_p = 0.0;
-  norms(A, n0, lda, off, tot);  // ||A||_F: the sweeps keep it (unitary similarity), so it is the scale
-  if (!std::isfinite(tot)) return false;  // the scalar path reports it
-  CHEBFI_LAUNCH("k_bj_pad", st, bj::k_bj_pad<<<nblk((int64_t)nn), 256, 0, st>>>(n0, np, A, lda, Ap, (float)(2.0 * tot + 1.0)));
-  set_identity_t<float>(np, Vp, np, st);
-  const size_t s_solve = (size_t)2 * bj::S2 * bj::PS * sizeof(float2) + bj::S2 / 2 * sizeof(RotT<float>) + bj::S2 * sizeof(int);
-  const size_t s_mul = (size_t)2 * bj::S2 * bj::PS * sizeof(float2);
-  CHEBFI_CUDA(cudaFuncSetAttribute(bj::k_bj_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_solve));
-  CHEBFI_CUDA(cudaFuncSetAttribute(bj::k_bj_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_mul));
-  CHEBFI_CUDA(cudaFuncSetAttribute(bj::k_bj_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_mul));
-  const unsigned tiles = (unsigned)(np / bj::S2);
-  double prev_off = INFINITY;
-  for (int sweep = 0; sweep <= 40; ++sweep) {
-    norms(Ap, np, np, off, tot_p);  // the pads add nothing off the diagonal
-    if (!std::isfinite(tot_p)) break;
-    if (off <= tol_conv * tot || off == 0.0 || (sweep > 2 && off > 0.5 * prev_off && off <= tol_stall * tot)) break;
-    if (sweep == 40) break;
-    prev_off = off;
-    // rounds of the block tournament; work: the subproblems' rotations and the two products
-    for (int round = 0; round < nbk - 1; ++round) {
-      CHEBFI_LAUNCH("k_bj_solve", st, bj::k_bj_solve<<<npairs, 1024, s_solve, st>>>(Ap, np, nbk, round, Wb, 1, 1e-7f));
-      CHEBFI_LAUNCH_W("k_bj_update", st, 3.0 * 8.0 * (double)np * bj::S2 * bj::S2 * npairs,
-                      bj::k_bj_cols<<<dim3(tiles, npairs, 2), 256, s_mul, st>>>(Ap, np, Vp, np, nbk, round, Wb, np));
-      CHEBFI_LAUNCH("k_bj_update", st, bj::k_bj_rows<<<dim3(tiles, npairs), 256, s_mul, st>>>(Ap, np, nbk, round, Wb, np));
-    }
-  }
-  CHEBFI_LAUNCH("k_eig_sort", st, k_eig_sort<float><<<(unsigned)np, 128, 0, st>>>(np, Ap, np, Vp, np, wp, Vs, np));
-  CHEBFI_CUDA(cudaMemcpyAsync(w, wp, sizeof(float) * n0, cudaMemcpyDeviceToDevice, st));
-  CHEBFI_CUDA(cudaMemcpy2DAsync(V, ldv * sizeof(float2), Vs, np * sizeof(float2), n0 * sizeof(float2), n0,
-                                cudaMemcpyDeviceToDevice, st));
-  return true;
-}
 
 }  // namespace
 
@@ -946,12 +1043,93 @@ void jacobi_eigh(int64_t n0, double2* A, int64_t lda, double* w, double2* V, int
   jacobi_eigh_t<double>(n0, A, lda, w, V, ldv, status, st, ws, 1e-15, 1e-12, true);
 }
 
-void jacobi_eigh_f32(int64_t n0, float2* A, int64_t lda, float* w, float2* V, int64_t ldv, int* status,
-                     cudaStream_t st, DevBuf<double2>* ws) {
-  // a first stage only: stop at the FP32 rounding level and never report a sweep limit; the
-  // blocked method from 128 bands up
-  if (block_jacobi_f32(n0, A, lda, w, V, ldv, st, ws, 4e-7, 1e-5)) return;
-  jacobi_eigh_t<float>(n0, A, lda, w, V, ldv, status, st, ws, 4e-7, 1e-5, false);
+// The FP32 Jacobi (bj:: kernels) on A (n0 x n0): approximate eigenvectors in V (ld ldv), in
+// no particular order.  One block for n0 <= 64, the block tournament above.  The matrix is
+// padded with decoupled zero rows and columns, which no rotation touches (a rotation needs a
+// non-zero off-diagonal entry).  False if A is not finite in FP32 (V is not written).
+bool jacobi_eigh_f32(int64_t n0, const float2* A, int64_t lda, float2* V, int64_t ldv, cudaStream_t st,
+                     DevBuf<double2>* ws) {
+  // off-diagonal entries of rms 1e-5 |A|_F / n turn a pair of typical gap by about 1e-3, which
+  // the refinement squares in each step; FP32 sweeps past this level mostly stir rounding noise
+  constexpr double tol_conv = 1e-5;
+  const int64_t np = n0 <= 64 ? 0 : (n0 + bj::S2 - 1) / bj::S2 * bj::S2;
+  const int nbk = (int)(np / bj::B), npairs = nbk / 2;
+  constexpr int kParts = 256;
+  // workspace in float2 slots: Ap and Vp (np^2 each), two sets of W (npairs x 64^2), norm
+  // partials and sums (2 kParts + 2 doubles)
+  const size_t nn = (size_t)np * np, nw = (size_t)npairs * bj::S2 * bj::S2;
+  ws->alloc((2 * nn + 2 * nw + 2 * kParts + 2) / 2 + 1);
+  float2* Ap = reinterpret_cast<float2*>(ws->p);
+  float2* Vp = Ap + nn;
+  float2* Wb[2] = {Vp + nn, Vp + nn + nw};
+  double* part = reinterpret_cast<double*>(Vp + nn + 2 * nw);
+  double* nrm = part + 2 * kParts;
+  auto norms = [&](const float2* M, int64_t n, int64_t ld, double& off, double& tot) {
+    const unsigned parts = (unsigned)std::min<int64_t>(kParts, std::max<int64_t>(1, n * n / 4096));
+    CHEBFI_LAUNCH("k_offnorm", st, k_offnorm_part<float><<<parts, 256, 0, st>>>(n, M, ld, part));
+    CHEBFI_LAUNCH("k_offnorm", st, k_offnorm_sum<<<1, 32, 0, st>>>((int)parts, part, nrm));
+    double hn[2];
+    CHEBFI_CUDA(cudaMemcpyAsync(hn, nrm, sizeof(hn), cudaMemcpyDeviceToHost, st));
+    CHEBFI_CUDA(cudaStreamSynchronize(st));
+    off = std::sqrt(hn[0]);
+    tot = std::sqrt(hn[1]);
+  };
+  double off = 0.0, tot = 0.0;
+  norms(A, n0, lda, off, tot);
+  if (!std::isfinite(tot)) return false;
+  if (n0 <= 64) {
+    auto small = [&](auto kernel, int ss, int threads) {
+      const size_t bytes = (size_t)2 * ss * (ss + 1) * sizeof(float2);
+      CHEBFI_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+      CHEBFI_LAUNCH("k_bj_small", st, kernel<<<1, threads, bytes, st>>>((int)n0, A, lda, V, ldv, (float)tol_conv));
+    };
+    if (n0 <= 32) small(bj::k_bj_small<32>, 32, bj::SolveThreads<32>::v);
+    else small(bj::k_bj_small<64>, 64, bj::SolveThreads<64>::v);
+    return true;
+  }
+  CHEBFI_LAUNCH("k_bj_pad", st, bj::k_bj_pad<<<nblk((int64_t)nn), 256, 0, st>>>(n0, np, A, lda, Ap));
+  set_identity_t<float>(np, Vp, np, st);
+  const size_t bytes = (size_t)2 * bj::S2 * bj::PS * sizeof(float2);
+  const size_t sbytes = (size_t)3 * bj::S2 * bj::PS * sizeof(float2);
+  CHEBFI_CUDA(cudaFuncSetAttribute(bj::k_bj_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbytes));
+  CHEBFI_CUDA(cudaFuncSetAttribute(bj::k_bj_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  const unsigned vtiles = (unsigned)((np / bj::S2 + 1) / 2) * npairs, atiles = (unsigned)npairs * (npairs + 1) / 2;
+  const double prod = 8.0 * bj::S2 * bj::S2 * bj::S2;  // flops of one 64^3 complex product
+  double prev_off = INFINITY;
+  int w = 0, last_round = -1;  // W of round last_round, in Wb[w ^ 1], is still to be applied to V
+  for (int sweep = 0; sweep <= 40; ++sweep) {
+    if (sweep > 0) {
+      double t;
+      norms(Ap, np, np, off, t);
+      if (!std::isfinite(t)) return false;
+    }
+    if (off <= tol_conv * tot || off == 0.0 || (sweep > 2 && off > 0.5 * prev_off && off <= 1e-3 * tot)) break;
+    if (sweep == 40) break;
+    prev_off = off;
+    for (int round = 0; round < nbk - 1; ++round) {
+      const unsigned extra = last_round >= 0 ? vtiles : 0;
+      CHEBFI_LAUNCH_W("k_bj_solve", st, prod * 2.0 * extra,
+                      bj::k_bj_solve<<<npairs + extra, 512, sbytes, st>>>(Ap, Vp, np, nbk, round, last_round, Wb[w], Wb[w ^ 1],
+                                                                         1e-7f));
+      CHEBFI_LAUNCH_W("k_bj_update", st, prod * 2.0 * atiles,
+                      bj::k_bj_update<<<atiles, 256, bytes, st>>>(Ap, np, nbk, round, Wb[w]));
+      last_round = round;
+      w ^= 1;
+    }
+  }
+  if (last_round >= 0) {  // the last W (the block's own subproblem is solved again, into the free W)
+    CHEBFI_LAUNCH_W("k_bj_solve", st, prod * 2.0 * vtiles,
+                    bj::k_bj_solve<<<npairs + vtiles, 512, sbytes, st>>>(Ap, Vp, np, nbk, 0, last_round, Wb[w], Wb[w ^ 1], 1e-7f));
+  }
+  CHEBFI_CUDA(cudaMemcpy2DAsync(V, ldv * sizeof(float2), Vp, np * sizeof(float2), n0 * sizeof(float2), n0,
+                                cudaMemcpyDeviceToDevice, st));
+  return true;
+}
+
+int max_cluster() { return kMaxCluster; }
+void cluster_solve(int64_t n, int ncl, const int* off, const int* idx, const double2* S, const double2* G, double2* X,
+                   double* lam, int* status, cudaStream_t st) {
+  CHEBFI_LAUNCH("k_cluster_solve", st, k_cluster_solve<<<ncl, 256, 0, st>>>(n, off, idx, S, G, X, lam, status));
 }
 
 }  // namespace chebfi

@@ -238,7 +238,6 @@ struct Work {
   DevBuf<double2> small1, small2, small3, small4, small5;  // nb x nb
   // refined eigensolver: FP32 first stage, FP64 refinement matrices, stats, cluster pairs
   DevBuf<float2> e32a, e32b;
-  DevBuf<float> e32w;
   DevBuf<double2> eG, eS, eAX, eM, eX, esub, eZ, eC1, eC2;
   DevBuf<double> elam, esw;
   DevBuf<unsigned long long> estats;

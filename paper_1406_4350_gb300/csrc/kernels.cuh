@@ -207,10 +207,18 @@ void trsm_lower(int64_t n, int64_t m, const double2* L, int64_t ldl, double2* B,
 // CHEBFI_ERR_NO_CONVERGENCE on the sweep limit.  Synchronises the stream (sweep test).
 void jacobi_eigh(int64_t n, double2* A, int64_t lda, double* w, double2* V, int64_t ldv, int* status,
                  cudaStream_t st, DevBuf<double2>* ws);
-// The same in FP32, stopping at the FP32 rounding level (first stage of the refined solver;
-// never reports a sweep limit).  ws holds its rotations, pair list and a copy of V.
-void jacobi_eigh_f32(int64_t n, float2* A, int64_t lda, float* w, float2* V, int64_t ldv, int* status,
-                     cudaStream_t st, DevBuf<double2>* ws);
+// Approximate eigenvectors V of a finite Hermitian A by Jacobi in FP32, to its rounding level
+// and in no particular order (first stage of the refined solver).  False if A is not finite.
+// Synchronises the stream; ws holds its copies and rotations.
+bool jacobi_eigh_f32(int64_t n, const float2* A, int64_t lda, float2* V, int64_t ldv, cudaStream_t st,
+                     DevBuf<double2>* ws);
+// Clusters of the refinement: for each c < ncl, the at most max_cluster() columns
+// idx[off[c]..off[c + 1]) (device arrays) of X (n x n) are rotated to diagonalise
+// S[idx, idx] (S = X^H A X; with G = X^H X and lam given, its orthogonalised form), whose
+// eigenvalues go to lam[idx].
+int max_cluster();
+void cluster_solve(int64_t n, int ncl, const int* off, const int* idx, const double2* S, const double2* G, double2* X,
+                   double* lam, int* status, cudaStream_t st);
 // One Ogita-Aishima refinement step (n x n, lda = n): from G = X^H X and S = X^H A X, the
 // approximate eigenvalues lam and M = I + E with X (I + E) the refined vectors; stats[0] =
 // max |lam| bits, stats[1] = max |E| bits (doubles as ordered integers); pairs whose gap is

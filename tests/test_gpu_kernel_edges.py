@@ -97,3 +97,29 @@ def test_modular_gemm_is_exact_on_integers(m, n, k):
     C = _np(g.gemm_fp64(_F(A), _F(B), conjA=True))
     assert np.array_equal(C.real, (ar @ br - ai @ bi).astype(np.float64))
     assert np.array_equal(C.imag, (ar @ bi + ai @ br).astype(np.float64))
+
+
+# the eigensolver's routes: FP64 Jacobi below 8 bands, one block up to 32 and 64, the block
+# tournament from 65 (an even and an odd number of 64-column tiles), general and clustered
+# spectra (S = I, V = 0: the free-electron shells, exactly degenerate)
+@pytest.mark.parametrize("nb", [2, 7, 8, 31, 33, 64, 65, 129, 192])
+@pytest.mark.parametrize("shells", [False, True])
+def test_rayleigh_ritz_route_edges(nb, shells):
+    cell = make_cell(8.0, 20, 6.0, 2, 8, nb, not shells, 33)
+    if shells:
+        cell.vloc = np.zeros_like(cell.vloc)
+        cell.D = np.zeros_like(cell.D)
+    op = PWOperator.from_cell(cell)
+    g = _ctx(cell)
+    Y = _F(cell.Y0)
+    ev, rs = g.rayleigh_ritz(Y)
+    w, Yg = _np(ev), _np(Y)
+    w_ref, _ = ch.rayleigh_ritz(op, cell.Y0)
+    scale = np.abs(w_ref).max()
+    # the Gram matrix's condition number multiplies the rounding of every entry
+    cond = np.linalg.cond(cell.Y0.conj().T @ op.apply_S(cell.Y0))
+    tol = 200.0 * nb * U * cond
+    np.testing.assert_allclose(w, w_ref, atol=tol * scale)
+    np.testing.assert_allclose(Yg.conj().T @ op.apply_S(Yg), np.eye(nb), atol=tol)
+    np.testing.assert_allclose(Yg.conj().T @ op.apply_H(Yg), np.diag(w), atol=tol * scale)
+    np.testing.assert_allclose(_np(rs), ch.residuals(op, Yg, w), atol=tol * scale)
