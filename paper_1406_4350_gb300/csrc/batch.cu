@@ -560,8 +560,8 @@ void bgemm(chebfi_batch* bt, int op, int first, const cplx<R>* Bb, cplx<R>* Cb, 
 template <typename R, int N>
 void set_fft_smem(chebfi_batch* bt) {
   const SphereFFT& s = bt->ks[0]->sph;
-  const size_t zbytes = (size_t)(N + kCBF * s.zpitch) * sizeof(cplx<R>);
-  const size_t pbytes = (size_t)(N + N * s.pitch) * sizeof(cplx<R>);
+  const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
+  const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
   CHEBFI_CUDA(cudaFuncSetAttribute((const void*)k_bzinv<R, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zbytes));
   CHEBFI_CUDA(cudaFuncSetAttribute((const void*)k_bzfwd<R, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zbytes));
   CHEBFI_CUDA(cudaFuncSetAttribute((const void*)k_bplane<R, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pbytes));
@@ -572,8 +572,8 @@ template <typename R, int N>
 void blocal(chebfi_batch* bt, const cplx<R>* cur, cplx<R>* Z, cplx<R>* prev, int first, cudaStream_t st) {
   chebfi_ctx* c0 = bt->ks[0];
   const SphereFFT& s = c0->sph;
-  const size_t zbytes = (size_t)(N + kCBF * s.zpitch) * sizeof(cplx<R>);
-  const size_t pbytes = (size_t)(N + N * s.pitch) * sizeof(cplx<R>);
+  const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
+  const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
   const KDesc<R>* d = BatchOps<R>::desc(bt).p;
   const cplx<R>* tw = BatchOps<R>::tw(c0);
   cplx<R>* T = BatchOps<R>::T(bt).p;
@@ -582,6 +582,9 @@ void blocal(chebfi_batch* bt, const cplx<R>* cur, cplx<R>* Z, cplx<R>* prev, int
   CHEBFI_LAUNCH("k_bplane", st, (k_bplane<R, N><<<dim3(N, (unsigned)(bt->nk * bt->nb)), kT, pbytes, st>>>(d, bt->nb, T, BatchOps<R>::Vs(c0), tw)));
   CHEBFI_LAUNCH("k_bzfwd", st, (k_bzfwd<R, N><<<gz, kT, zbytes, st>>>(d, T, tw, bt->cb_k.p, bt->cb_c0.p, cur, Z, prev, first)));
 }
+
+// the grouped kernels are compiled for these lengths
+bool batch_fft_size(int n) { return n == 24 || n == 32 || n == 48 || n == 64 || n == 72 || n == 96; }
 
 template <typename R>
 void blocal_n(chebfi_batch* bt, const cplx<R>* cur, cplx<R>* Z, cplx<R>* prev, int first, cudaStream_t st) {
@@ -1016,7 +1019,7 @@ int chebfi_batch_create(chebfi_batch** out, chebfi_ctx* const* kctx, int nk, int
       CHEBFI_REQUIRE(c->has_cell && c->has_sphere && c->has_vloc && c->has_proj, CHEBFI_ERR_STATE,
                      "k-point context " + std::to_string(k) + " is not fully set up");
       CHEBFI_REQUIRE(c->device == c0->device, CHEBFI_ERR_ARG, "k-point contexts on different devices");
-      CHEBFI_REQUIRE(c->fast_fft, CHEBFI_ERR_ARG,
+      CHEBFI_REQUIRE(c->fast_fft && batch_fft_size(c->grid[0]), CHEBFI_ERR_ARG,
                      "batched k-points need a cubic grid of 24, 32, 48, 64, 72 or 96 points per side");
       CHEBFI_REQUIRE(c->grid[0] == c0->grid[0] && c->grid[1] == c0->grid[1] && c->grid[2] == c0->grid[2],
                      CHEBFI_ERR_ARG, "k-point contexts with different grids");

@@ -17,7 +17,7 @@
 
 #include "fft_core.cuh"
 #include "fft_fast.cuh"
-#include "fft_fast_kernels.cuh"
+#include "fft_launch.cuh"
 #include "internal.cuh"
 #include "kernels.cuh"
 
@@ -225,44 +225,6 @@ __global__ void k_density_accum(int n1, int n2, int n3, int64_t nbc, const cplx<
   gV[((int64_t)x * n2 + y) * n3 + z] += scale * acc;
 }
 
-// ---------------------------------------------------------------- compile-time-length path
-// The pass bodies live in fft_fast_kernels.cuh; here each block finds its columns or plane
-// from its grid position.
-using fk::FastArgs;
-using fk::kCBF;
-
-// R: the arithmetic of the transforms (float, double, or dfl, the double-float form of the
-// FP64 path); blocks, the kinetic diagonal and the epilogue's operands are stored in
-// SphT<R> (double for dfl), the column buffer and the planes in cplx<R>.
-template <typename R, int N3>
-__global__ void __launch_bounds__(kThreads) k_zinv_f(const cplx<typename SphT<R>::type>* __restrict__ Y, int64_t ldy,
-                                                     cplx<R>* __restrict__ T, FastArgs fa, const cplx<R>* __restrict__ twz) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  fk::zinv_body<R, N3>(Y, ldy, T, fa, twz, blockIdx.x * kCBF, blockIdx.y, smem_raw);
-}
-
-// threads of a plane block: the double-float plane (16 bytes a point, one block per SM)
-// takes 16 warps to keep its FP32 pipes fed, the others 8 with three blocks per SM
-template <typename R> struct PlaneThreads { static constexpr int v = kThreads; };
-template <> struct PlaneThreads<dfl> { static constexpr int v = 2 * kThreads; };
-
-template <typename R, int N>
-__global__ void __launch_bounds__(PlaneThreads<R>::v) k_plane_f(cplx<R>* __restrict__ T, const R* __restrict__ Vs,
-                                                                FastArgs fa, const cplx<R>* __restrict__ twxy) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  (void)twxy;
-  fk::plane_body_pruned<R, N, PlaneThreads<R>::v>(T, Vs, fa, blockIdx.x, blockIdx.y, smem_raw);
-}
-
-template <typename R, int N3>
-__global__ void __launch_bounds__(kThreads) k_zfwd_f(const cplx<R>* __restrict__ T, FastArgs fa,
-                                                     const cplx<R>* __restrict__ twz,
-                                                     const typename SphT<R>::type* __restrict__ K,
-                                                     LocalEpi<typename SphT<R>::type> ep) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  fk::zfwd_body<R, N3>(T, fa, twz, K, ep, blockIdx.x * kCBF, blockIdx.y, smem_raw);
-}
-
 template <typename R> void set_smem(const void* f, size_t bytes) {
   CHEBFI_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
 }
@@ -274,89 +236,15 @@ size_t local_workspace_elems(const chebfi_ctx* ctx, int64_t nb) {
   return (size_t)ctx->grid[2] * ncolp * (size_t)nb;
 }
 
-template <typename R> const R* vtable(const chebfi_ctx* c);
-template <> const float* vtable<float>(const chebfi_ctx* c) { return c->d_vsf.p; }
-template <> const double* vtable<double>(const chebfi_ctx* c) { return c->d_vs.p; }
-template <> const dfl* vtable<dfl>(const chebfi_ctx* c) { return reinterpret_cast<const dfl*>(c->d_vsdf.p); }
-
-template <typename R, int N>
-void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t ldy, int64_t nb, cplx<R>* T,
-                 LocalEpi<typename SphT<R>::type> ep, cudaStream_t st, const typename SphT<R>::type* K) {
-  using S = typename SphT<R>::type;
-  const SphereFFT& s = ctx->sph;
-  FastArgs fa;
-  fa.ncol = s.ncol;
-  fa.nxa = s.nxa;
-  fa.pitch = s.pitch;
-  fa.zpitch = s.zpitch;
-  fa.ncolp = (s.ncol + 15) / 16 * 16;
-  fa.ldt = (int64_t)N * fa.ncolp;
-  fa.col_start = s.col_start.p;
-  fa.pw_line = s.pw_line.p;
-  fa.pw_z = s.pw_z.p;
-  fa.col_off = s.col_off_nat.p;
-  fa.row_off = s.rows_nat.p;
-  fa.row_col = s.row_col.p;
-  fa.act_lo = s.act_lo;
-  fa.nact = s.nact;
-  // ceil(2^32 / nact): exact quotients t / nact for t < 2^32 / nact (the row passes use t < 2^12)
-  fa.nl_magic = s.nact > 1 ? (unsigned)(((1ull << 32) + s.nact - 1) / (unsigned long long)s.nact) : 0u;
-  CHEBFI_REQUIRE(s.nxa >= 1 && s.nact >= 1, CHEBFI_ERR_STATE, "sphere without columns");
-  CHEBFI_REQUIRE(s.pitch == N + 1, CHEBFI_ERR_STATE, "plane pitch of the compile-time path");
-  const cplx<R>* tw = nullptr;  // the passes read their twiddles from constant tables
-  const R* Vs = vtable<R>(ctx);
-  const size_t zbytes = (size_t)(N + kCBF * s.zpitch) * sizeof(cplx<R>);
-  const size_t pbytes = (size_t)(N + N * s.pitch) * sizeof(cplx<R>);
-  fk::init_twiddles();
-  set_smem<R>((const void*)k_plane_f<R, N>, pbytes);
-  set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
-  set_smem<R>((const void*)k_zfwd_f<R, N>, zbytes);
-  for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
-    const int nbc = (int)std::min<int64_t>(65535, nb - b0);
-    dim3 gz((s.ncol + kCBF - 1) / kCBF, nbc);
-    const double esz = sizeof(cplx<R>), col = (double)N * s.ncol * nbc * esz, sph = (double)ctx->npw * nbc * esz;
-    CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
-    CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col,
-                    k_plane_f<R, N><<<dim3(N, nbc), PlaneThreads<R>::v, pbytes, st>>>(T, Vs, fa, tw));
-    LocalEpi<S> e = ep;
-    e.Y = ep.Y + b0 * ep.ldy;
-    if (e.Z) e.Z = ep.Z + b0 * ep.ldz;
-    if (e.Zhi) {
-      e.Zhi = ep.Zhi + b0 * ep.ldzb;
-      e.Zlo = ep.Zlo + b0 * ep.ldzb;
-    }
-    if (e.T) e.T = ep.T + b0 * ep.ldt;
-    if (e.Yprev) e.Yprev = ep.Yprev + b0 * ep.ldt;
-    e.inv_n3 = (S)(1.0 / ((double)N * N * N));
-    const double epi = sph * (1.0 + (e.Z ? 1.0 : 0.0) + (e.T ? 1.0 : 0.0) + (e.Yprev ? 1.0 : 0.0)) +
-                       (e.Zhi ? (double)ctx->npw * nbc * (e.zplane ? 12.0 : 8.0) : 0.0);
-    CHEBFI_LAUNCH_W("k_zfwd", st, col + epi, k_zfwd_f<R, N><<<gz, kThreads, zbytes, st>>>(T, fa, tw, K, e));
-  }
-}
-
-// Compile-time-length path for cubic grids of the supported sizes; false = not taken.
-template <typename R>
-bool fast_dispatch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t ldy, int64_t nb, cplx<R>* T,
-                   LocalEpi<typename SphT<R>::type> ep, cudaStream_t st, const typename SphT<R>::type* K) {
-  switch (ctx->grid[0]) {
-    case 24: fast_launch<R, 24>(ctx, Y, ldy, nb, T, ep, st, K); return true;
-    case 32: fast_launch<R, 32>(ctx, Y, ldy, nb, T, ep, st, K); return true;
-    case 48: fast_launch<R, 48>(ctx, Y, ldy, nb, T, ep, st, K); return true;
-    case 64: fast_launch<R, 64>(ctx, Y, ldy, nb, T, ep, st, K); return true;
-    case 72: fast_launch<R, 72>(ctx, Y, ldy, nb, T, ep, st, K); return true;
-    case 96: fast_launch<R, 96>(ctx, Y, ldy, nb, T, ep, st, K); return true;
-    default: return false;
-  }
-}
-// The FP64 path runs its transforms in double-float on the FP32 units unless the FP64 units
-// are asked for (chebfi_set_fft64); the column buffer's complex doubles then hold
+// The FP64 path runs its transforms in double-float on the FP32 units, at the lengths that
+// have them, unless the FP64 units are asked for (chebfi_set_fft64); the column buffer's complex doubles then hold
 // double-float values, 16 bytes each as well.
 template <typename R>
 bool fast_apply(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx<R>* T, LocalEpi<R> ep,
                 cudaStream_t st, const R* K) {
   if constexpr (std::is_same<R, double>::value) {
-    if (ctx->fft64 == CHEBFI_FFT64_DOUBLE_FLOAT)
-      return fast_dispatch<dfl>(ctx, Y, ldy, nb, reinterpret_cast<cdf*>(T), ep, st, K);
+    if (ctx->fft64 == CHEBFI_FFT64_DOUBLE_FLOAT && fast_dispatch<dfl>(ctx, Y, ldy, nb, reinterpret_cast<cdf*>(T), ep, st, K))
+      return true;
   }
   return fast_dispatch<R>(ctx, Y, ldy, nb, T, ep, st, K);
 }
@@ -364,19 +252,20 @@ bool fast_apply(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx
 bool fast_fft_supported(int n1, int n2, int n3) {
   if (n1 != n2 || n1 != n3) return false;
   switch (n1) {
-    case 24: case 32: case 48: case 64: case 72: case 96: return true;
+#define CHEBFI_X(n) case n:
+    CHEBFI_FFT_SIZES(CHEBFI_X)
+#undef CHEBFI_X
+    return true;
     default: return false;
   }
 }
 
 int split_index(int n, int p) {
   switch (n) {
-    case 24: return fast::split_index<24>(p);
-    case 32: return fast::split_index<32>(p);
-    case 48: return fast::split_index<48>(p);
-    case 64: return fast::split_index<64>(p);
-    case 72: return fast::split_index<72>(p);
-    case 96: return fast::split_index<96>(p);
+#define CHEBFI_X(n) \
+  case n: return fast::split_index<n>(p);
+    CHEBFI_FFT_SIZES(CHEBFI_X)
+#undef CHEBFI_X
     default: return p;
   }
 }

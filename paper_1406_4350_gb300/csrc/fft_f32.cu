@@ -1,0 +1,7 @@
+// The compile-time-length FFT passes in FP32.
+#include "fft_launch_impl.cuh"
+
+namespace chebfi {
+template bool fast_dispatch<float>(chebfi_ctx*, const cplx<float>*, int64_t, int64_t, cplx<float>*, LocalEpi<float>, cudaStream_t,
+                                const float*);
+}  // namespace chebfi

@@ -1,0 +1,7 @@
+// The compile-time-length FFT passes in the FP64 units.
+#include "fft_launch_impl.cuh"
+
+namespace chebfi {
+template bool fast_dispatch<double>(chebfi_ctx*, const cplx<double>*, int64_t, int64_t, cplx<double>*, LocalEpi<double>, cudaStream_t,
+                                const double*);
+}  // namespace chebfi

@@ -17,26 +17,11 @@
 namespace chebfi {
 namespace fast {
 
-// cos(2 pi m / L), sin(2 pi m / L) for the composite codelet lengths
+// cos(2 pi m / L), sin(2 pi m / L) for the composite codelet lengths with twiddles
 template <int L> struct SmallTw;
-#define CHEBFI_R32 0.86602540378443864676
 #define CHEBFI_R22 0.70710678118654752440
 #define CHEBFI_C8 0.92387953251128675613
 #define CHEBFI_S8 0.38268343236508977173
-#define CHEBFI_C5a 0.30901699437494742410
-#define CHEBFI_S5a 0.95105651629515357212
-#define CHEBFI_C5b 0.80901699437494742410
-#define CHEBFI_S5b 0.58778525229247312917
-template <> struct SmallTw<6> {
-  __host__ __device__ static double c(int m) {
-    const double t[6] = {1, 0.5, -0.5, -1, -0.5, 0.5};
-    return t[m];
-  }
-  __host__ __device__ static double s(int m) {
-    const double t[6] = {0, CHEBFI_R32, CHEBFI_R32, 0, -CHEBFI_R32, -CHEBFI_R32};
-    return t[m];
-  }
-};
 template <> struct SmallTw<8> {
   __host__ __device__ static double c(int m) {
     const double t[8] = {1, CHEBFI_R22, 0, -CHEBFI_R22, -1, -CHEBFI_R22, 0, CHEBFI_R22};
@@ -47,23 +32,13 @@ template <> struct SmallTw<8> {
     return t[m];
   }
 };
-template <> struct SmallTw<10> {
+template <> struct SmallTw<9> {  // multiples of 40 degrees; the codelet uses m = 1, 2, 4
   __host__ __device__ static double c(int m) {
-    const double t[10] = {1, CHEBFI_C5b, CHEBFI_C5a, -CHEBFI_C5a, -CHEBFI_C5b, -1, -CHEBFI_C5b, -CHEBFI_C5a, CHEBFI_C5a, CHEBFI_C5b};
+    const double t[5] = {1, 0.76604444311897803520, 0.17364817766693034885, -0.5, -0.93969262078590838405};
     return t[m];
   }
   __host__ __device__ static double s(int m) {
-    const double t[10] = {0, CHEBFI_S5b, CHEBFI_S5a, CHEBFI_S5a, CHEBFI_S5b, 0, -CHEBFI_S5b, -CHEBFI_S5a, -CHEBFI_S5a, -CHEBFI_S5b};
-    return t[m];
-  }
-};
-template <> struct SmallTw<12> {
-  __host__ __device__ static double c(int m) {
-    const double t[12] = {1, CHEBFI_R32, 0.5, 0, -0.5, -CHEBFI_R32, -1, -CHEBFI_R32, -0.5, 0, 0.5, CHEBFI_R32};
-    return t[m];
-  }
-  __host__ __device__ static double s(int m) {
-    const double t[12] = {0, 0.5, CHEBFI_R32, 1, CHEBFI_R32, 0.5, 0, -0.5, -CHEBFI_R32, -1, -CHEBFI_R32, -0.5};
+    const double t[5] = {0, 0.64278760968653932632, 0.98480775301220805937, 0.86602540378443864676, 0.34202014332566873304};
     return t[m];
   }
 };
@@ -83,9 +58,18 @@ template <> struct SmallTw<16> {
 template <int L> struct Split;  // L = A * B for the composite codelets
 template <> struct Split<6> { static constexpr int A = 2, B = 3; };
 template <> struct Split<8> { static constexpr int A = 2, B = 4; };
+template <> struct Split<9> { static constexpr int A = 3, B = 3; };
 template <> struct Split<10> { static constexpr int A = 2, B = 5; };
 template <> struct Split<12> { static constexpr int A = 4, B = 3; };
 template <> struct Split<16> { static constexpr int A = 4, B = 4; };
+
+// x with x a = 1 (mod b)
+constexpr int inv_mod(int a, int b) {
+  int x = 1;
+  while (x * a % b != 1 % b) ++x;
+  return x;
+}
+constexpr int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
 
 // In-register DFT of length L, natural order in and out: X[k] = sum_n x[n] exp(SIGN 2 pi i nk/L).
 template <int L, int SIGN, typename C> __host__ __device__ __forceinline__ void dft(C* x) {
@@ -95,6 +79,31 @@ template <int L, int SIGN, typename C> __host__ __device__ __forceinline__ void 
   } else {
     constexpr int A = Split<L>::A, B = Split<L>::B;
     C y[L];
+    if constexpr (gcd(A, B) == 1) {
+      // coprime factors (Good 1958, Thomas 1963): n = B a + A b and k = ka B (B^-1 mod A) +
+      // kb A (A^-1 mod B) modulo L turn the transform into A x B without twiddles; in registers
+      // the two permutations cost nothing (length 12: four complex products less)
+      constexpr int ea = B * inv_mod(B % A, A), eb = A * inv_mod(A % B, B);
+#pragma unroll
+      for (int nb = 0; nb < B; ++nb) {
+        C t[A];
+#pragma unroll
+        for (int na = 0; na < A; ++na) t[na] = x[(B * na + A * nb) % L];
+        dft<A, SIGN>(t);
+#pragma unroll
+        for (int ka = 0; ka < A; ++ka) y[ka * B + nb] = t[ka];
+      }
+#pragma unroll
+      for (int ka = 0; ka < A; ++ka) {
+        C u[B];
+#pragma unroll
+        for (int nb = 0; nb < B; ++nb) u[nb] = y[ka * B + nb];
+        dft<B, SIGN>(u);
+#pragma unroll
+        for (int kb = 0; kb < B; ++kb) x[(ea * ka + eb * kb) % L] = u[kb];
+      }
+      return;
+    } else {
 #pragma unroll
     for (int nb = 0; nb < B; ++nb) {
       C t[A];
@@ -136,21 +145,38 @@ template <int L, int SIGN, typename C> __host__ __device__ __forceinline__ void 
 #pragma unroll
       for (int kb = 0; kb < B; ++kb) x[ka + A * kb] = u[kb];
     }
+    }
   }
 }
 
 // Two-factor plan of a line length.
 template <int N> struct Plan;
 template <> struct Plan<16> { static constexpr int NA = 4, NB = 4; };
+template <> struct Plan<20> { static constexpr int NA = 5, NB = 4; };
 template <> struct Plan<24> { static constexpr int NA = 4, NB = 6; };
+template <> struct Plan<30> { static constexpr int NA = 6, NB = 5; };
 template <> struct Plan<32> { static constexpr int NA = 8, NB = 4; };
+template <> struct Plan<36> { static constexpr int NA = 6, NB = 6; };
+template <> struct Plan<40> { static constexpr int NA = 8, NB = 5; };
+template <> struct Plan<45> { static constexpr int NA = 9, NB = 5; };
 template <> struct Plan<48> { static constexpr int NA = 8, NB = 6; };
+template <> struct Plan<54> { static constexpr int NA = 9, NB = 6; };
+template <> struct Plan<60> { static constexpr int NA = 12, NB = 5; };
 template <> struct Plan<64> { static constexpr int NA = 8, NB = 8; };
 template <> struct Plan<72> { static constexpr int NA = 12, NB = 6; };
+template <> struct Plan<80> { static constexpr int NA = 10, NB = 8; };
+template <> struct Plan<90> { static constexpr int NA = 10, NB = 9; };
 template <> struct Plan<96> { static constexpr int NA = 12, NB = 8; };
+template <> struct Plan<100> { static constexpr int NA = 10, NB = 10; };
+template <> struct Plan<108> { static constexpr int NA = 12, NB = 9; };
 template <> struct Plan<120> { static constexpr int NA = 12, NB = 10; };
 template <> struct Plan<128> { static constexpr int NA = 16, NB = 8; };
 template <> struct Plan<144> { static constexpr int NA = 12, NB = 12; };
+
+// the lengths with compiled kernels (fft_launch.cuh); of them, those with double-float kernels
+#define CHEBFI_FFT_SIZES(X) \
+  X(16) X(20) X(24) X(30) X(32) X(36) X(40) X(45) X(48) X(54) X(60) X(64) X(72) X(80) X(90) X(96) X(100) X(108)
+#define CHEBFI_FFT_DF_SIZES(X) X(24) X(32) X(48) X(64) X(72) X(96)
 
 // twiddle w^e = exp(SIGN 2 pi i e / N) from the table tw[e] = exp(-2 pi i e / N), held in
 // memory (a pointer) or behind an accessor object tw(e)

@@ -39,23 +39,23 @@ struct FastArgs {
   unsigned nl_magic = 0;                       // t / nact == umulhi(t, nl_magic) for t < 2^16
 };
 
-template <typename R, int N>
-__device__ __forceinline__ void load_tw(cplx<R>* s, const cplx<R>* g) {
-  for (int i = threadIdx.x; i < N; i += blockDim.x) s[i] = g[i];
-}
-
 // Twiddle tables tw[e] = exp(-2 pi i e / N) of the compiled line lengths, in constant memory:
 // a warp of a pass reads one entry (two where it straddles two sub-transforms), which the
 // constant cache broadcasts without using the shared-memory pipe that bounds these kernels.
 // Each translation unit has its own copy, filled by init_twiddles before its first launch.
-template <int N> struct TwOff;
-template <> struct TwOff<24> { static constexpr int v = 0; };
-template <> struct TwOff<32> { static constexpr int v = 24; };
-template <> struct TwOff<48> { static constexpr int v = 56; };
-template <> struct TwOff<64> { static constexpr int v = 104; };
-template <> struct TwOff<72> { static constexpr int v = 168; };
-template <> struct TwOff<96> { static constexpr int v = 240; };
-constexpr int kTwTotal = 336;
+#define CHEBFI_X(n) n,
+constexpr int kTwLens[] = {CHEBFI_FFT_SIZES(CHEBFI_X)};
+#undef CHEBFI_X
+constexpr int tw_offset(int n) {
+  int o = 0;
+  for (int l : kTwLens) {
+    if (l == n) break;
+    o += l;
+  }
+  return o;
+}
+constexpr int kTwTotal = tw_offset(0);  // 0 is no length: the sum of all
+template <int N> struct TwOff { static constexpr int v = tw_offset(N); };
 static __constant__ float2 c_twf[kTwTotal];
 static __constant__ double2 c_twd[kTwTotal];
 static __constant__ float4 c_twdf[kTwTotal];  // double-float: (re.h, re.l, im.h, im.l)
@@ -81,11 +81,10 @@ static inline void init_twiddles() {
   int dev = 0;
   CHEBFI_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || done[dev]) return;
-  const int lens[6] = {24, 32, 48, 64, 72, 96};
   std::vector<float2> f;
   std::vector<double2> d;
   std::vector<float4> df;
-  for (int n : lens)
+  for (int n : kTwLens)
     for (int k = 0; k < n; ++k) {
       const double a = 2.0 * M_PI * (double)k / (double)n;
       d.push_back(make_double2(std::cos(a), -std::sin(a)));
@@ -107,7 +106,7 @@ __device__ __forceinline__ void zinv_body(const cplx<typename SphT<R>::type>* __
                                           unsigned char* smem_raw) {
   (void)twz;
   const ConstTw<R, N3> tw;
-  cplx<R>* lines = reinterpret_cast<cplx<R>*>(smem_raw) + N3;
+  cplx<R>* lines = reinterpret_cast<cplx<R>*>(smem_raw);
   const int nc = min(kCBF, fa.ncol - c0);
   const cplx<R> zero = cmake<cplx<R>>(0.0, 0.0);
   for (int i = threadIdx.x; i < kCBF * fa.zpitch; i += blockDim.x) lines[i] = zero;
@@ -137,7 +136,7 @@ __device__ __forceinline__ void plane_body(cplx<R>* __restrict__ T, const R* __r
                                            unsigned char* smem_raw) {
   (void)twxy;
   const ConstTw<R, N> tw;
-  cplx<R>* plane = reinterpret_cast<cplx<R>*>(smem_raw) + N;
+  cplx<R>* plane = reinterpret_cast<cplx<R>*>(smem_raw);
   const cplx<R> zero = cmake<cplx<R>>(0.0, 0.0);
   for (int i = threadIdx.x; i < N * fa.pitch; i += blockDim.x) plane[i] = zero;
   __syncthreads();
@@ -182,23 +181,25 @@ __device__ __forceinline__ void plane_body(cplx<R>* __restrict__ T, const R* __r
   for (int c = threadIdx.x; c < fa.ncol; c += blockDim.x) t[c] = plane[fa.col_off[c]];
 }
 
+// rows of a plane are an odd pitch apart: the row-wise passes meet no bank conflicts
+constexpr int plane_pitch(int n) { return n % 2 ? n : n + 1; }
+
 // The plane pass of plane_body with its zero rows pruned and its scatter / gather fused:
 // the first y pass reads the sphere columns straight from the column buffer (no zeroed
 // plane, no scatter), the x passes skip the loads of rows outside the active slot range
 // [act_lo, act_lo + nact) (they are zero) and the stores of rows no later pass reads, and
 // the last y pass stores the columns straight to the column buffer (no gather).  Same
-// arithmetic, in the same order.  The row pitch is the compile-time N + 1 (odd: the
-// row-wise passes meet no bank conflicts), so every shared-memory offset of a pass is an
+// arithmetic, in the same order.  The row pitch is the compile-time plane_pitch(N), so every shared-memory offset of a pass is an
 // immediate; where the block's NT / 32 warps are a multiple of NB (N = 64, 96) each warp of
 // an x pass keeps one nb and its twiddles in registers.
 template <typename R, int N, int NT = kThreadsF>
 __device__ __forceinline__ void plane_body_pruned(cplx<R>* __restrict__ T, const R* __restrict__ Vs,
                                                   const FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
   using C = cplx<R>;
-  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = N + 1, W = NT / 32;
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N), W = NT / 32;
   constexpr bool kWarpNb = N % 32 == 0 && W % NB == 0;
   const ConstTw<R, N> tw;
-  C* plane = reinterpret_cast<C*>(smem_raw) + N;
+  C* plane = reinterpret_cast<C*>(smem_raw);
   const C zero = cmake<C>(0.0, 0.0);
   C* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
   const int nl = fa.nact, lo = fa.act_lo;
@@ -379,7 +380,7 @@ __device__ __forceinline__ void zfwd_body(const cplx<R>* __restrict__ T, const F
   using CS = cplx<typename SphT<R>::type>;
   (void)twz;
   const ConstTw<R, N3> tw;
-  cplx<R>* lines = reinterpret_cast<cplx<R>*>(smem_raw) + N3;
+  cplx<R>* lines = reinterpret_cast<cplx<R>*>(smem_raw);
   const int nc = min(kCBF, fa.ncol - c0);
   const cplx<R>* t = T + b * fa.ldt + c0;
   {

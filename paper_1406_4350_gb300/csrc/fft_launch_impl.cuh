@@ -1,0 +1,133 @@
+// Kernels and launches of the compile-time-length FFT path of the local-potential operator
+// (Section 2.1): the definition of fast_dispatch<R>, included by one translation unit per
+// arithmetic R.
+#pragma once
+
+#include "fft_launch.cuh"
+
+namespace chebfi {
+namespace {
+constexpr int kThreads = 256;
+
+// ---------------------------------------------------------------- compile-time-length path
+// The pass bodies live in fft_fast_kernels.cuh; here each block finds its columns or plane
+// from its grid position.
+using fk::FastArgs;
+using fk::kCBF;
+
+// R: the arithmetic of the transforms (float, double, or dfl, the double-float form of the
+// FP64 path); blocks, the kinetic diagonal and the epilogue's operands are stored in
+// SphT<R> (double for dfl), the column buffer and the planes in cplx<R>.
+template <typename R, int N3>
+__global__ void __launch_bounds__(kThreads) k_zinv_f(const cplx<typename SphT<R>::type>* __restrict__ Y, int64_t ldy,
+                                                     cplx<R>* __restrict__ T, FastArgs fa, const cplx<R>* __restrict__ twz) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fk::zinv_body<R, N3>(Y, ldy, T, fa, twz, blockIdx.x * kCBF, blockIdx.y, smem_raw);
+}
+
+// threads of a plane block: the double-float plane (16 bytes a point, one block per SM)
+// takes 16 warps to keep its FP32 pipes fed, the others 8 with three blocks per SM
+template <typename R> struct PlaneThreads { static constexpr int v = kThreads; };
+template <> struct PlaneThreads<dfl> { static constexpr int v = 2 * kThreads; };
+
+template <typename R, int N>
+__global__ void __launch_bounds__(PlaneThreads<R>::v) k_plane_f(cplx<R>* __restrict__ T, const R* __restrict__ Vs,
+                                                                FastArgs fa, const cplx<R>* __restrict__ twxy) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  (void)twxy;
+  fk::plane_body_pruned<R, N, PlaneThreads<R>::v>(T, Vs, fa, blockIdx.x, blockIdx.y, smem_raw);
+}
+
+template <typename R, int N3>
+__global__ void __launch_bounds__(kThreads) k_zfwd_f(const cplx<R>* __restrict__ T, FastArgs fa,
+                                                     const cplx<R>* __restrict__ twz,
+                                                     const typename SphT<R>::type* __restrict__ K,
+                                                     LocalEpi<typename SphT<R>::type> ep) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fk::zfwd_body<R, N3>(T, fa, twz, K, ep, blockIdx.x * kCBF, blockIdx.y, smem_raw);
+}
+
+template <typename R> void set_smem(const void* f, size_t bytes) {
+  CHEBFI_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+}
+
+template <typename R> const R* vtable(const chebfi_ctx* c);
+template <> const float* vtable<float>(const chebfi_ctx* c) { return c->d_vsf.p; }
+template <> const double* vtable<double>(const chebfi_ctx* c) { return c->d_vs.p; }
+template <> const dfl* vtable<dfl>(const chebfi_ctx* c) { return reinterpret_cast<const dfl*>(c->d_vsdf.p); }
+
+template <typename R, int N>
+void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t ldy, int64_t nb, cplx<R>* T,
+                 LocalEpi<typename SphT<R>::type> ep, cudaStream_t st, const typename SphT<R>::type* K) {
+  using S = typename SphT<R>::type;
+  const SphereFFT& s = ctx->sph;
+  FastArgs fa;
+  fa.ncol = s.ncol;
+  fa.nxa = s.nxa;
+  fa.pitch = s.pitch;
+  fa.zpitch = s.zpitch;
+  fa.ncolp = (s.ncol + 15) / 16 * 16;
+  fa.ldt = (int64_t)N * fa.ncolp;
+  fa.col_start = s.col_start.p;
+  fa.pw_line = s.pw_line.p;
+  fa.pw_z = s.pw_z.p;
+  fa.col_off = s.col_off_nat.p;
+  fa.row_off = s.rows_nat.p;
+  fa.row_col = s.row_col.p;
+  fa.act_lo = s.act_lo;
+  fa.nact = s.nact;
+  // ceil(2^32 / nact): exact quotients t / nact for t < 2^32 / nact (the row passes use t < 2^12)
+  fa.nl_magic = s.nact > 1 ? (unsigned)(((1ull << 32) + s.nact - 1) / (unsigned long long)s.nact) : 0u;
+  CHEBFI_REQUIRE(s.nxa >= 1 && s.nact >= 1, CHEBFI_ERR_STATE, "sphere without columns");
+  CHEBFI_REQUIRE(s.pitch == fk::plane_pitch(N), CHEBFI_ERR_STATE, "plane pitch of the compile-time path");
+  const cplx<R>* tw = nullptr;  // the passes read their twiddles from constant tables
+  const R* Vs = vtable<R>(ctx);
+  const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
+  const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
+  fk::init_twiddles();
+  set_smem<R>((const void*)k_plane_f<R, N>, pbytes);
+  set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
+  set_smem<R>((const void*)k_zfwd_f<R, N>, zbytes);
+  for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
+    const int nbc = (int)std::min<int64_t>(65535, nb - b0);
+    dim3 gz((s.ncol + kCBF - 1) / kCBF, nbc);
+    const double esz = sizeof(cplx<R>), col = (double)N * s.ncol * nbc * esz, sph = (double)ctx->npw * nbc * esz;
+    CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
+    CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col,
+                    k_plane_f<R, N><<<dim3(N, nbc), PlaneThreads<R>::v, pbytes, st>>>(T, Vs, fa, tw));
+    LocalEpi<S> e = ep;
+    e.Y = ep.Y + b0 * ep.ldy;
+    if (e.Z) e.Z = ep.Z + b0 * ep.ldz;
+    if (e.Zhi) {
+      e.Zhi = ep.Zhi + b0 * ep.ldzb;
+      e.Zlo = ep.Zlo + b0 * ep.ldzb;
+    }
+    if (e.T) e.T = ep.T + b0 * ep.ldt;
+    if (e.Yprev) e.Yprev = ep.Yprev + b0 * ep.ldt;
+    e.inv_n3 = (S)(1.0 / ((double)N * N * N));
+    const double epi = sph * (1.0 + (e.Z ? 1.0 : 0.0) + (e.T ? 1.0 : 0.0) + (e.Yprev ? 1.0 : 0.0)) +
+                       (e.Zhi ? (double)ctx->npw * nbc * (e.zplane ? 12.0 : 8.0) : 0.0);
+    CHEBFI_LAUNCH_W("k_zfwd", st, col + epi, k_zfwd_f<R, N><<<gz, kThreads, zbytes, st>>>(T, fa, tw, K, e));
+  }
+}
+
+}  // namespace
+
+// Compile-time-length path for cubic grids of the compiled sizes; false = not taken.
+template <typename R>
+bool fast_dispatch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t ldy, int64_t nb, cplx<R>* T,
+                   LocalEpi<typename SphT<R>::type> ep, cudaStream_t st, const typename SphT<R>::type* K) {
+  switch (ctx->grid[0]) {
+#define CHEBFI_X(n) \
+  case n: fast_launch<R, n>(ctx, Y, ldy, nb, T, ep, st, K); return true;
+#ifdef CHEBFI_FFT_DF
+    CHEBFI_FFT_DF_SIZES(CHEBFI_X)
+#else
+    CHEBFI_FFT_SIZES(CHEBFI_X)
+#endif
+#undef CHEBFI_X
+    default: return false;
+  }
+}
+
+}  // namespace chebfi

@@ -123,3 +123,18 @@ def test_rayleigh_ritz_route_edges(nb, shells):
     np.testing.assert_allclose(Yg.conj().T @ op.apply_S(Yg), np.eye(nb), atol=tol)
     np.testing.assert_allclose(Yg.conj().T @ op.apply_H(Yg), np.diag(w), atol=tol * scale)
     np.testing.assert_allclose(_np(rs), ch.residuals(op, Yg, w), atol=tol * scale)
+
+
+# every grid length with compiled FFT passes (and two without: 18 and 50), a sphere that is
+# not centred (general k), band counts that leave the last block ragged
+@pytest.mark.parametrize("n", [16, 18, 20, 24, 30, 32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 80, 90, 96, 100, 108])
+def test_apply_h_on_every_grid_length(n):
+    L = 0.42 * n
+    ecut = 0.5 * (2.0 * np.pi / L * 0.24 * n) ** 2
+    cell = make_cell(L, n, ecut, 1, 8, 3, True, 35, kpt=(0.02, -0.05, 0.03))
+    ref = PWOperator.from_cell(cell).apply_H(cell.Y0)
+    g = _ctx(cell)
+    scale = np.abs(ref).max()
+    # the parity tolerances of the FP64 and FP32 forms
+    assert np.abs(_np(g.apply_H(_F(cell.Y0), prec=0)) - ref).max() <= 1e-11 * scale
+    assert np.abs(_np(g.apply_H(_F(cell.Y0), prec=1)) - ref).max() <= 2e-5 * scale
