@@ -1416,14 +1416,23 @@ int chebfi_set_vloc(chebfi_ctx* ctx, const double* vloc, int on_device) {
           vs[((size_t)pz * n1 + px) * n2 + py] = v;
           vsf[((size_t)pz * n1 + px) * n2 + py] = (float)v;
         }
-    std::vector<float2> vsdf(n);
-    for (size_t i = 0; i < (size_t)n; ++i) {
-      const float h = (float)vs[i];
-      vsdf[i] = make_float2(h, (float)(vs[i] - (double)h));
+    // |V_loc| < 2^e (1 - 2^-31); both parts are exact roundings of the scaled double
+    double top = 0.0;
+    for (size_t i = 0; i < n; ++i) top = std::max(top, std::fabs(vs[i]));
+    int e = 0;
+    if (top > 0.0) {
+      std::frexp(top, &e);
+      if (top > std::ldexp(1.0 - 1e-9, e)) ++e;
     }
+    std::vector<int2> vsfx(n);
+    for (size_t i = 0; i < n; ++i) {
+      const double s = std::ldexp(vs[i], 31 - e), h = std::nearbyint(s);
+      vsfx[i] = make_int2((int)h, (int)std::nearbyint((s - h) * 2147483648.0));
+    }
+    ctx->v_exp = e;
     ctx->d_vs.upload(vs.data(), n);
     ctx->d_vsf.upload(vsf.data(), n);
-    ctx->d_vsdf.upload(vsdf.data(), n);
+    ctx->d_vsfx.upload(vsfx.data(), n);
   }
   CHEBFI_CUDA(cudaDeviceSynchronize());
   ctx->vmax = vmax;

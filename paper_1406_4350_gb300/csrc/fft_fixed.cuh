@@ -1,0 +1,468 @@
+// The plane pass of the FP64 form in 64-bit fixed point.
+//
+// GB300 issues FP64 FMAs at 1/64 of its FP32 rate; double-float sums (11 packed FP32
+// instructions per complex sum) bound the plane pass instead.  A complex sum of 64-bit
+// integers is four integer instructions, and a transform is mostly sums.  So the planes are
+// transformed as integers with one power-of-two scale per plane (block floating point):
+//
+//  * a component is an integer below 2^62 in magnitude.  Every intermediate value of an
+//    unnormalised transform is a sum of inputs with unit weights, so the sum of the inputs'
+//    magnitudes bounds them all: the inverse transforms' scale makes sum |c| <= 2^61;
+//  * products with constants |c| <= 1 (twiddles, V_loc / 2^e) keep 62-bit constants as two
+//    31-bit parts, c = (h 2^31 + l) 2^-62, and give x c / 2 from three 32 x 32 -> 64-bit
+//    multiply-adds per real product: with x = xh 2^32 + 2 xm (+ the dropped lowest bit),
+//      x c / 2 = xh h + (xh l + xm h) 2^-31, rounded.
+//    The halving at each twiddle is headroom that the sums after it use;
+//  * before the forward x and y transforms the plane's largest component, taken while the
+//    plane is stored, sets a new common shift, so the forward passes also start with their
+//    full word length, whatever V_loc's range;
+//  * sums that could pass the word length shift their inputs first, by compile-time amounts.
+//
+// Against the double-float planes: rounding is 1 part in 2^61 of the plane's scale instead of
+// 2^-48 of each value.  A complex sum issues in 5 clocks per warp and scheduler (double-float:
+// 24), a twiddle product in 87 (55), so the pass is now bound by its products; per
+// 256-band application at 48^3 0.86 -> 0.60 ms, per 2048 at 96^3 48.5 -> 41 ms.
+#pragma once
+
+#include <cmath>
+
+#include "dfloat.cuh"
+#include "fft_fast.cuh"
+#include "fft_fast_kernels.cuh"
+
+namespace chebfi {
+namespace fx {
+
+using ll = long long;
+struct cfx {
+  ll x, y;
+};
+
+// c = (h 2^31 + l) 2^-62, |c| <= 1 (1 itself as the largest representable value)
+struct Cst {
+  int h, l;
+};
+__host__ __device__ constexpr Cst make_cst(double c) {
+  const double s = c * 2147483648.0;
+  ll h = (ll)(s + (s >= 0 ? 0.5 : -0.5));
+  if (h > 2147483647) h = 2147483647;
+  if (h < -2147483647) h = -2147483647;
+  const double r = (s - (double)h) * 2147483648.0;
+  ll l = (ll)(r + (r >= 0 ? 0.5 : -0.5));
+  if (l > 2147483647) l = 2147483647;
+  if (l < -2147483647) l = -2147483647;
+  return Cst{(int)h, (int)l};
+}
+
+__device__ __forceinline__ int hi32(ll v) { return (int)(v >> 32); }
+__device__ __forceinline__ int mid31(ll v) { return (int)((unsigned)v >> 1); }
+__device__ __forceinline__ ll mad(int a, int b, ll c) { return (ll)a * (ll)b + c; }
+constexpr ll kHalfUlp = 1ll << 30;
+
+// x c / 2
+__device__ __forceinline__ ll mulh(ll x, Cst c) {
+  ll u = mad(hi32(x), c.l, kHalfUlp);
+  u = mad(mid31(x), c.h, u);
+  return mad(hi32(x), c.h, u >> 31);
+}
+__device__ __forceinline__ cfx operator+(cfx a, cfx b) { return cfx{a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ cfx operator-(cfx a, cfx b) { return cfx{a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ cfx sar(cfx a, int s) { return cfx{a.x >> s, a.y >> s}; }
+// a (c + i s) / 2: the two products of a component share their carry chain (|c| + |s| <= sqrt 2)
+__device__ __forceinline__ cfx cmulh(cfx a, Cst c, Cst s) {
+  const int xh = hi32(a.x), xm = mid31(a.x), yh = hi32(a.y), ym = mid31(a.y);
+  ll u = mad(xh, c.l, kHalfUlp), v = mad(xh, s.l, kHalfUlp);
+  u = mad(xm, c.h, u);
+  v = mad(xm, s.h, v);
+  u = mad(yh, -s.l, u);
+  v = mad(yh, c.l, v);
+  u = mad(ym, -s.h, u);
+  v = mad(ym, c.h, v);
+  cfx r;
+  r.x = mad(yh, -s.h, mad(xh, c.h, u >> 31));
+  r.y = mad(yh, c.h, mad(xh, s.h, v >> 31));
+  return r;
+}
+// SIGN i a
+template <int SIGN> __device__ __forceinline__ cfx rot(cfx a) { return SIGN > 0 ? cfx{-a.y, a.x} : cfx{a.y, -a.x}; }
+
+// In-register transforms, natural order in and out (fast::dft on integers).
+template <int L, int SIGN> __device__ __forceinline__ void dft(cfx* x) {
+  if constexpr (L == 1) {
+  } else if constexpr (L == 2) {
+    const cfx a = x[0], b = x[1];
+    x[0] = a + b;
+    x[1] = a - b;
+  } else if constexpr (L == 3) {
+    constexpr Cst h = make_cst(0.86602540378443864676);
+    const cfx s = x[1] + x[2], d = x[1] - x[2];
+    const cfx t = x[0] - sar(s, 1);
+    cfx u{mulh(d.y, h), mulh(d.x, h)};  // half of sqrt(3)/2 (d.y, d.x)
+    u = cfx{u.x + u.x, u.y + u.y};
+    x[0] = x[0] + s;
+    if (SIGN > 0) {
+      x[1] = cfx{t.x - u.x, t.y + u.y};
+      x[2] = cfx{t.x + u.x, t.y - u.y};
+    } else {
+      x[1] = cfx{t.x + u.x, t.y - u.y};
+      x[2] = cfx{t.x - u.x, t.y + u.y};
+    }
+  } else if constexpr (L == 4) {
+    const cfx a = x[0] + x[2], b = x[0] - x[2], c = x[1] + x[3], d = x[1] - x[3];
+    x[0] = a + c;
+    x[2] = a - c;
+    if (SIGN > 0) {
+      x[1] = cfx{b.x - d.y, b.y + d.x};
+      x[3] = cfx{b.x + d.y, b.y - d.x};
+    } else {
+      x[1] = cfx{b.x + d.y, b.y - d.x};
+      x[3] = cfx{b.x - d.y, b.y + d.x};
+    }
+  } else if constexpr (L == 8) {
+    constexpr Cst h = make_cst(0.70710678118654752440);
+    cfx e[4], o[4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      e[n] = x[n] + x[n + 4];
+      o[n] = x[n] - x[n + 4];
+    }
+    // o[1] w, o[3] w^3, w = exp(SIGN i pi / 4): (1 + SIGN i) / sqrt 2 and (-1 + SIGN i) / sqrt 2
+    const cfx p = o[1] + rot<SIGN>(o[1]), q = rot<SIGN>(o[3]) - o[3];
+    const cfx ph{mulh(p.x, h), mulh(p.y, h)}, qh{mulh(q.x, h), mulh(q.y, h)};
+    o[1] = cfx{ph.x + ph.x, ph.y + ph.y};
+    o[2] = rot<SIGN>(o[2]);
+    o[3] = cfx{qh.x + qh.x, qh.y + qh.y};
+    dft<4, SIGN>(e);
+    dft<4, SIGN>(o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[2 * k] = e[k];
+      x[2 * k + 1] = o[k];
+    }
+  } else {
+    constexpr int A = fast::Split<L>::A, B = fast::Split<L>::B;
+    static_assert(fast::gcd(A, B) == 1, "coprime factors only");
+    constexpr int ea = B * fast::inv_mod(B % A, A), eb = A * fast::inv_mod(A % B, B);
+    cfx y[L];
+#pragma unroll
+    for (int nb = 0; nb < B; ++nb) {
+      cfx t[A];
+#pragma unroll
+      for (int na = 0; na < A; ++na) t[na] = x[(B * na + A * nb) % L];
+      dft<A, SIGN>(t);
+#pragma unroll
+      for (int ka = 0; ka < A; ++ka) y[ka * B + nb] = t[ka];
+    }
+#pragma unroll
+    for (int ka = 0; ka < A; ++ka) {
+      dft<B, SIGN>(y + ka * B);
+#pragma unroll
+      for (int kb = 0; kb < B; ++kb) x[(ea * ka + eb * kb) % L] = y[ka * B + kb];
+    }
+  }
+}
+
+// upper bounds of 8 log2 n, the bits by which an n-point transform can grow
+constexpr int grow8(int n) {
+  return n <= 1 ? 0 : n == 2 ? 8 : n == 3 ? 13 : n == 4 ? 16 : n == 5 ? 19 : n == 6 ? 21 : n <= 8 ? 24 : n <= 9 ? 26 : n <= 10 ? 27 : n <= 12 ? 29 : 32;
+}
+constexpr int kTop8 = 8 * 61 + 4;  // magnitudes stay below 2^61.5
+// shift before an n-point transform of values below 2^(b8 / 8), and the bound after it
+constexpr int pre_shift(int b8, int n) {
+  int s = 0;
+  while (b8 - 8 * s + grow8(n) > kTop8) ++s;
+  return s;
+}
+constexpr int after(int b8, int n) { return b8 - 8 * pre_shift(b8, n) + grow8(n); }
+
+// Twiddles (cos, -sin)(2 pi e / N) of the compiled lengths as (c.h, c.l, s.h, s.l); filled by
+// init_twiddles before a translation unit's first launch.
+static __constant__ int4 c_twfx[fk::kTwTotal];
+template <int N, int SIGN> __device__ __forceinline__ void twiddle(int e, Cst& c, Cst& s) {
+  const int4 w = c_twfx[fk::TwOff<N>::v + e];
+  c = Cst{w.x, w.y};
+  s = SIGN > 0 ? Cst{-w.z, -w.w} : Cst{w.z, w.w};
+}
+static inline void init_twiddles() {
+  static bool done[64] = {false};
+  int dev = 0;
+  CHEBFI_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64 || done[dev]) return;
+  std::vector<int4> t;
+  for (int n : fk::kTwLens)
+    for (int k = 0; k < n; ++k) {
+      const long double a = 2.0L * 3.14159265358979323846264338327950288L * k / n;
+      // the two parts from the extended-precision value: 62 bits
+      auto part = [](long double v) {
+        const long double s = v * 2147483648.0L;
+        ll h = std::llround(s);
+        h = std::max(-2147483647ll, std::min(2147483647ll, h));
+        ll l = std::llround((s - (long double)h) * 2147483648.0L);
+        l = std::max(-2147483647ll, std::min(2147483647ll, l));
+        return std::make_pair((int)h, (int)l);
+      };
+      const auto c = part(std::cos(a)), s = part(-std::sin(a));
+      t.push_back(make_int4(c.first, c.second, s.first, s.second));
+    }
+  CHEBFI_CUDA(cudaMemcpyToSymbol(c_twfx, t.data(), sizeof(int4) * t.size()));
+  done[dev] = true;
+}
+
+// 2^e as a float, |e| <= 126
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+// v 2^e for |e| <= 252, in two exact steps (where the result is a normal float)
+struct Pow2 {
+  float a, b;
+};
+__device__ __forceinline__ Pow2 pow2(int e) {
+  const int i = max(-126, min(126, e)), j = max(-126, min(126, e - i));
+  return Pow2{pow2f(i), pow2f(j)};
+}
+__device__ __forceinline__ float scale(float v, Pow2 p) { return __fmul_rn(__fmul_rn(v, p.a), p.b); }
+
+// The conversions between scaled double-float values and integers, chunk by chunk through
+// 1.5 2^23 (adding it rounds a float below 2^22 to an integer in the low mantissa bits): the
+// 64-bit conversion instructions issue every 65 clocks per warp, which made them a third of
+// the pass (96^3: 45.8 ms per 2048-band application, now 41).
+constexpr float kMagic = 12582912.0f;
+constexpr int kMagicBits = 0x4B400000;
+// round(v 2^e) for |v 2^e| < 2^61
+__device__ __forceinline__ ll to_fixed(dfl v, Pow2 p) {
+  const float h = scale(v.h, p), l = scale(v.l, p);  // |l| <= 2^37
+  const float ta = __fmaf_rn(h, 0x1p-40f, kMagic);
+  const float r1 = __fmaf_rn(__fsub_rn(ta, kMagic), -0x1p40f, h);   // exact, |r1| <= 2^39
+  const float tb = __fmaf_rn(r1, 0x1p-18f, kMagic);
+  const float r2 = __fmaf_rn(__fsub_rn(tb, kMagic), -0x1p18f, r1);  // exact, |r2| <= 2^17
+  const float tl = __fmaf_rn(l, 0x1p-18f, kMagic);
+  const float r3 = __fmaf_rn(__fsub_rn(tl, kMagic), -0x1p18f, l);   // exact, |r3| <= 2^17
+  const float tc = __fadd_rn(__fadd_rn(r2, r3), kMagic);
+  const int a = __float_as_int(ta) - kMagicBits, b = __float_as_int(tb) + __float_as_int(tl) - 2 * kMagicBits;
+  const int c = __float_as_int(tc) - kMagicBits;
+  return ((ll)(a << 8) << 32) + ((ll)b << 18) + (ll)c;
+}
+// v 2^(e - 21) as a double-float: v = a 2^42 + b 2^21 + c
+__device__ __forceinline__ dfl from_fixed(ll v, Pow2 p) {
+  const float fa = __fsub_rn(__int_as_float(kMagicBits + (int)(v >> 42)), kMagic);  // |a| <= 2^20
+  const float fb = __fsub_rn(__int_as_float(0x4B000000 + ((int)(v >> 21) & 0x1FFFFF)), 8388608.0f);
+  const float fc = __fsub_rn(__int_as_float(0x4B000000 + ((int)v & 0x1FFFFF)), 8388608.0f);
+  // a 2^21 + b, exact as a pair; |a 2^21| >= |b| or a = 0
+  const float h = __fmaf_rn(fa, 0x1p21f, fb), e = __fsub_rn(fb, __fmaf_rn(fa, -0x1p21f, h));
+  const dfl r = df_fast2sum(h, __fmaf_rn(fc, 0x1p-21f, e));
+  return dfl(scale(r.h, p), scale(r.l, p));
+}
+
+// bits of magnitude of the high words: their OR bounds the largest component
+__device__ __forceinline__ unsigned mag(ll v) {
+  const int h = hi32(v);
+  return (unsigned)(h ^ (h >> 31));
+}
+// left shift that brings components with the given OR of magnitudes below 2^(top - 1/2), so
+// that complex magnitudes are below 2^top
+__device__ __forceinline__ int norm_shift(unsigned m, int top) {
+  const int bits = 64 - __clz((int)m);  // components < 2^bits (the high words' bits, above bit 32)
+  return top - 1 - bits;
+}
+__device__ __forceinline__ cfx shl(cfx a, int s) { return cfx{a.x << s, a.y << s}; }
+
+// Plane z of band b (fk::plane_body_pruned in fixed point): inverse y and x transforms,
+// multiply by V_loc (Vs: (h, l) of V_loc / 2^ve in split order), forward x and y.  The column
+// buffer holds double-float pairs.  NT threads; the plane (16 bytes a point) fills the SM's
+// shared memory, so one block runs per SM at N = 96.
+template <int N, int NT>
+__device__ __forceinline__ void plane_body(cdf* __restrict__ T, const int2* __restrict__ Vs, int ve,
+                                           const fk::FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = fk::plane_pitch(N);
+  __shared__ float red[NT / 32];
+  __shared__ unsigned ored[2];
+  // a warp of a y pass holds several nb: its twiddles come from shared memory (the constant
+  // cache serves one address per warp at a time), those of the x passes from constant memory
+  __shared__ int4 tws[N];
+  cfx* plane = reinterpret_cast<cfx*>(smem_raw);
+  cdf* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
+  const int nl = fa.nact, lo = fa.act_lo, tid = threadIdx.x;
+  cfx* rows = plane + lo * P;  // row a of the active range
+  const cfx zero{0, 0};
+  // the scale: 2^s sum (|re| + |im|) <= 2^61 (summed 2^-13 down, against overflow)
+  int s;
+  {
+    float sum = 0.f;
+    for (int c = tid; c < fa.ncol; c += NT) {
+      const cdf v = t[c];
+      sum += (fabsf(v.x.h) + fabsf(v.y.h)) * 1.220703125e-4f;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (tid % 32 == 0) red[tid / 32] = sum;
+    if (tid < 2) ored[tid] = 0u;
+    for (int i = tid; i < N; i += NT) tws[i] = c_twfx[fk::TwOff<N>::v + i];
+    __syncthreads();
+    sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) sum += red[i];
+    if (!(sum < INFINITY)) {  // Inf or NaN in the plane: so is every value of its transform
+      const float q = __int_as_float(0x7fc00000);
+      for (int c = tid; c < fa.ncol; c += NT) t[c] = cdf{dfl(q, q), dfl(q, q)};
+      return;
+    }
+    s = 61 - 13 - (sum > 0.f ? ilogbf(sum) + 1 : 0) - 1;  // one bit spare for the sum's rounding
+  }
+  const Pow2 in = pow2(s);
+  // y, inverse, pass A on the active rows, its inputs read from the column buffer
+  for (int it = tid; it < nl * NB; it += NT) {
+    const int a = it / NB, nb = it - a * NB;
+    cfx* row = rows + a * P + nb;
+    const int32_t* rc = fa.row_col + a * N + nb;
+    cfx v[NA];
+#pragma unroll
+    for (int na = 0; na < NA; ++na) {
+      const int c = __ldg(rc + NB * na);
+      v[na] = zero;
+      if (c >= 0) {
+        const cdf u = t[c];
+        v[na] = cfx{to_fixed(u.x, in), to_fixed(u.y, in)};
+      }
+    }
+    dft<NA, +1>(v);
+    row[0] = sar(v[0], 1);
+#pragma unroll
+    for (int ka = 1; ka < NA; ++ka) {
+      const int4 w = tws[nb * ka];
+      row[NB * ka] = cmulh(v[ka], Cst{w.x, w.y}, Cst{-w.z, -w.w});
+    }
+  }
+  __syncthreads();
+  for (int it = tid; it < nl * NA; it += NT) {  // pass B
+    const int ka = nl == 1 ? it : (int)__umulhi((unsigned)it, fa.nl_magic), a = it - ka * nl;
+    cfx* g = rows + a * P + NB * ka;
+    cfx u[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) u[q] = g[q];
+    dft<NB, +1>(u);
+#pragma unroll
+    for (int q = 0; q < NB; ++q) g[q] = u[q];
+  }
+  __syncthreads();
+  // x, inverse: pass A on every y line, rows outside the active range are zero
+  for (int it = tid; it < N * NB; it += NT) {
+    const int nb = it / N, yy = it - nb * N, d = nb - lo;
+    cfx* a = plane + yy + nb * P;
+    cfx v[NA];
+#pragma unroll
+    for (int na = 0; na < NA; ++na) v[na] = (unsigned)(d + NB * na) < (unsigned)nl ? a[NB * na * P] : zero;
+    dft<NA, +1>(v);
+    a[0] = sar(v[0], 1);
+#pragma unroll
+    for (int ka = 1; ka < NA; ++ka) {
+      Cst c, sn;
+      twiddle<N, +1>(nb * ka, c, sn);
+      a[NB * ka * P] = cmulh(v[ka], c, sn);
+    }
+  }
+  __syncthreads();
+  {  // pass B and the multiply by V_loc; the largest component of the product
+    const int2* v = Vs + (int64_t)z * N * N;
+    unsigned m = 0;
+    for (int it = tid; it < N * NA; it += NT) {
+      const int ka = it / N, yy = it - ka * N;
+      cfx* a = plane + yy + NB * ka * P;
+      const int2* vv = v + (NB * ka) * N + yy;
+      cfx u[NB];
+#pragma unroll
+      for (int q = 0; q < NB; ++q) u[q] = a[q * P];
+      dft<NB, +1>(u);
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        const int2 w = __ldg(vv + q * N);
+        const Cst c{w.x, w.y};
+        u[q] = cfx{mulh(u[q].x, c), mulh(u[q].y, c)};
+        m |= mag(u[q].x) | mag(u[q].y);
+        a[q * P] = u[q];
+      }
+    }
+    m = __reduce_or_sync(0xffffffffu, m);
+    if (tid % 32 == 0 && m) atomicOr(&ored[0], m);
+  }
+  __syncthreads();
+  // forward bounds in 1/8 bits: values enter below 2^58, and again after the x transform
+  constexpr int b0 = 58 * 8;
+  static_assert(pre_shift(b0, NB) == 0, "the normalised plane leaves room for pass B");
+  constexpr int b1 = after(b0, NB) - 8;  // pass B, halved by its twiddles
+  constexpr int s2 = pre_shift(b1, NA);  // pass A
+  // the product is below 2^57 (2^60 of the inverse transforms, halved three times), so its
+  // shift is to the left; the x transform's result may need either direction
+  const int na1 = max(norm_shift(ored[0], 58), 0);
+  // x, forward: pass B with the normalising shift
+  for (int it = tid; it < N * NA; it += NT) {
+    const int ka = it / N, yy = it - ka * N;
+    cfx* a = plane + yy + NB * ka * P;
+    cfx u[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) u[q] = shl(a[q * P], na1);
+    dft<NB, -1>(u);
+    a[0] = sar(u[0], 1);
+#pragma unroll
+    for (int q = 1; q < NB; ++q) {
+      Cst c, sn;
+      twiddle<N, -1>(q * ka, c, sn);
+      a[q * P] = cmulh(u[q], c, sn);
+    }
+  }
+  __syncthreads();
+  {  // pass A, storing only the rows the y pass reads; their largest component
+    unsigned m = 0;
+    for (int it = tid; it < N * NB; it += NT) {
+      const int nb = it / N, yy = it - nb * N, d = nb - lo;
+      cfx* a = plane + yy + nb * P;
+      cfx v[NA];
+#pragma unroll
+      for (int ka = 0; ka < NA; ++ka) v[ka] = sar(a[NB * ka * P], s2);
+      dft<NA, -1>(v);
+#pragma unroll
+      for (int na = 0; na < NA; ++na)
+        if ((unsigned)(d + NB * na) < (unsigned)nl) {
+          m |= mag(v[na].x) | mag(v[na].y);
+          a[NB * na * P] = v[na];
+        }
+    }
+    m = __reduce_or_sync(0xffffffffu, m);
+    if (tid % 32 == 0 && m) atomicOr(&ored[1], m);
+  }
+  __syncthreads();
+  const int na2 = norm_shift(ored[1], 58), up2 = max(na2, 0), down2 = max(-na2, 0);
+  // y, forward: pass B with the normalising shift
+  for (int it = tid; it < nl * NA; it += NT) {
+    const int ka = nl == 1 ? it : (int)__umulhi((unsigned)it, fa.nl_magic), a = it - ka * nl;
+    cfx* g = rows + a * P + NB * ka;
+    cfx u[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) u[q] = sar(shl(g[q], up2), down2);
+    dft<NB, -1>(u);
+    g[0] = sar(u[0], 1);
+#pragma unroll
+    for (int q = 1; q < NB; ++q) {
+      const int4 w = tws[q * ka];
+      g[q] = cmulh(u[q], Cst{w.x, w.y}, Cst{w.z, w.w});
+    }
+  }
+  __syncthreads();
+  // pass A, storing the columns to the column buffer.  Scale so far: s - 2 (inverse twiddles)
+  // - 1 - ve (V_loc), then per forward transform the normalising shift - 1 - s2
+  const Pow2 out = pow2(21 - (s - 3 - ve + (na1 - 1 - s2) + (na2 - 1 - s2)));  // from_fixed's unit is 2^21
+  for (int it = tid; it < nl * NB; it += NT) {
+    const int a = it / NB, nb = it - a * NB;  // consecutive columns per warp
+    const cfx* row = rows + a * P + nb;
+    const int32_t* rc = fa.row_col + a * N + nb;
+    cfx v[NA];
+#pragma unroll
+    for (int ka = 0; ka < NA; ++ka) v[ka] = sar(row[NB * ka], s2);
+    dft<NA, -1>(v);
+#pragma unroll
+    for (int na = 0; na < NA; ++na) {
+      const int c = __ldg(rc + NB * na);
+      if (c >= 0) t[c] = cdf{from_fixed(v[na].x, out), from_fixed(v[na].y, out)};
+    }
+  }
+}
+
+}  // namespace fx
+}  // namespace chebfi

@@ -4,6 +4,9 @@
 #pragma once
 
 #include "fft_launch.cuh"
+#ifdef CHEBFI_FFT_DF
+#include "fft_fixed.cuh"
+#endif
 
 namespace chebfi {
 namespace {
@@ -25,18 +28,24 @@ __global__ void __launch_bounds__(kThreads) k_zinv_f(const cplx<typename SphT<R>
   fk::zinv_body<R, N3>(Y, ldy, T, fa, twz, blockIdx.x * kCBF, blockIdx.y, smem_raw);
 }
 
-// threads of a plane block: the double-float plane (16 bytes a point, one block per SM)
-// takes 16 warps to keep its FP32 pipes fed, the others 8 with three blocks per SM
-template <typename R> struct PlaneThreads { static constexpr int v = kThreads; };
-template <> struct PlaneThreads<dfl> { static constexpr int v = 2 * kThreads; };
-
 template <typename R, int N>
-__global__ void __launch_bounds__(PlaneThreads<R>::v) k_plane_f(cplx<R>* __restrict__ T, const R* __restrict__ Vs,
-                                                                FastArgs fa, const cplx<R>* __restrict__ twxy) {
+__global__ void __launch_bounds__(kThreads) k_plane_f(cplx<R>* __restrict__ T, const R* __restrict__ Vs, FastArgs fa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  (void)twxy;
-  fk::plane_body_pruned<R, N, PlaneThreads<R>::v>(T, Vs, fa, blockIdx.x, blockIdx.y, smem_raw);
+  fk::plane_body_pruned<R, N, kThreads>(T, Vs, fa, blockIdx.x, blockIdx.y, smem_raw);
 }
+
+#ifdef CHEBFI_FFT_DF
+// The plane pass of the double-float path runs in 64-bit fixed point (16 bytes a point: the
+// 96-point plane fills an SM, whose one block then takes 24 warps; smaller planes run in
+// smaller blocks so that several share an SM and fill each other's barriers).
+template <int N> constexpr int fx_threads() { return N >= 96 ? 768 : N >= 48 ? 256 : 128; }
+template <int N>
+__global__ void __launch_bounds__(fx_threads<N>()) k_plane_fx(cdf* __restrict__ T, const int2* __restrict__ Vs, int ve,
+                                                              FastArgs fa) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fx::plane_body<N, fx_threads<N>()>(T, Vs, ve, fa, blockIdx.x, blockIdx.y, smem_raw);
+}
+#endif
 
 template <typename R, int N3>
 __global__ void __launch_bounds__(kThreads) k_zfwd_f(const cplx<R>* __restrict__ T, FastArgs fa,
@@ -54,7 +63,6 @@ template <typename R> void set_smem(const void* f, size_t bytes) {
 template <typename R> const R* vtable(const chebfi_ctx* c);
 template <> const float* vtable<float>(const chebfi_ctx* c) { return c->d_vsf.p; }
 template <> const double* vtable<double>(const chebfi_ctx* c) { return c->d_vs.p; }
-template <> const dfl* vtable<dfl>(const chebfi_ctx* c) { return reinterpret_cast<const dfl*>(c->d_vsdf.p); }
 
 template <typename R, int N>
 void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t ldy, int64_t nb, cplx<R>* T,
@@ -81,11 +89,15 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
   CHEBFI_REQUIRE(s.nxa >= 1 && s.nact >= 1, CHEBFI_ERR_STATE, "sphere without columns");
   CHEBFI_REQUIRE(s.pitch == fk::plane_pitch(N), CHEBFI_ERR_STATE, "plane pitch of the compile-time path");
   const cplx<R>* tw = nullptr;  // the passes read their twiddles from constant tables
-  const R* Vs = vtable<R>(ctx);
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
   const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
   fk::init_twiddles();
+#ifdef CHEBFI_FFT_DF
+  fx::init_twiddles();
+  set_smem<R>((const void*)k_plane_fx<N>, pbytes);
+#else
   set_smem<R>((const void*)k_plane_f<R, N>, pbytes);
+#endif
   set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
   set_smem<R>((const void*)k_zfwd_f<R, N>, zbytes);
   for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
@@ -93,8 +105,12 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
     dim3 gz((s.ncol + kCBF - 1) / kCBF, nbc);
     const double esz = sizeof(cplx<R>), col = (double)N * s.ncol * nbc * esz, sph = (double)ctx->npw * nbc * esz;
     CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
+#ifdef CHEBFI_FFT_DF
     CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col,
-                    k_plane_f<R, N><<<dim3(N, nbc), PlaneThreads<R>::v, pbytes, st>>>(T, Vs, fa, tw));
+                    k_plane_fx<N><<<dim3(N, nbc), fx_threads<N>(), pbytes, st>>>(T, ctx->d_vsfx.p, ctx->v_exp, fa));
+#else
+    CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col, k_plane_f<R, N><<<dim3(N, nbc), kThreads, pbytes, st>>>(T, vtable<R>(ctx), fa));
+#endif
     LocalEpi<S> e = ep;
     e.Y = ep.Y + b0 * ep.ldy;
     if (e.Z) e.Z = ep.Z + b0 * ep.ldz;

@@ -138,3 +138,55 @@ def test_apply_h_on_every_grid_length(n):
     # the parity tolerances of the FP64 and FP32 forms
     assert np.abs(_np(g.apply_H(_F(cell.Y0), prec=0)) - ref).max() <= 1e-11 * scale
     assert np.abs(_np(g.apply_H(_F(cell.Y0), prec=1)) - ref).max() <= 2e-5 * scale
+
+
+# the fixed-point plane pass of the FP64 form: potentials and blocks at the ends of its scales
+# (a band's planes are scaled by their own sums, the product with V_loc by its own maximum)
+@pytest.mark.parametrize("n", [24, 32, 48, 64, 72, 96])
+@pytest.mark.parametrize("kind", ["plain", "tiny", "huge", "spike", "zero", "core"])
+def test_fixed_point_planes_at_every_scale(n, kind):
+    L = 0.42 * n
+    ecut = 0.5 * (2.0 * np.pi / L * 0.23 * n) ** 2
+    cell = make_cell(L, n, ecut, 1, 8, 6, False, 36, kpt=(0.02, -0.05, 0.03))
+    cell.D = np.zeros_like(cell.D)
+    V = cell.vloc
+    if kind == "tiny":
+        V = V * 1e-12
+    elif kind == "huge":
+        V = V * 1e9
+    elif kind == "zero":
+        V = np.zeros_like(V)
+    elif kind == "spike":
+        V = np.zeros_like(V)
+        V[n // 3, n // 5, n // 2] = -7.0
+    elif kind == "core":  # a hard core beside an ordinary potential
+        V = V.copy()
+        V[1, 2, 3] = 1e6
+    cell.vloc = V
+    Y = cell.Y0.copy()
+    Y[:, 1] *= 1e18
+    Y[:, 2] *= 1e-18
+    Y[:, 3] = 0.0
+    Y[:, 4] = 0.0
+    Y[cell.npw // 2, 4] = 1.0  # one plane wave: every plane's sum is its one column's value
+    Y[:, 5] = 1.0              # all in phase: the sum is attained at the origin
+    op = PWOperator.from_cell(cell)
+    ref = op.apply_H(Y)
+    got = _np(_ctx(cell).apply_H(_F(Y)))
+    # H y = K y + V y: the double-float z passes round 2^-44 of a line's norm, the planes less
+    norm = np.linalg.norm(Y, axis=0)
+    tol = 2.0 ** -43 * (np.abs(V).max() + ecut) * norm
+    assert np.all(np.linalg.norm(got - ref, axis=0) <= tol)
+    assert np.all(got[:, 3] == 0.0)
+
+
+def test_fixed_point_planes_keep_non_finite_bands_apart():
+    cell = make_cell(10.0, 24, 6.0, 1, 8, 4, False, 37)
+    Y = cell.Y0.copy()
+    Y[5, 1] = np.nan
+    Y[7, 2] = np.inf
+    g = _ctx(cell)
+    got = _np(g.apply_H(_F(Y)))
+    good = _np(g.apply_H(_F(cell.Y0)))
+    assert np.isnan(got[:, 1]).all() and np.isnan(got[:, 2]).all()
+    assert np.array_equal(got[:, [0, 3]], good[:, [0, 3]])
