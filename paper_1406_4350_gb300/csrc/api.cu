@@ -1352,8 +1352,6 @@ int chebfi_set_sphere(chebfi_ctx* ctx, int64_t npw, const int32_t* miller) {
   s.col_off.upload(col_off.data(), col_off.size());
   s.rows_act.upload(rows.data(), rows.size());
   s.pw_z.upload(pw_znat.data(), npw);
-  s.col_off_nat.upload(col_nat.data(), col_nat.size());
-  s.rows_nat.upload(rows_nat.data(), rows_nat.size());
   ctx->sorted_to_user = order;
   ctx->d_sorted_to_user.upload(order.data(), npw);
   // kinetic diagonal |k + G|^2 / 2 (Section 2.1), sorted order

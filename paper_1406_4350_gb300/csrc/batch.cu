@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "fft_fast_kernels.cuh"
+#include "gemm_tile.cuh"
 #include "internal.cuh"
 #include "kernels.cuh"
 
@@ -87,12 +88,12 @@ __global__ void __launch_bounds__(kT) k_bzinv(const KDesc<R>* __restrict__ ks, c
 
 template <typename R, int N>
 __global__ void __launch_bounds__(kT) k_bplane(const KDesc<R>* __restrict__ ks, int64_t nb, cplx<R>* __restrict__ T,
-                                               const R* __restrict__ Vs, const cplx<R>* __restrict__ tw) {
+                                               const R* __restrict__ Vs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int64_t kb = blockIdx.y, k = kb / nb, b = kb - k * nb;
   const KDesc<R>& d = ks[k];
   const FastArgs fa = d.fa;
-  fk::plane_body<R, N>(T + d.t_off, Vs, fa, tw, blockIdx.x, b, smem_raw);
+  fk::plane_body_pruned<R, N, kT>(T + d.t_off, Vs, fa, blockIdx.x, b, smem_raw);
 }
 
 // z pass back with the Chebyshev epilogue of step `first` (0: later steps, 1: the first):
@@ -193,34 +194,30 @@ __device__ __forceinline__ Prob<R> make_prob(const KDesc<R>& d, int op, int firs
 }
 
 // Persistent CTAs take (k, tile) items from the queue until it is empty.  Tile BM x BN with
-// BM = 16 TM, BN = 16 TN; 256 threads, TM x TN complex outputs per thread.  CA: op(A) = A^H.
-// The K loop is double-buffered: the next BKb-deep slices of A and B are fetched into
-// registers while the current ones are multiplied from shared memory (one barrier per slice).
+// BM = 16 TM, BN = 16 TN (gemm_tile.cuh).  CA: op(A) = A^H.
 // With nsplit > 1 (the P^H Z class, whose inner dimension is a whole sphere) an item is
 // (k, tile * nsplit + chunk): it sums one K-chunk into its own slice of ws, and
 // k_bsplit_reduce adds the slices in chunk order (deterministic).
-constexpr int BKb = 16;
-
 template <typename R, int TM, int TN>
 constexpr size_t bgemm_smem() {
-  return (size_t)2 * BKb * (16 * TM + 1 + 16 * TN + 1) * sizeof(cplx<R>);
+  return gt::smem_bytes<R, TM, TN>();
+}
+
+// resident blocks per SM that the FP32 shapes are compiled for (FP64 is bound by its units)
+template <typename R, int TM, int TN> constexpr int bgemm_blocks() {
+  return sizeof(R) == 8 || TM * TN > 16 ? 1 : TM * TN == 16 ? 3 : 4;
 }
 
 template <typename R, int TM, int TN, bool CA>
-__global__ void __launch_bounds__(256) k_bgemm(const KDesc<R>* __restrict__ ks, int op, int first, int64_t nq,
+__global__ void __launch_bounds__(256, bgemm_blocks<R, TM, TN>()) k_bgemm(const KDesc<R>* __restrict__ ks, int op, int first, int64_t nq,
                                                int64_t nb, const int2* __restrict__ items, int nitems,
                                                int* __restrict__ counter, const cplx<R>* Bb, cplx<R>* Cb,
                                                int nsplit, cplx<R>* __restrict__ ws) {
   using C = cplx<R>;
   constexpr int BM = 16 * TM, BN = 16 * TN;
-  constexpr int LA = BM * BKb / 256, LB = BN * BKb / 256;
-  static_assert(LA * 256 == BM * BKb && LB * 256 == BN * BKb, "tile slices must split evenly over 256 threads");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* As = reinterpret_cast<C*>(smem_raw);  // [2][BKb][BM + 1]
-  C* Bs = As + 2 * BKb * (BM + 1);         // [2][BKb][BN + 1]
   __shared__ int s_item;
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const C zero = cmake<C>(0.0, 0.0);
   for (;;) {
     if (tid == 0) s_item = atomicAdd(counter, 1);
     __syncthreads();
@@ -232,7 +229,7 @@ __global__ void __launch_bounds__(256) k_bgemm(const KDesc<R>* __restrict__ ks, 
     const int tile = it.y / nsplit, chunk = it.y - tile * nsplit;
     int64_t klo = 0, khi = p.K;
     if (nsplit > 1) {
-      const int64_t kc = ((p.K + nsplit - 1) / nsplit + BKb - 1) / BKb * BKb;
+      const int64_t kc = ((p.K + nsplit - 1) / nsplit + gt::BK - 1) / gt::BK * gt::BK;
       klo = min(p.K, (int64_t)chunk * kc);
       khi = min(p.K, klo + kc);
       p.C = ws + ((int64_t)it.x * nsplit + chunk) * p.M * p.N;
@@ -243,89 +240,14 @@ __global__ void __launch_bounds__(256) k_bgemm(const KDesc<R>* __restrict__ ks, 
     const int64_t tm = (p.M + BM - 1) / BM;
     const int64_t i0 = (int64_t)(tile % tm) * BM, j0 = (int64_t)(tile / tm) * BN;
     R accr[TM][TN], acci[TM][TN];
-#pragma unroll
-    for (int a = 0; a < TM; ++a)
-#pragma unroll
-      for (int b = 0; b < TN; ++b) accr[a][b] = acci[a][b] = (R)0;
-    C ra[LA], rb[LB];
-    auto fetch = [&](int64_t k0) {
-#pragma unroll
-      for (int l = 0; l < LA; ++l) {
-        const int e = l * 256 + tid;
-        int i, k;
-        if (!CA) { i = e % BM; k = e / BM; } else { k = e % BKb; i = e / BKb; }
-        const int64_t gi = i0 + i, gk = k0 + k;
-        C v = zero;
-        if (gi < p.M && gk < khi) {
-          v = CA ? p.A[gk + gi * p.lda] : p.A[gi + gk * p.lda];
-          if (CA) v.y = -v.y;
-        }
-        ra[l] = v;
-      }
-#pragma unroll
-      for (int l = 0; l < LB; ++l) {
-        const int e = l * 256 + tid;
-        const int k = e % BKb, j = e / BKb;
-        const int64_t gj = j0 + j, gk = k0 + k;
-        rb[l] = (gj < p.N && gk < khi) ? p.B[gk + gj * p.ldb] : zero;
-      }
-    };
-    auto stash = [&](int buf) {
-      C* as = As + buf * BKb * (BM + 1);
-      C* bs = Bs + buf * BKb * (BN + 1);
-#pragma unroll
-      for (int l = 0; l < LA; ++l) {
-        const int e = l * 256 + tid;
-        int i, k;
-        if (!CA) { i = e % BM; k = e / BM; } else { k = e % BKb; i = e / BKb; }
-        as[k * (BM + 1) + i] = ra[l];
-      }
-#pragma unroll
-      for (int l = 0; l < LB; ++l) {
-        const int e = l * 256 + tid;
-        const int k = e % BKb, j = e / BKb;
-        bs[k * (BN + 1) + j] = rb[l];
-      }
-    };
-    if (klo < khi) {
-      fetch(klo);
-      stash(0);
-    }
-    __syncthreads();
-    int buf = 0;
-    for (int64_t k0 = klo; k0 < khi; k0 += BKb) {
-      const bool more = k0 + BKb < khi;
-      if (more) fetch(k0 + BKb);  // in flight while the current slice is multiplied
-      const C* as = As + buf * BKb * (BM + 1);
-      const C* bs = Bs + buf * BKb * (BN + 1);
-#pragma unroll
-      for (int k = 0; k < BKb; ++k) {
-        C av[TM], bv[TN];
-#pragma unroll
-        for (int a = 0; a < TM; ++a) av[a] = as[k * (BM + 1) + tx + 16 * a];
-#pragma unroll
-        for (int b = 0; b < TN; ++b) bv[b] = bs[k * (BN + 1) + ty + 16 * b];
-#pragma unroll
-        for (int a = 0; a < TM; ++a)
-#pragma unroll
-          for (int b = 0; b < TN; ++b) {
-            accr[a][b] = fma(av[a].x, bv[b].x, accr[a][b]);
-            accr[a][b] = fma(-av[a].y, bv[b].y, accr[a][b]);
-            acci[a][b] = fma(av[a].x, bv[b].y, acci[a][b]);
-            acci[a][b] = fma(av[a].y, bv[b].x, acci[a][b]);
-          }
-      }
-      if (more) stash(buf ^ 1);  // that buffer was last read before the previous barrier
-      __syncthreads();
-      buf ^= 1;
-    }
+    gt::tile<R, TM, TN, CA, false>(p.A, p.lda, p.B, p.ldb, p.M, p.N, i0, j0, klo, khi, smem_raw, accr, acci);
 #pragma unroll
     for (int b = 0; b < TN; ++b) {
-      const int64_t gj = j0 + ty + 16 * b;
+      const int64_t gj = j0 + TN * ty + b;
       if (gj >= p.N) continue;
 #pragma unroll
       for (int a = 0; a < TM; ++a) {
-        const int64_t gi = i0 + tx + 16 * a;
+        const int64_t gi = i0 + gt::row_of<R>(tx, a);
         if (gi >= p.M) continue;
         C r;
         r.x = p.alpha * accr[a][b];
@@ -482,23 +404,6 @@ template <> struct BatchOps<float> {
   static const float2* tw(chebfi_ctx* c) { return c->ax[0].tw32.p; }
 };
 
-FastArgs fast_args(const chebfi_ctx* c) {
-  const SphereFFT& s = c->sph;
-  FastArgs fa;
-  fa.ncol = s.ncol;
-  fa.nxa = s.nxa;
-  fa.pitch = s.pitch;
-  fa.zpitch = s.zpitch;
-  fa.ncolp = (s.ncol + 15) / 16 * 16;
-  fa.ldt = (int64_t)c->grid[2] * fa.ncolp;
-  fa.col_start = s.col_start.p;
-  fa.pw_line = s.pw_line.p;
-  fa.pw_z = s.pw_z.p;
-  fa.col_off = s.col_off_nat.p;
-  fa.row_off = s.rows_nat.p;
-  return fa;
-}
-
 // (k, tile[, chunk]) items of a GEMM class for tile shape `shape` and split factor
 // `nsplit`, longest problems first
 void build_items(chebfi_batch* bt, int gc, int shape, int nsplit) {
@@ -579,7 +484,7 @@ void blocal(chebfi_batch* bt, const cplx<R>* cur, cplx<R>* Z, cplx<R>* prev, int
   cplx<R>* T = BatchOps<R>::T(bt).p;
   const dim3 gz((unsigned)bt->ncb, (unsigned)bt->nb);
   CHEBFI_LAUNCH("k_bzinv", st, (k_bzinv<R, N><<<gz, kT, zbytes, st>>>(d, cur, T, tw, bt->cb_k.p, bt->cb_c0.p)));
-  CHEBFI_LAUNCH("k_bplane", st, (k_bplane<R, N><<<dim3(N, (unsigned)(bt->nk * bt->nb)), kT, pbytes, st>>>(d, bt->nb, T, BatchOps<R>::Vs(c0), tw)));
+  CHEBFI_LAUNCH("k_bplane", st, (k_bplane<R, N><<<dim3(N, (unsigned)(bt->nk * bt->nb)), kT, pbytes, st>>>(d, bt->nb, T, BatchOps<R>::Vs(c0))));
   CHEBFI_LAUNCH("k_bzfwd", st, (k_bzfwd<R, N><<<gz, kT, zbytes, st>>>(d, T, tw, bt->cb_k.p, bt->cb_c0.p, cur, Z, prev, first)));
 }
 
@@ -1077,7 +982,7 @@ int chebfi_batch_create(chebfi_batch** out, chebfi_ctx* const* kctx, int nk, int
       chebfi_ctx* c = kctx[k];
       KDesc<double>& a = bt->h64[k];
       KDesc<float>& b = bt->h32[k];
-      a.fa = b.fa = fast_args(c);
+      a.fa = b.fa = fk::fast_args(c);
       a.K = BatchOps<double>::K(c);
       b.K = BatchOps<float>::K(c);
       a.P = BatchOps<double>::P(c);

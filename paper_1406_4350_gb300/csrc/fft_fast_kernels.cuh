@@ -27,17 +27,35 @@ constexpr int kCBF = 32;  // columns per z-pass block
 static_assert(kThreadsF % kCBF == 0, "z-pass blocks are whole groups of kCBF threads");
 
 struct FastArgs {
-  int ncol, nxa, pitch, zpitch, ncolp;
+  int ncol, zpitch, ncolp;
   int64_t ldt;
   const int32_t* col_start;
   const int32_t* pw_line;
-  const int32_t* pw_z;      // natural z of each sorted sphere point
-  const int32_t* col_off;   // slot(x) * pitch + y of each column (plane rows cyclically shifted)
-  const int32_t* row_off;   // slot(x) * pitch of each active x
-  const int32_t* row_col = nullptr;            // (row act_lo + a, natural y) -> column, or -1
-  int act_lo = 0, nact = 0;                    // slot range of the pruned plane pass
-  unsigned nl_magic = 0;                       // t / nact == umulhi(t, nl_magic) for t < 2^16
+  const int32_t* pw_z;     // natural z of each sorted sphere point
+  const int32_t* row_col;  // (row act_lo + a, natural y) -> column, or -1
+  int act_lo, nact;        // slot range of the rows that hold columns
+  unsigned nl_magic;       // t / nact == umulhi(t, nl_magic) for t < 2^16
 };
+
+// the arguments of a context's compiled grid
+inline FastArgs fast_args(const chebfi_ctx* ctx) {
+  const SphereFFT& s = ctx->sph;
+  FastArgs fa;
+  fa.ncol = s.ncol;
+  fa.zpitch = s.zpitch;
+  fa.ncolp = (s.ncol + 15) / 16 * 16;
+  fa.ldt = (int64_t)s.n3 * fa.ncolp;
+  fa.col_start = s.col_start.p;
+  fa.pw_line = s.pw_line.p;
+  fa.pw_z = s.pw_z.p;
+  fa.row_col = s.row_col.p;
+  fa.act_lo = s.act_lo;
+  fa.nact = s.nact;
+  // ceil(2^32 / nact): exact quotients t / nact for t < 2^32 / nact (the row passes use t < 2^12)
+  fa.nl_magic = s.nact > 1 ? (unsigned)(((1ull << 32) + s.nact - 1) / (unsigned long long)s.nact) : 0u;
+  CHEBFI_REQUIRE(s.nxa >= 1 && s.nact >= 1, CHEBFI_ERR_STATE, "sphere without columns");
+  return fa;
+}
 
 // Twiddle tables tw[e] = exp(-2 pi i e / N) of the compiled line lengths, in constant memory:
 // a warp of a pass reads one entry (two where it straddles two sub-transforms), which the
@@ -129,67 +147,15 @@ __device__ __forceinline__ void zinv_body(const cplx<typename SphT<R>::type>* __
       t[(int64_t)z * fa.ncolp + l] = lines[l * fa.zpitch + z];
 }
 
-// plane z of block b: inverse y and x transforms, multiply by V_loc, forward x and y
-template <typename R, int N>
-__device__ __forceinline__ void plane_body(cplx<R>* __restrict__ T, const R* __restrict__ Vs, const FastArgs& fa,
-                                           const cplx<R>* __restrict__ twxy, int z, int64_t b,
-                                           unsigned char* smem_raw) {
-  (void)twxy;
-  const ConstTw<R, N> tw;
-  cplx<R>* plane = reinterpret_cast<cplx<R>*>(smem_raw);
-  const cplx<R> zero = cmake<cplx<R>>(0.0, 0.0);
-  for (int i = threadIdx.x; i < N * fa.pitch; i += blockDim.x) plane[i] = zero;
-  __syncthreads();
-  cplx<R>* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
-  for (int c = threadIdx.x; c < fa.ncol; c += blockDim.x) plane[fa.col_off[c]] = t[c];
-  __syncthreads();
-  LineMap rows;
-  rows.off = fa.row_off;
-  LineMap cols;
-  cols.stride = 1;
-  fast::lines_F<N, +1>(plane, fa.nxa, rows, 1, tw);       // along y on the rows that hold columns
-  // along x on every y: F's pass A; then, per contiguous group, F's pass B, the multiply by
-  // V_loc and G's pass B in registers; then G's pass A
-  fast::F_passA<N, +1>(plane, N, cols, fa.pitch, tw, threadIdx.x, blockDim.x);
-  __syncthreads();
-  {
-    constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB;
-    const R* v = Vs + (int64_t)z * N * N;
-    for (int it = threadIdx.x; it < N * NA; it += blockDim.x) {
-      const int ka = it / N, yy = it - ka * N;
-      cplx<R>* a = plane + yy + NB * ka * fa.pitch;
-      const R* vv = v + (NB * ka) * N + yy;
-      cplx<R> u[NB];
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb) u[nb] = a[nb * fa.pitch];
-      fast::dft<NB, +1>(u);
-#pragma unroll
-      for (int kb = 0; kb < NB; ++kb) {
-        const R s = vv[kb * N];
-        u[kb] = cscale(u[kb], s);
-      }
-      fast::dft<NB, -1>(u);
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb)
-        a[nb * fa.pitch] = (ka == 0 || nb == 0) ? u[nb] : u[nb] * fast::twN<-1>(tw, nb * ka);
-    }
-  }
-  __syncthreads();
-  fast::G_passA<N, -1>(plane, N, cols, fa.pitch, threadIdx.x, blockDim.x);
-  __syncthreads();
-  fast::lines_G<N, -1>(plane, fa.nxa, rows, 1, tw);       // along y on the needed rows
-  for (int c = threadIdx.x; c < fa.ncol; c += blockDim.x) t[c] = plane[fa.col_off[c]];
-}
-
 // rows of a plane are an odd pitch apart: the row-wise passes meet no bank conflicts
 constexpr int plane_pitch(int n) { return n % 2 ? n : n + 1; }
 
-// The plane pass of plane_body with its zero rows pruned and its scatter / gather fused:
+// Plane z of block b: inverse y and x transforms, multiply by V_loc, forward x and y, its
+// zero rows pruned and its scatter / gather fused:
 // the first y pass reads the sphere columns straight from the column buffer (no zeroed
 // plane, no scatter), the x passes skip the loads of rows outside the active slot range
 // [act_lo, act_lo + nact) (they are zero) and the stores of rows no later pass reads, and
-// the last y pass stores the columns straight to the column buffer (no gather).  Same
-// arithmetic, in the same order.  The row pitch is the compile-time plane_pitch(N), so every shared-memory offset of a pass is an
+// the last y pass stores the columns straight to the column buffer (no gather).    The row pitch is the compile-time plane_pitch(N), so every shared-memory offset of a pass is an
 // immediate; where the block's NT / 32 warps are a multiple of NB (N = 64, 96) each warp of
 // an x pass keeps one nb and its twiddles in registers.
 template <typename R, int N, int NT = kThreadsF>

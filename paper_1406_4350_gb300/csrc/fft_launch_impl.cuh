@@ -69,24 +69,7 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
                  LocalEpi<typename SphT<R>::type> ep, cudaStream_t st, const typename SphT<R>::type* K) {
   using S = typename SphT<R>::type;
   const SphereFFT& s = ctx->sph;
-  FastArgs fa;
-  fa.ncol = s.ncol;
-  fa.nxa = s.nxa;
-  fa.pitch = s.pitch;
-  fa.zpitch = s.zpitch;
-  fa.ncolp = (s.ncol + 15) / 16 * 16;
-  fa.ldt = (int64_t)N * fa.ncolp;
-  fa.col_start = s.col_start.p;
-  fa.pw_line = s.pw_line.p;
-  fa.pw_z = s.pw_z.p;
-  fa.col_off = s.col_off_nat.p;
-  fa.row_off = s.rows_nat.p;
-  fa.row_col = s.row_col.p;
-  fa.act_lo = s.act_lo;
-  fa.nact = s.nact;
-  // ceil(2^32 / nact): exact quotients t / nact for t < 2^32 / nact (the row passes use t < 2^12)
-  fa.nl_magic = s.nact > 1 ? (unsigned)(((1ull << 32) + s.nact - 1) / (unsigned long long)s.nact) : 0u;
-  CHEBFI_REQUIRE(s.nxa >= 1 && s.nact >= 1, CHEBFI_ERR_STATE, "sphere without columns");
+  const FastArgs fa = fk::fast_args(ctx);
   CHEBFI_REQUIRE(s.pitch == fk::plane_pitch(N), CHEBFI_ERR_STATE, "plane pitch of the compile-time path");
   const cplx<R>* tw = nullptr;  // the passes read their twiddles from constant tables
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);

@@ -3,17 +3,16 @@
 // Used for the FP64 and FP32 forms of the projector products P^H psi and P W
 // (Algorithm 1, Section 5.1), the Woodbury core products, and the subspace matrices and
 // rotations of Algorithm 2.  FP32: 64 x 64 output tiles, 256 threads, 4 x 4 complex outputs
-// per thread.  FP64: 256 outputs per tile, one per thread (k_gemm_d).  Both split K, with a
+// per thread (gemm_tile.cuh).  FP64: 256 outputs per tile, one per thread (k_gemm_d).  Both split K, with a
 // deterministic second pass, when the output has too few tiles to fill the 152 SMs.
 #include <algorithm>
 
+#include "gemm_tile.cuh"
 #include "internal.cuh"
 #include "kernels.cuh"
 
 namespace chebfi {
 namespace {
-
-constexpr int BM = 64, BN = 64, BK = 8;
 
 template <typename C> __device__ __forceinline__ C ld_op(const C* p, bool conj_) {
   C v = *p;
@@ -21,86 +20,39 @@ template <typename C> __device__ __forceinline__ C ld_op(const C* p, bool conj_)
   return v;
 }
 
-template <typename R, bool CA, bool CB>
-__global__ void __launch_bounds__(256) k_gemm(int64_t M, int64_t N, int64_t K, R alpha, const cplx<R>* __restrict__ A,
-                                              int64_t lda, const cplx<R>* __restrict__ B, int64_t ldb, R beta,
-                                              cplx<R>* __restrict__ Cm, int64_t ldc, int64_t kchunk,
-                                              cplx<R>* __restrict__ ws, int lower, int n_fastest) {
-  using C = cplx<R>;
-  // n_fastest: blockIdx.x walks the column tiles, so CTAs launched together share a row
-  // tile of A (the large operand when M >> N) in L2
-  const int64_t tile_i = n_fastest ? blockIdx.y : blockIdx.x, tile_j = n_fastest ? blockIdx.x : blockIdx.y;
-  if (lower && tile_i < tile_j) return;  // tile strictly above the diagonal
-  __shared__ C As[BK][BM + 1];
-  __shared__ C Bs[BK][BN + 1];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int64_t i0 = tile_i * BM, j0 = tile_j * BN;
-  const int64_t kbeg = (int64_t)blockIdx.z * kchunk;
-  const int64_t kend = min(K, kbeg + kchunk);
-  R accr[4][4], acci[4][4];
+// FP32: one tile of gemm_tile.cuh per block, blockIdx.z the K range.  Shapes with few tiles
+// split K down to 64 products so that every SM gets blocks.  256 x 256 x 8217: 238 us with an
+// unbuffered loop and ranges of 1024, now 106 us; 256^3: 52 us on 16 SMs, now 10 us.
+template <int TM, int TN, bool CA, bool CB>
+__global__ void __launch_bounds__(256, TN == 4 ? 3 : 4)
+    k_gemm_f(int64_t M, int64_t N, int64_t K, float alpha, const float2* __restrict__ A, int64_t lda,
+             const float2* __restrict__ B, int64_t ldb, float beta, float2* __restrict__ Cm, int64_t ldc, int64_t kchunk,
+             float2* __restrict__ ws, int lower, int tiles_m, int tiles_n, int n_fastest) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int BM = 16 * TM, BN = 16 * TN;
+  // n_fastest: consecutive blocks walk the column tiles, so blocks launched together share a
+  // row tile of A (the large operand when M >> N) in L2
+  const int64_t tile_i = n_fastest ? blockIdx.x / tiles_n : blockIdx.x % tiles_m;
+  const int64_t tile_j = n_fastest ? blockIdx.x % tiles_n : blockIdx.x / tiles_m;
+  const int64_t i0 = tile_i * BM, j0 = tile_j * BN, kbeg = (int64_t)blockIdx.z * kchunk;
+  if (lower && i0 + BM - 1 < j0) return;  // tile strictly above the diagonal
+  float accr[TM][TN], acci[TM][TN];
+  gt::tile<float, TM, TN, CA, CB>(A, lda, B, ldb, M, N, i0, j0, kbeg, min(K, kbeg + kchunk), smem_raw, accr, acci);
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) accr[a][b] = acci[a][b] = (R)0;
-  const C zero = cmake<C>(0.0, 0.0);
-  for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
-#pragma unroll
-    for (int e0 = 0; e0 < BM * BK; e0 += 256) {
-      const int e = e0 + tid;
-      int i, k;
-      if (!CA) { i = e % BM; k = e / BM; } else { k = e % BK; i = e / BK; }
-      const int64_t gi = i0 + i, gk = k0 + k;
-      C v = zero;
-      if (gi < M && gk < kend) v = CA ? ld_op(A + gk + gi * lda, true) : A[gi + gk * lda];
-      As[k][i] = v;
-    }
-#pragma unroll
-    for (int e0 = 0; e0 < BN * BK; e0 += 256) {
-      const int e = e0 + tid;
-      int j, k;
-      if (!CB) { k = e % BK; j = e / BK; } else { j = e % BN; k = e / BN; }
-      const int64_t gj = j0 + j, gk = k0 + k;
-      C v = zero;
-      if (gj < N && gk < kend) v = CB ? ld_op(B + gj + gk * ldb, true) : B[gk + gj * ldb];
-      Bs[k][j] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < BK; ++k) {
-      C av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[k][tx + 16 * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[k][ty + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          accr[a][b] = fma(av[a].x, bv[b].x, accr[a][b]);
-          accr[a][b] = fma(-av[a].y, bv[b].y, accr[a][b]);
-          acci[a][b] = fma(av[a].x, bv[b].y, acci[a][b]);
-          acci[a][b] = fma(av[a].y, bv[b].x, acci[a][b]);
-        }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int64_t gj = j0 + ty + 16 * b;
+  for (int b = 0; b < TN; ++b) {
+    const int64_t gj = j0 + TN * ty + b;
     if (gj >= N) continue;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int64_t gi = i0 + tx + 16 * a;
+    for (int a = 0; a < TM; ++a) {
+      const int64_t gi = i0 + gt::row_of<float>(tx, a);
       if (gi >= M) continue;
-      C r;
-      r.x = alpha * accr[a][b];
-      r.y = alpha * acci[a][b];
+      float2 r = make_float2(alpha * accr[a][b], alpha * acci[a][b]);
       if (ws) {
         ws[(int64_t)blockIdx.z * M * N + gi + gj * M] = r;
       } else {
-        if (beta != (R)0) {
-          const C c = Cm[gi + gj * ldc];
+        if (beta != 0.f) {
+          const float2 c = Cm[gi + gj * ldc];
           r.x = fma(beta, c.x, r.x);
           r.y = fma(beta, c.y, r.y);
         }
@@ -215,37 +167,47 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(int64_t M, int64_t N, int
   Cm[i + j * ldc] = r;
 }
 
-template <typename R, bool CA, bool CB>
-void launch(int64_t M, int64_t N, int64_t K, double alpha, const cplx<R>* A, int64_t lda, const cplx<R>* B,
-            int64_t ldb, double beta, cplx<R>* Cm, int64_t ldc, cudaStream_t st, DevBuf<cplx<R>>* ws,
-            const char* tag, bool lower) {
-  const int64_t tm = (M + BM - 1) / BM, tn = (N + BN - 1) / BN;
-  int splits = 1;
-  const int64_t tiles = tm * tn;
-  if (ws && tiles < 304 && K >= 2048) {
-    splits = (int)std::min<int64_t>((304 + tiles - 1) / tiles, K / 1024);
-    splits = std::max(1, std::min(splits, 64));
-  }
-  int64_t kchunk = (K + splits - 1) / splits;
-  kchunk = (kchunk + BK - 1) / BK * BK;
-  splits = (int)((K + kchunk - 1) / kchunk);
-  if (K == 0) { splits = 1; kchunk = BK; }
-
-  cplx<R>* wsp = nullptr;
+template <bool CA, bool CB>
+void launch_f(int64_t M, int64_t N, int64_t K, double alpha, const float2* A, int64_t lda, const float2* B, int64_t ldb,
+              double beta, float2* Cm, int64_t ldc, cudaStream_t st, DevBuf<float2>* ws, const char* tag, bool lower) {
+  // 64 x 64 tiles (three blocks per SM) or 64 x 32 ones (four, about 10 % slower per output):
+  // whichever leaves the shorter schedule; a shape with less than a round of tiles splits K
+  // into ranges of at least 64 until it fills one.  8217 x 256 x 256: 516 and 1032 tiles, 125
+  // us (a second round of 60 tiles) and 107 us.
+  const int64_t tm = (M + 63) / 64;
+  auto plan = [&](int64_t tn, int64_t per_round, int64_t& splits, int64_t& kchunk) {
+    const int64_t tiles = tm * tn;
+    splits = 1;
+    if (ws && tiles < per_round) splits = std::max<int64_t>(1, std::min<int64_t>({per_round / tiles, K / 64, 64}));
+    kchunk = std::max<int64_t>(gt::BK, ((K + splits - 1) / splits + gt::BK - 1) / gt::BK * gt::BK);
+    splits = std::max<int64_t>(1, (K + kchunk - 1) / kchunk);
+    return (double)((tiles * splits + per_round - 1) / per_round) * (double)kchunk;
+  };
+  constexpr int64_t kSMs = 152;
+  int64_t s4, c4, s2, c2;
+  const double cost4 = 3.0 * plan((N + 63) / 64, 3 * kSMs, s4, c4), cost2 = 4.0 * 0.5 * 1.1 * plan((N + 31) / 32, 4 * kSMs, s2, c2);
+  const bool narrow = cost2 < cost4;
+  const int64_t tn = narrow ? (N + 31) / 32 : (N + 63) / 64, tiles = tm * tn, splits = narrow ? s2 : s4, kchunk = narrow ? c2 : c4;
+  float2* wsp = nullptr;
   if (splits > 1) {
-    ws->alloc((size_t)splits * M * N);
+    ws->alloc((size_t)(splits * M * N));
     wsp = ws->p;
   }
-  const bool n_fastest = tm > 4 * tn;
-  CHEBFI_REQUIRE((n_fastest ? tm : tn) <= 65535, CHEBFI_ERR_ARG, "GEMM too large");
-  dim3 grid(n_fastest ? (unsigned)tn : (unsigned)tm, n_fastest ? (unsigned)tm : (unsigned)tn, (unsigned)splits);
-  const double tiles_done = lower ? (double)(tm * (tm + 1) / 2) / (double)(tm * tn) : 1.0;
-  CHEBFI_LAUNCH_W(tag, st, 8.0 * (double)M * (double)N * (double)K * tiles_done,
-                  k_gemm<R, CA, CB><<<grid, 256, 0, st>>>(M, N, K, (R)alpha, A, lda, B, ldb, (R)beta, Cm, ldc, kchunk,
-                                                          wsp, lower ? 1 : 0, n_fastest ? 1 : 0));
+  CHEBFI_REQUIRE(tiles < (1ll << 31), CHEBFI_ERR_ARG, "GEMM too large");
+  static_assert(gt::smem_bytes<float, 4, 4>() <= 48 * 1024, "within the default shared memory limit");
+  const double tiles_done = lower ? 0.5 * (1.0 + 1.0 / (double)tm) : 1.0;
+  auto go = [&](auto kernel, size_t smem) {
+    CHEBFI_LAUNCH_W(tag, st, 8.0 * (double)M * (double)N * (double)K * tiles_done,
+                    kernel<<<dim3((unsigned)tiles, 1, (unsigned)splits), 256, smem, st>>>(
+                        M, N, K, (float)alpha, A, lda, B, ldb, (float)beta, Cm, ldc, kchunk, wsp, lower ? 1 : 0, (int)tm,
+                        (int)tn, tm > 4 * tn ? 1 : 0));
+  };
+  if (narrow) go(k_gemm_f<4, 2, CA, CB>, gt::smem_bytes<float, 4, 2>());
+  else go(k_gemm_f<4, 4, CA, CB>, gt::smem_bytes<float, 4, 4>());
   if (splits > 1) {
     const int64_t tot = M * N;
-    CHEBFI_LAUNCH("k_splitk_reduce", st, k_splitk_reduce<R><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, splits, wsp, (R)beta, Cm, ldc));
+    CHEBFI_LAUNCH("k_splitk_reduce", st,
+                  k_splitk_reduce<float><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, (int)splits, wsp, (float)beta, Cm, ldc));
   }
 }
 
@@ -290,7 +252,7 @@ void launch_d(int64_t M, int64_t N, int64_t K, double alpha, const double2* A, i
 
 template <typename R, bool CA, bool CB, typename... Args> void route(Args... args) {
   if constexpr (sizeof(R) == 8) launch_d<CA, CB>(args...);
-  else launch<R, CA, CB>(args...);
+  else launch_f<CA, CB>(args...);
 }
 
 }  // namespace

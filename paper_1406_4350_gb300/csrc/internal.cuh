@@ -219,8 +219,6 @@ struct SphereFFT {
   DevBuf<int32_t> rows_act;    // active rows rev(x) of the plane (nxa)
   // natural-index maps of the compile-time-length path
   DevBuf<int32_t> pw_z;        // sorted sphere point -> z
-  DevBuf<int32_t> col_off_nat; // column -> slot(x) * pitch + y, slot(x) = (x + n1/2) mod n1
-  DevBuf<int32_t> rows_nat;    // slot(x) * pitch of the active rows, consecutive slots
   // the pruned plane pass works on the slot range [act_lo, act_lo + nact) that covers every
   // active row (for a sphere the active rows are that range)
   int act_lo = 0, nact = 0;
