@@ -207,21 +207,24 @@ __global__ void __launch_bounds__(kThreads) k_plane_real(const cplx<R>* __restri
   }
 }
 
-// gV[(x n2 + y) n3 + z] += scale * sum_b Re(conj(g_b(r)) psi_b(r)), r = (x, y, z); fixed band order.
+// gV[(x n2 + y) n3 + z] += scale * sum_b Re(conj(g_b(r)) psi_b(r)), r = (x, y, z); fixed band
+// order.  The values' positions p along each axis hold the index p / qb + qa (p mod qb) (the
+// compiled passes' split order; qa = 0, qb = 1: natural order).
 template <typename R>
 __global__ void k_density_accum(int n1, int n2, int n3, int64_t nbc, const cplx<R>* __restrict__ psi,
-                                const cplx<R>* __restrict__ g, double scale, double* __restrict__ gV) {
+                                const cplx<R>* __restrict__ g, double scale, int qa, int qb, double* __restrict__ gV) {
   const int64_t n = (int64_t)n1 * n2 * n3;
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   double acc = 0.0;
+#pragma unroll 4
   for (int64_t b = 0; b < nbc; ++b) {
     const cplx<R> u = psi[b * n + r], v = g[b * n + r];
     acc += (double)v.x * (double)u.x + (double)v.y * (double)u.y;
   }
   const int64_t plane = (int64_t)n1 * n2;
-  const int z = (int)(r / plane), rem = (int)(r - (int64_t)z * plane);
-  const int x = rem / n2, y = rem - x * n2;
+  const int pz = (int)(r / plane), rem = (int)(r - (int64_t)pz * plane), px = rem / n2, py = rem - px * n2;
+  const int x = px / qb + qa * (px % qb), y = py / qb + qa * (py % qb), z = pz / qb + qa * (pz % qb);
   gV[((int64_t)x * n2 + y) * n3 + z] += scale * acc;
 }
 
@@ -254,6 +257,28 @@ bool fast_fft_supported(int n1, int n2, int n3) {
   switch (n1) {
 #define CHEBFI_X(n) case n:
     CHEBFI_FFT_SIZES(CHEBFI_X)
+#undef CHEBFI_X
+    return true;
+    default: return false;
+  }
+}
+
+// the second factor of a compiled length: positions p < split_factor hold multiples of
+// split_index(n, 1)
+int split_factor(int n) {
+  switch (n) {
+#define CHEBFI_X(n) \
+  case n: return fast::Plan<n>::NB;
+    CHEBFI_FFT_SIZES(CHEBFI_X)
+#undef CHEBFI_X
+    default: return 1;
+  }
+}
+
+bool fixed_fft_size(int n) {
+  switch (n) {
+#define CHEBFI_X(n) case n:
+    CHEBFI_FFT_DF_SIZES(CHEBFI_X)
 #undef CHEBFI_X
     return true;
     default: return false;
@@ -331,6 +356,21 @@ void local_apply(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cpl
   }
 }
 
+// Real-space values of a chunk of bands by the compiled passes: FP64 blocks keep the z pass on
+// the FP64 units (a small part of the work) and take the fixed-point planes unless the FP64
+// units are asked for, at the sizes that have them (48^3, 128 bands: 0.94 ms on the FP64
+// units; the backward of a degree-8 filter there 49.4 -> 36.7 ms).
+template <typename R>
+bool real_space(chebfi_ctx* ctx, const cplx<R>* src, int64_t nb, cplx<R>* T, cplx<R>* out, cudaStream_t st) {
+  if constexpr (std::is_same<R, double>::value) {
+    const bool fixed = ctx->fft64 == CHEBFI_FFT64_DOUBLE_FLOAT && fixed_fft_size(ctx->grid[0]);
+    return fast_real_space<double>(ctx, src, ctx->npw, nb, T, out, !fixed, st) &&
+           (!fixed || fixed_planes_real(ctx, nb, T, out, st));
+  } else {
+    return fast_real_space<R>(ctx, src, ctx->npw, nb, T, out, true, st);
+  }
+}
+
 template <typename R>
 void vloc_gradient(chebfi_ctx* ctx, const cplx<R>* Ys, const cplx<R>* Gs, int64_t nb, double* gV, cudaStream_t st,
                    DevBuf<cplx<R>>& T, DevBuf<cplx<R>>& Rb, DevBuf<cplx<R>>& Gb, double scale, bool accumulate) {
@@ -373,16 +413,19 @@ void vloc_gradient(chebfi_ctx* ctx, const cplx<R>* Ys, const cplx<R>* Gs, int64_
   for (int64_t b0 = 0; b0 < nb; b0 += chunk) {
     const int nbc = (int)std::min<int64_t>(chunk, nb - b0);
     dim3 gz((s.ncol + kCB - 1) / kCB, nbc);
+    bool fast = false;
     for (int which = 0; which < 2; ++which) {
       const cplx<R>* src = (which == 0 ? Ys : Gs) + b0 * ctx->npw;
       cplx<R>* dst = which == 0 ? Rb.p : Gb.p;
+      if ((fast = ctx->fast_fft && real_space<R>(ctx, src, nbc, T.p, dst, st))) continue;
       CHEBFI_LAUNCH("k_zinv", st, k_zinv<R><<<gz, kThreads, zbytes, st>>>(src, ctx->npw, T.p, sa, pz));
       CHEBFI_LAUNCH("k_plane_real", st,
                     k_plane_real<R><<<dim3(n3, nbc), kThreads, pbytes, st>>>(T.p, pa, px, py, dst));
     }
     CHEBFI_LAUNCH("k_density_accum", st,
-                  k_density_accum<R><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n1, n2, n3, nbc, Rb.p, Gb.p,
-                                                                                    scale / (double)n, gV));
+                  k_density_accum<R><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
+                      n1, n2, n3, nbc, Rb.p, Gb.p, scale / (double)n, fast ? split_index(n1, 1) : 0,
+                      fast ? split_factor(n1) : 1, gV));
   }
 }
 

@@ -4,4 +4,5 @@
 namespace chebfi {
 template bool fast_dispatch<float>(chebfi_ctx*, const cplx<float>*, int64_t, int64_t, cplx<float>*, LocalEpi<float>, cudaStream_t,
                                 const float*);
+template bool fast_real_space<float>(chebfi_ctx*, const cplx<float>*, int64_t, int64_t, cplx<float>*, cplx<float>*, bool, cudaStream_t);
 }  // namespace chebfi

@@ -158,16 +158,15 @@ constexpr int plane_pitch(int n) { return n % 2 ? n : n + 1; }
 // the last y pass stores the columns straight to the column buffer (no gather).    The row pitch is the compile-time plane_pitch(N), so every shared-memory offset of a pass is an
 // immediate; where the block's NT / 32 warps are a multiple of NB (N = 64, 96) each warp of
 // an x pass keeps one nb and its twiddles in registers.
-template <typename R, int N, int NT = kThreadsF>
-__device__ __forceinline__ void plane_body_pruned(cplx<R>* __restrict__ T, const R* __restrict__ Vs,
-                                                  const FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
+//
+// inverse_passes: the inverse y transform and pass A of the inverse x transform.
+template <typename R, int N, int NT>
+__device__ __forceinline__ void inverse_passes(const cplx<R>* __restrict__ t, const FastArgs& fa, cplx<R>* plane) {
   using C = cplx<R>;
   constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N), W = NT / 32;
   constexpr bool kWarpNb = N % 32 == 0 && W % NB == 0;
   const ConstTw<R, N> tw;
-  C* plane = reinterpret_cast<C*>(smem_raw);
   const C zero = cmake<C>(0.0, 0.0);
-  C* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
   const int nl = fa.nact, lo = fa.act_lo;
   C* rows = plane + lo * P;  // row a of the active range
   // y, inverse: F's pass A on the active rows, its inputs read from the column buffer;
@@ -256,6 +255,20 @@ __device__ __forceinline__ void plane_body_pruned(cplx<R>* __restrict__ T, const
     }
   }
   __syncthreads();
+}
+
+template <typename R, int N, int NT = kThreadsF>
+__device__ __forceinline__ void plane_body_pruned(cplx<R>* __restrict__ T, const R* __restrict__ Vs,
+                                                  const FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
+  using C = cplx<R>;
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N), W = NT / 32;
+  constexpr bool kWarpNb = N % 32 == 0 && W % NB == 0;
+  const ConstTw<R, N> tw;
+  C* plane = reinterpret_cast<C*>(smem_raw);
+  C* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
+  const int nl = fa.nact, lo = fa.act_lo;
+  C* rows = plane + lo * P;  // row a of the active range
+  inverse_passes<R, N, NT>(t, fa, plane);
   {
     // F's pass B, the multiply by V_loc and G's pass B, in registers per contiguous group
     const R* v = Vs + (int64_t)z * N * N;
@@ -332,6 +345,28 @@ __device__ __forceinline__ void plane_body_pruned(cplx<R>* __restrict__ T, const
       const int c = __ldg(rc + NB * na);
       if (c >= 0) t[c] = v[na];
     }
+  }
+}
+
+// real-space values of plane z of block b, for the derivative with respect to V_loc:
+// out[x'][y'] in split order
+template <typename R, int N, int NT>
+__device__ __forceinline__ void plane_real_body(const cplx<R>* __restrict__ T, cplx<R>* __restrict__ out,
+                                                const FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
+  using C = cplx<R>;
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N);
+  C* plane = reinterpret_cast<C*>(smem_raw);
+  inverse_passes<R, N, NT>(T + b * fa.ldt + (int64_t)z * fa.ncolp, fa, plane);
+  for (int it = threadIdx.x; it < N * NA; it += NT) {
+    const int ka = it / N, yy = it - ka * N;
+    const C* a = plane + yy + NB * ka * P;
+    C u[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) u[q] = a[q * P];
+    fast::dft<NB, +1>(u);
+    C* o = out + (int64_t)(NB * ka) * N + yy;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) o[q * N] = u[q];
   }
 }
 

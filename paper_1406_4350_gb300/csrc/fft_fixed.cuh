@@ -264,49 +264,16 @@ __device__ __forceinline__ int norm_shift(unsigned m, int top) {
 }
 __device__ __forceinline__ cfx shl(cfx a, int s) { return cfx{a.x << s, a.y << s}; }
 
-// Plane z of band b (fk::plane_body_pruned in fixed point): inverse y and x transforms,
-// multiply by V_loc (Vs: (h, l) of V_loc / 2^ve in split order), forward x and y.  The column
-// buffer holds double-float pairs.  NT threads; the plane (16 bytes a point) fills the SM's
-// shared memory, so one block runs per SM at N = 96.
-template <int N, int NT>
-__device__ __forceinline__ void plane_body(cdf* __restrict__ T, const int2* __restrict__ Vs, int ve,
-                                           const fk::FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
+// The inverse y transform and pass A of the inverse x transform of a plane whose columns
+// load(c) gives as scaled integers: the plane then holds pass B's inputs at a quarter of
+// their value.  tws: the twiddles in shared memory (a warp of a y pass holds several nb, and
+// the constant cache serves one address per warp at a time; the x passes use constant memory).
+template <int N, int NT, typename Load>
+__device__ __forceinline__ void inverse_passes(Load load, const fk::FastArgs& fa, cfx* plane, const int4* tws) {
   constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = fk::plane_pitch(N);
-  __shared__ float red[NT / 32];
-  __shared__ unsigned ored[2];
-  // a warp of a y pass holds several nb: its twiddles come from shared memory (the constant
-  // cache serves one address per warp at a time), those of the x passes from constant memory
-  __shared__ int4 tws[N];
-  cfx* plane = reinterpret_cast<cfx*>(smem_raw);
-  cdf* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
   const int nl = fa.nact, lo = fa.act_lo, tid = threadIdx.x;
   cfx* rows = plane + lo * P;  // row a of the active range
   const cfx zero{0, 0};
-  // the scale: 2^s sum (|re| + |im|) <= 2^61 (summed 2^-13 down, against overflow)
-  int s;
-  {
-    float sum = 0.f;
-    for (int c = tid; c < fa.ncol; c += NT) {
-      const cdf v = t[c];
-      sum += (fabsf(v.x.h) + fabsf(v.y.h)) * 1.220703125e-4f;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (tid % 32 == 0) red[tid / 32] = sum;
-    if (tid < 2) ored[tid] = 0u;
-    for (int i = tid; i < N; i += NT) tws[i] = c_twfx[fk::TwOff<N>::v + i];
-    __syncthreads();
-    sum = 0.f;
-#pragma unroll
-    for (int i = 0; i < NT / 32; ++i) sum += red[i];
-    if (!(sum < INFINITY)) {  // Inf or NaN in the plane: so is every value of its transform
-      const float q = __int_as_float(0x7fc00000);
-      for (int c = tid; c < fa.ncol; c += NT) t[c] = cdf{dfl(q, q), dfl(q, q)};
-      return;
-    }
-    s = 61 - 13 - (sum > 0.f ? ilogbf(sum) + 1 : 0) - 1;  // one bit spare for the sum's rounding
-  }
-  const Pow2 in = pow2(s);
   // y, inverse, pass A on the active rows, its inputs read from the column buffer
   for (int it = tid; it < nl * NB; it += NT) {
     const int a = it / NB, nb = it - a * NB;
@@ -316,11 +283,7 @@ __device__ __forceinline__ void plane_body(cdf* __restrict__ T, const int2* __re
 #pragma unroll
     for (int na = 0; na < NA; ++na) {
       const int c = __ldg(rc + NB * na);
-      v[na] = zero;
-      if (c >= 0) {
-        const cdf u = t[c];
-        v[na] = cfx{to_fixed(u.x, in), to_fixed(u.y, in)};
-      }
+      v[na] = c >= 0 ? load(c) : zero;
     }
     dft<NA, +1>(v);
     row[0] = sar(v[0], 1);
@@ -359,6 +322,52 @@ __device__ __forceinline__ void plane_body(cdf* __restrict__ T, const int2* __re
     }
   }
   __syncthreads();
+}
+
+// Plane z of band b (fk::plane_body_pruned in fixed point): inverse y and x transforms,
+// multiply by V_loc (Vs: (h, l) of V_loc / 2^ve in split order), forward x and y.  The column
+// buffer holds double-float pairs.  NT threads; the plane (16 bytes a point) fills the SM's
+// shared memory, so one block runs per SM at N = 96.
+template <int N, int NT>
+__device__ __forceinline__ void plane_body(cdf* __restrict__ T, const int2* __restrict__ Vs, int ve,
+                                           const fk::FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = fk::plane_pitch(N);
+  __shared__ float red[NT / 32];
+  __shared__ unsigned ored[2];
+  __shared__ int4 tws[N];
+  cfx* plane = reinterpret_cast<cfx*>(smem_raw);
+  cdf* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
+  const int nl = fa.nact, lo = fa.act_lo, tid = threadIdx.x;
+  cfx* rows = plane + lo * P;  // row a of the active range
+  // the scale: 2^s sum (|re| + |im|) <= 2^61 (summed 2^-13 down, against overflow)
+  int s;
+  {
+    float sum = 0.f;
+    for (int c = tid; c < fa.ncol; c += NT) {
+      const cdf v = t[c];
+      sum += (fabsf(v.x.h) + fabsf(v.y.h)) * 1.220703125e-4f;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (tid % 32 == 0) red[tid / 32] = sum;
+    if (tid < 2) ored[tid] = 0u;
+    for (int i = tid; i < N; i += NT) tws[i] = c_twfx[fk::TwOff<N>::v + i];
+    __syncthreads();
+    sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) sum += red[i];
+    if (!(sum < INFINITY)) {  // Inf or NaN in the plane: so is every value of its transform
+      const float q = __int_as_float(0x7fc00000);
+      for (int c = tid; c < fa.ncol; c += NT) t[c] = cdf{dfl(q, q), dfl(q, q)};
+      return;
+    }
+    s = 61 - 13 - (sum > 0.f ? ilogbf(sum) + 1 : 0) - 1;  // one bit spare for the sum's rounding
+  }
+  const Pow2 in = pow2(s);
+  inverse_passes<N, NT>([&](int c) {
+    const cdf u = t[c];
+    return cfx{to_fixed(u.x, in), to_fixed(u.y, in)};
+  }, fa, plane, tws);
   {  // pass B and the multiply by V_loc; the largest component of the product
     const int2* v = Vs + (int64_t)z * N * N;
     unsigned m = 0;
@@ -461,6 +470,86 @@ __device__ __forceinline__ void plane_body(cdf* __restrict__ T, const int2* __re
       const int c = __ldg(rc + NB * na);
       if (c >= 0) t[c] = cdf{from_fixed(v[na].x, out), from_fixed(v[na].y, out)};
     }
+  }
+}
+
+// x 2^s rounded to an integer, |x 2^s| < 2^61, by integer operations on the bits (the FP64
+// unit takes 65 clocks a warp for a conversion); subnormals count as zero
+__device__ __forceinline__ ll to_fixed(double x, int s) {
+  const ll b = __double_as_longlong(x);
+  const int e = (int)(b >> 52) & 0x7FF, k = e - 1075 + s;
+  ll q = (b & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+  q = e == 0 || k < -54 ? 0 : k >= 0 ? q << k : (q + (1ll << (-k - 1))) >> -k;
+  return b < 0 ? -q : q;
+}
+// v 2^-s as a double
+__device__ __forceinline__ double to_double(ll v, int s) {
+  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+  const int lz = __clzll((ll)u), e = 63 - lz - s;
+  if (u == 0 || e < -1022) return 0.0;
+  const unsigned long long m = u << lz;  // leading one at bit 63
+  // the implicit bit and the rounding carry add into the exponent field
+  const ll bits = ((ll)(e + 1022) << 52) + (ll)((m >> 11) + ((m >> 10) & 1));
+  return __longlong_as_double(bits | (v < 0 ? 1ll << 63 : 0));
+}
+
+// Real-space values of plane z of band b from the FP64 column buffer, for the derivative with
+// respect to V_loc: out[x'][y'] in split order.
+template <int N, int NT>
+__device__ __forceinline__ void plane_real_body(const double2* __restrict__ T, double2* __restrict__ out,
+                                                const fk::FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = fk::plane_pitch(N);
+  __shared__ float red[NT / 32];
+  __shared__ int emax;
+  __shared__ int4 tws[N];
+  cfx* plane = reinterpret_cast<cfx*>(smem_raw);
+  const double2* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
+  const int tid = threadIdx.x;
+  if (tid == 0) emax = 0;
+  for (int i = tid; i < N; i += NT) tws[i] = c_twfx[fk::TwOff<N>::v + i];
+  __syncthreads();
+  // the largest exponent, then the magnitudes' sum relative to it
+  int e = 0;
+  for (int c = tid; c < fa.ncol; c += NT)
+    e = max(e, max((__double2hiint(t[c].x) >> 20) & 0x7FF, (__double2hiint(t[c].y) >> 20) & 0x7FF));
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (tid % 32 == 0) atomicMax(&emax, e);
+  __syncthreads();
+  e = emax;
+  if (e == 0x7FF) {
+    const double q = __longlong_as_double(0x7FF8000000000000ll);
+    for (int i = tid; i < N * N; i += NT) out[i] = make_double2(q, q);
+    return;
+  }
+  auto part = [&](double v) {  // |v| 2^(1023 - e) from the top bits
+    const int h = __double2hiint(v) & 0x7FFFFFFF, k = (h >> 20) - e + 127;
+    return k > 0 ? __int_as_float((k << 23) | ((h & 0xFFFFF) << 3)) : 0.f;
+  };
+  float sum = 0.f;
+  for (int c = tid; c < fa.ncol; c += NT) sum += part(t[c].x) + part(t[c].y);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (tid % 32 == 0) red[tid / 32] = sum;
+  __syncthreads();
+  sum = 0.f;
+#pragma unroll
+  for (int i = 0; i < NT / 32; ++i) sum += red[i];
+  // sum (|re| + |im|) 2^s <= 2^60, one bit spare for the truncated parts
+  const int s = 60 - (e - 1023) - (sum > 0.f ? ilogbf(sum) + 1 : 0);
+  inverse_passes<N, NT>([&](int c) {
+    const double2 u = t[c];
+    return cfx{to_fixed(u.x, s), to_fixed(u.y, s)};
+  }, fa, plane, tws);
+  for (int it = tid; it < N * NA; it += NT) {  // pass B; the twiddles halved the values twice
+    const int ka = it / N, yy = it - ka * N;
+    const cfx* a = plane + yy + NB * ka * P;
+    cfx u[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) u[q] = a[q * P];
+    dft<NB, +1>(u);
+    double2* o = out + (int64_t)(NB * ka) * N + yy;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) o[q * N] = make_double2(to_double(u[q].x, s - 2), to_double(u[q].y, s - 2));
   }
 }
 

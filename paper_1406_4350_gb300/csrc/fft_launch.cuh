@@ -15,4 +15,13 @@ template <typename R>
 bool fast_dispatch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t ldy, int64_t nb, cplx<R>* T,
                    LocalEpi<typename SphT<R>::type> ep, cudaStream_t st, const typename SphT<R>::type* K);
 
+// Real-space values of nb <= 65535 bands on a compiled grid, out[band][z'][x'][y'] in split
+// order (T: column buffer): the z pass, and with `planes` the plane pass; false if the size
+// has no compiled kernels.  fixed_planes_real: the plane pass from an FP64 column buffer in
+// fixed point (false at sizes without it).
+template <typename R>
+bool fast_real_space(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx<R>* T, cplx<R>* out, bool planes,
+                     cudaStream_t st);
+bool fixed_planes_real(chebfi_ctx* ctx, int64_t nb, const double2* T, double2* out, cudaStream_t st);
+
 }  // namespace chebfi

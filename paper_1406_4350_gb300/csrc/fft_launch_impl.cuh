@@ -47,6 +47,24 @@ __global__ void __launch_bounds__(fx_threads<N>()) k_plane_fx(cdf* __restrict__ 
 }
 #endif
 
+#ifndef CHEBFI_FFT_DF
+template <typename R, int N>
+__global__ void __launch_bounds__(kThreads) k_plane_real_f(const cplx<R>* __restrict__ T, cplx<R>* __restrict__ out,
+                                                           FastArgs fa) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fk::plane_real_body<R, N, kThreads>(T, out + ((int64_t)blockIdx.y * N + blockIdx.x) * N * N, fa, blockIdx.x, blockIdx.y,
+                                      smem_raw);
+}
+#else
+template <int N>
+__global__ void __launch_bounds__(fx_threads<N>()) k_plane_real_fx(const double2* __restrict__ T, double2* __restrict__ out,
+                                                                   FastArgs fa) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fx::plane_real_body<N, fx_threads<N>()>(T, out + ((int64_t)blockIdx.y * N + blockIdx.x) * N * N, fa, blockIdx.x, blockIdx.y,
+                                          smem_raw);
+}
+#endif
+
 template <typename R, int N3>
 __global__ void __launch_bounds__(kThreads) k_zfwd_f(const cplx<R>* __restrict__ T, FastArgs fa,
                                                      const cplx<R>* __restrict__ twz,
@@ -110,6 +128,33 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
   }
 }
 
+#ifndef CHEBFI_FFT_DF
+template <typename R, int N>
+void real_launch(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx<R>* T, cplx<R>* out, bool planes,
+                 cudaStream_t st) {
+  const SphereFFT& s = ctx->sph;
+  const FastArgs fa = fk::fast_args(ctx);
+  CHEBFI_REQUIRE(nb <= 65535, CHEBFI_ERR_ARG, "too many bands in a chunk");
+  const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>), pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
+  const cplx<R>* tw = nullptr;
+  fk::init_twiddles();
+  set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
+  const dim3 gz((s.ncol + kCBF - 1) / kCBF, (unsigned)nb);
+  CHEBFI_LAUNCH("k_zinv", st, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y, ldy, T, fa, tw));
+  if (!planes) return;
+  set_smem<R>((const void*)k_plane_real_f<R, N>, pbytes);
+  CHEBFI_LAUNCH("k_plane_real", st, k_plane_real_f<R, N><<<dim3(N, (unsigned)nb), kThreads, pbytes, st>>>(T, out, fa));
+}
+#else
+template <int N> void real_launch_fx(chebfi_ctx* ctx, int64_t nb, const double2* T, double2* out, cudaStream_t st) {
+  const size_t pbytes = (size_t)(N * ctx->sph.pitch) * sizeof(double2);
+  fx::init_twiddles();
+  set_smem<dfl>((const void*)k_plane_real_fx<N>, pbytes);
+  CHEBFI_LAUNCH("k_plane_real", st,
+                k_plane_real_fx<N><<<dim3(N, (unsigned)nb), fx_threads<N>(), pbytes, st>>>(T, out, fk::fast_args(ctx)));
+}
+#endif
+
 }  // namespace
 
 // Compile-time-length path for cubic grids of the compiled sizes; false = not taken.
@@ -128,5 +173,30 @@ bool fast_dispatch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64
     default: return false;
   }
 }
+
+
+#ifndef CHEBFI_FFT_DF
+template <typename R>
+bool fast_real_space(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx<R>* T, cplx<R>* out, bool planes,
+                     cudaStream_t st) {
+  switch (ctx->grid[0]) {
+#define CHEBFI_X(n) \
+  case n: real_launch<R, n>(ctx, Y, ldy, nb, T, out, planes, st); return true;
+    CHEBFI_FFT_SIZES(CHEBFI_X)
+#undef CHEBFI_X
+    default: return false;
+  }
+}
+#else
+bool fixed_planes_real(chebfi_ctx* ctx, int64_t nb, const double2* T, double2* out, cudaStream_t st) {
+  switch (ctx->grid[0]) {
+#define CHEBFI_X(n) \
+  case n: real_launch_fx<n>(ctx, nb, T, out, st); return true;
+    CHEBFI_FFT_DF_SIZES(CHEBFI_X)
+#undef CHEBFI_X
+    default: return false;
+  }
+}
+#endif
 
 }  // namespace chebfi

@@ -190,3 +190,44 @@ def test_fixed_point_planes_keep_non_finite_bands_apart():
     good = _np(g.apply_H(_F(cell.Y0)))
     assert np.isnan(got[:, 1]).all() and np.isnan(got[:, 2]).all()
     assert np.array_equal(got[:, [0, 3]], good[:, [0, 3]])
+
+
+# the FP32 CUDA-core GEMM through the FP32 filter: projector and band counts at the edges of
+# its 64 x 64 and 64 x 32 tiles and of its K splits, with and without S
+@pytest.mark.parametrize("nb", [1, 31, 33, 64, 65, 130])
+@pytest.mark.parametrize("natoms,nlmn,paw", [(1, 1, False), (8, 8, True), (9, 8, True)])
+def test_fp32_filter_tile_edges(nb, natoms, nlmn, paw):
+    cell = make_cell(12.0, 30, 5.0, natoms, nlmn, nb, paw, 38)
+    op = PWOperator.from_cell(cell)
+    lo, hi, _, _ = ch.bounds(op, cell.Y0, mode="rigorous")
+    ref = ch.filter_plain(op, cell.Y0, 3, lo, hi)
+    g = _ctx(cell)
+    Y = _F(cell.Y0)
+    g.cheb_filter(Y, 3, lo, hi, prec=1)
+    assert np.abs(_np(Y) - ref).max() <= 2e-5 * 3 * np.abs(ref).max()  # the FP32 tolerance per step
+
+
+# the derivative with respect to V_loc on grids with fixed-point planes, compiled FP64 planes
+# and the general passes; bands of very different sizes share no scale
+@pytest.mark.parametrize("n", [16, 18, 24, 30, 32, 45, 48, 60, 64])
+def test_vloc_gradient_on_every_kind_of_grid(n):
+    L = 0.42 * n
+    ecut = 0.5 * (2.0 * np.pi / L * 0.24 * n) ** 2
+    cell = make_cell(L, n, ecut, 1, 8, 5, True, 39, kpt=(0.02, -0.05, 0.03))
+    rng = np.random.default_rng(n)
+    Y, G = cell.Y0.copy(), _rand(rng, cell.npw, 5)
+    Y[:, 1] *= 1e9
+    G[:, 1] *= 1e-9
+    Y[:, 2] = 0.0
+    m = np.asarray(cell.miller)
+
+    def box(c):
+        b = np.zeros((n, n, n), dtype=complex)
+        b[m[:, 0] % n, m[:, 1] % n, m[:, 2] % n] = c
+        return np.fft.ifftn(b) * n ** 3
+    ref = sum((box(G[:, j]).conj() * box(Y[:, j])).real for j in range(5)) / n ** 3
+    g = _ctx(cell)
+    _, gV, _ = g.apply_H_backward(_F(Y), _F(G), (n, n, n), len(cell.D))
+    # two transforms of log2(n^3) levels and the product, each about 2^-52 of its norm
+    bound = 64.0 * 2.0 ** -52 * sum(np.linalg.norm(G[:, j]) * np.linalg.norm(Y[:, j]) for j in range(5)) / n ** 1.5
+    assert np.linalg.norm(_np(gV) - ref) <= bound
