@@ -199,8 +199,18 @@ void gemm64(chebfi_ctx* ctx, bool conjA, bool conjB, int64_t M, int64_t N, int64
   const OzOperand* a = &z.A;
   const bool is_P = ctx->has_proj && A == ctx->d_P.p && lda == ctx->npw &&
                     (conjA ? (M == ctx->nproj && K == ctx->npw) : (M == ctx->npw && K == ctx->nproj));
-  if (is_P) a = &oz_P(ctx, conjA, st);
-  else oz_prepare(A, lda, M, K, conjA, conjA, ctx->oz_nmod, z.A, st);
+  const bool square = ctx->has_proj && !conjA && lda == ctx->nproj && M == ctx->nproj && K == ctx->nproj;
+  if (is_P) {
+    a = &oz_P(ctx, conjA, st);
+  } else if (square && (A == ctx->d_G.p || A == ctx->d_M.p)) {
+    // the Woodbury core's constant matrices: three of a filter step's products, whose operand
+    // preparation costs as much as the product
+    OzOperand& o = A == ctx->d_G.p ? ctx->ozG : ctx->ozM;
+    if (o.nmod != ctx->oz_nmod) oz_prepare(A, lda, M, K, false, false, ctx->oz_nmod, o, st);
+    a = &o;
+  } else {
+    oz_prepare(A, lda, M, K, conjA, conjA, ctx->oz_nmod, z.A, st);
+  }
   oz_prepare(B, ldb, N, K, !conjB, conjB, ctx->oz_nmod, z.B, st);
   oz_gemm(*a, z.B, alpha, beta, C, ldc, lower, z.R, ctx->d_status.p, st, tag);
 }
@@ -1451,7 +1461,7 @@ int chebfi_set_projectors(chebfi_ctx* ctx, int64_t nproj, const void* P, int64_t
   ctx->paw = false;
   ctx->bound_rigorous = -1.0;
   ctx->has_proj = false;
-  ctx->ozPh.nmod = ctx->ozP.nmod = 0;  // residues of the previous P are stale
+  ctx->ozPh.nmod = ctx->ozP.nmod = ctx->ozG.nmod = ctx->ozM.nmod = 0;  // residues of the previous P are stale
   ctx->tc_ready = ctx->tcP_ready = ctx->tc3_ready = false;  // and so are its bf16 embeddings
   if (nproj == 0) {
     ctx->has_proj = true;
