@@ -306,11 +306,12 @@ cplx<R>* filter_sorted(chebfi_ctx* ctx, FilterBufs<R> b, int64_t nb0, int degree
     const int64_t nb = active ? active[k] : nb0;  // bands still being filtered (a prefix)
     const double a = (k == 0 ? 1.0 : 2.0) / r;
     const double bp = k == 0 ? 0.0 : 1.0;
+    const bool last = k + 1 == degree;  // p_{k+1} has no reader: only what W needs is formed
     // Z = (K + V_loc) Y_k and T = a (Z - c Y_k) - bp Y_{k-1}, T written over Y_{k-1}
     LocalEpi<R> ep;
     ep.Y = cur;
     ep.ldy = npw;
-    ep.Z = nq > 0 ? b.Z : nullptr;
+    ep.Z = nq > 0 && (!last || ctx->paw) ? b.Z : nullptr;
     ep.ldz = npw;
     ep.T = prev;
     ep.Yprev = k == 0 ? nullptr : prev;
@@ -320,25 +321,29 @@ cplx<R>* filter_sorted(chebfi_ctx* ctx, FilterBufs<R> b, int64_t nb0, int degree
     ep.bprev = (R)bp;
     local_apply<R>(ctx, cur, npw, nb, b.T, ep, st);
     if (nq > 0) {
-      // P^H H Y_k = P^H Z + G D p_k
-      cgemm<R>(ctx, true, false, nq, nb, npw, 1.0, Ops<R>::P(ctx), npw, b.Z, npw, 0.0, b.pz, nq, st, Ops<R>::ws(ctx),
-              "gemm_PhY");
       blockdiag_apply<R>(ctx, Ops<R>::D(ctx), pcur, nq, b.pw, nq, nb, st);
-      cgemm<R>(ctx, false, false, nq, nb, nq, 1.0, Ops<R>::G(ctx), nq, b.pw, nq, 1.0, b.pz, nq, st, Ops<R>::ws(ctx),
-              "gemm_small");
+      if (!last || ctx->paw) {
+        // P^H H Y_k = P^H Z + G D p_k
+        cgemm<R>(ctx, true, false, nq, nb, npw, 1.0, Ops<R>::P(ctx), npw, b.Z, npw, 0.0, b.pz, nq, st, Ops<R>::ws(ctx),
+                "gemm_PhY");
+        cgemm<R>(ctx, false, false, nq, nb, nq, 1.0, Ops<R>::G(ctx), nq, b.pw, nq, 1.0, b.pz, nq, st, Ops<R>::ws(ctx),
+                "gemm_small");
+      }
       if (ctx->paw) {
         // q = M P^H H Y_k;  W = D p_k - q;  P^H S^{-1} H Y_k = P^H H Y_k - G q
         cgemm<R>(ctx, false, false, nq, nb, nq, 1.0, Ops<R>::M(ctx), nq, b.pz, nq, 0.0, b.pq, nq, st, Ops<R>::ws(ctx),
                 "gemm_small");
         axpby<R>(nq, nb, (R)1, b.pw, nq, (R)-1, b.pq, nq, b.pw, nq, st);
-        cgemm<R>(ctx, false, false, nq, nb, nq, -1.0, Ops<R>::G(ctx), nq, b.pq, nq, 1.0, b.pz, nq, st, Ops<R>::ws(ctx),
-                "gemm_small");
+        if (!last)
+          cgemm<R>(ctx, false, false, nq, nb, nq, -1.0, Ops<R>::G(ctx), nq, b.pq, nq, 1.0, b.pz, nq, st, Ops<R>::ws(ctx),
+                  "gemm_small");
       }
       // Y_{k+1} = T + a P W
       cgemm<R>(ctx, false, false, npw, nb, nq, a, Ops<R>::P(ctx), npw, b.pw, nq, 1.0, prev, npw, st, Ops<R>::ws(ctx),
               "gemm_PW");
       // p_{k+1} = a (P^H S^{-1} H Y_k - c p_k) - bp p_{k-1}
-      cheb_combine<R>(nq, nb, (R)a, b.pz, nq, (R)c, pcur, nq, (R)bp, k == 0 ? nullptr : pprev, nq, pprev, nq, st);
+      if (!last)
+        cheb_combine<R>(nq, nb, (R)a, b.pz, nq, (R)c, pcur, nq, (R)bp, k == 0 ? nullptr : pprev, nq, pprev, nq, st);
     }
     std::swap(cur, prev);
     std::swap(pcur, pprev);
@@ -403,10 +408,11 @@ float2* filter_mixed(chebfi_ctx* ctx, FilterBufs<float> b, int64_t nb0, int degr
     const int64_t nb = active ? active[k] : nb0;  // bands still being filtered (a prefix)
     const double a = (k == 0 ? 1.0 : 2.0) / r;
     const double bp = k == 0 ? 0.0 : 1.0;
+    const bool last = k + 1 == degree;  // as in filter_sorted
     LocalEpi<float> ep;
     ep.Y = cur;
     ep.ldy = npw;
-    if (nq > 0) {
+    if (nq > 0 && (!last || ctx->paw)) {
       ep.Zhi = w.Zb.hi.p;
       ep.Zlo = w.Zb.lo.p;
       ep.ldzb = ldzb;
@@ -419,28 +425,33 @@ float2* filter_mixed(chebfi_ctx* ctx, FilterBufs<float> b, int64_t nb0, int degr
     ep.bprev = (float)bp;
     local_apply<float>(ctx, cur, npw, nb, b.T, ep, st);
     if (nq > 0) {
-      // P^H H Y_k = P^H Z + G D p_k
-      tc_gemm(ctx->tcA1.view(), w.Zb.view(), 2 * nq, nb, 2 * npw, 1.f, 0.f, nullptr, 0, (float*)b.pz, 2 * nq, status,
-              st, "tc_gemm_PhY", &ctx->w.tcws);
       blockdiag_apply<float>(ctx, ctx->d_Dblkf.p, pcur, nq, b.pw, nq, nb, st);
-      split_block(nq, nb, b.pw, nq, w.Sb, st);
-      tc_gemm(ctx->tcAG.view(), w.Sb.view(), 2 * nq, nb, 2 * nq, 1.f, 1.f, (float*)b.pz, 2 * nq, (float*)b.pz, 2 * nq,
-              status, st, "tc_gemm_small", &ctx->w.tcws);
+      if (!last || ctx->paw) {
+        // P^H H Y_k = P^H Z + G D p_k
+        tc_gemm(ctx->tcA1.view(), w.Zb.view(), 2 * nq, nb, 2 * npw, 1.f, 0.f, nullptr, 0, (float*)b.pz, 2 * nq, status,
+                st, "tc_gemm_PhY", &ctx->w.tcws);
+        split_block(nq, nb, b.pw, nq, w.Sb, st);
+        tc_gemm(ctx->tcAG.view(), w.Sb.view(), 2 * nq, nb, 2 * nq, 1.f, 1.f, (float*)b.pz, 2 * nq, (float*)b.pz, 2 * nq,
+                status, st, "tc_gemm_small", &ctx->w.tcws);
+      }
       if (ctx->paw) {
         split_block(nq, nb, b.pz, nq, w.Sb, st);
         tc_gemm(ctx->tcAM.view(), w.Sb.view(), 2 * nq, nb, 2 * nq, 1.f, 0.f, nullptr, 0, (float*)b.pq, 2 * nq, status,
                 st, "tc_gemm_small", &ctx->w.tcws);
         axpby<float>(nq, nb, 1.f, b.pw, nq, -1.f, b.pq, nq, b.pw, nq, st);
-        split_block(nq, nb, b.pq, nq, w.Sb, st);
-        tc_gemm(ctx->tcAG.view(), w.Sb.view(), 2 * nq, nb, 2 * nq, -1.f, 1.f, (float*)b.pz, 2 * nq, (float*)b.pz,
-                2 * nq, status, st, "tc_gemm_small", &ctx->w.tcws);
+        if (!last) {
+          split_block(nq, nb, b.pq, nq, w.Sb, st);
+          tc_gemm(ctx->tcAG.view(), w.Sb.view(), 2 * nq, nb, 2 * nq, -1.f, 1.f, (float*)b.pz, 2 * nq, (float*)b.pz,
+                  2 * nq, status, st, "tc_gemm_small", &ctx->w.tcws);
+        }
       }
       // Y_{k+1} = T + a P W
       split3_block(nq, nb, b.pw, nq, w.W3, st);
       tc_cgemm3(ctx->tcP3, w.W3, false, npw, nb, nq, (float)a, 1.f, prev, npw, prev, npw, status, st, "tc_gemm_PW",
                 &ctx->w.tcws);
-      cheb_combine<float>(nq, nb, (float)a, b.pz, nq, (float)c, pcur, nq, (float)bp, k == 0 ? nullptr : pprev, nq,
-                          pprev, nq, st);
+      if (!last)
+        cheb_combine<float>(nq, nb, (float)a, b.pz, nq, (float)c, pcur, nq, (float)bp, k == 0 ? nullptr : pprev, nq,
+                            pprev, nq, st);
     }
     std::swap(cur, prev);
     std::swap(pcur, pprev);

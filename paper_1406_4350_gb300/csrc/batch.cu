@@ -543,18 +543,20 @@ void batch_filter_body(chebfi_batch* bt, int degree, cudaStream_t st) {
   if (nq > 0) bgemm<R>(bt, OP_PHY, 0, cur, pcur, slot++, st);
   for (int k = 0; k < degree; ++k) {
     const int first = k == 0 ? 1 : 0;
-    blocal_n<R>(bt, cur, nq > 0 ? Z : nullptr, prev, first, st);
+    const bool last = k + 1 == degree, need_pz = !last || bt->paw;  // p_{k+1} has no reader after the last step
+    blocal_n<R>(bt, cur, nq > 0 && need_pz ? Z : nullptr, prev, first, st);
     if (nq > 0) {
-      bgemm<R>(bt, OP_PHY, first, Z, pz, slot++, st);                       // P^H Z
+      if (need_pz) bgemm<R>(bt, OP_PHY, first, Z, pz, slot++, st);          // P^H Z
       blockdiag_apply<R>(bt->ks[0], BatchOps<R>::D(bt->ks[0]), pcur, nq, pw, nq, nk * nb, st);  // D p
-      bgemm<R>(bt, OP_G, first, pw, pz, slot++, st);                        // + G D p
+      if (need_pz) bgemm<R>(bt, OP_G, first, pw, pz, slot++, st);           // + G D p
       if (bt->paw) {
         bgemm<R>(bt, OP_M, first, pz, pq, slot++, st);                      // q = M P^H H Y
         axpby<R>(nq, nk * nb, (R)1, pw, nq, (R)-1, pq, nq, pw, nq, st);     // W = D p - q
-        bgemm<R>(bt, OP_GNEG, first, pq, pz, slot++, st);                   // P^H S^{-1} H Y
+        if (!last) bgemm<R>(bt, OP_GNEG, first, pq, pz, slot++, st);        // P^H S^{-1} H Y
       }
       bgemm<R>(bt, OP_PW, first, pw, prev, slot++, st);                     // Y_{k+1} = T + a P W
-      CHEBFI_LAUNCH("k_bcombine", st, (k_bcombine<R><<<nblk(nk * nq * nb), 256, 0, st>>>(d, nq * nb, nk * nq * nb, pz, pcur, pprev, first)));
+      if (!last)
+        CHEBFI_LAUNCH("k_bcombine", st, (k_bcombine<R><<<nblk(nk * nq * nb), 256, 0, st>>>(d, nq * nb, nk * nq * nb, pz, pcur, pprev, first)));
     }
     std::swap(cur, prev);
     std::swap(pcur, pprev);
@@ -714,22 +716,30 @@ void batch_filter_body_mixed(chebfi_batch* bt, int degree, cudaStream_t st) {
   tc_group(bt, TV_PHY0, 1.f, st);  // p_0 = P^H Y_0, into pa
   for (int k = 0; k < degree; ++k) {
     const int first = k == 0 ? 1 : 0;
+    const bool last = k + 1 == degree, need_pz = !last || bt->paw;
     blocal_n<float>(bt, cur, Z, prev, first, st);
-    CHEBFI_LAUNCH("k_bsplit_z", st, (k_bsplit_z<float><<<gg, 256, 0, st>>>(d, nb, Z, bt->d_zb_off.p, bt->d_zb_ld.p, bt->zb.hi.p, bt->zb.lo.p)));
-    tc_group(bt, TV_PHY, 1.f, st);                                                                    // P^H Z
+    if (need_pz) {
+      CHEBFI_LAUNCH("k_bsplit_z", st, (k_bsplit_z<float><<<gg, 256, 0, st>>>(d, nb, Z, bt->d_zb_off.p, bt->d_zb_ld.p, bt->zb.hi.p, bt->zb.lo.p)));
+      tc_group(bt, TV_PHY, 1.f, st);                                                                  // P^H Z
+    }
     blockdiag_apply<float>(bt->ks[0], BatchOps<float>::D(bt->ks[0]), pcur, nq, pw, nq, nk * nb, st);  // D p
-    split_block(nq, nk * nb, pw, nq, bt->sb, st);
-    tc_group(bt, TV_G, 1.f, st);                                                                      // + G D p
+    if (need_pz) {
+      split_block(nq, nk * nb, pw, nq, bt->sb, st);
+      tc_group(bt, TV_G, 1.f, st);                                                                    // + G D p
+    }
     if (bt->paw) {
       split_block(nq, nk * nb, pz, nq, bt->sb, st);
       tc_group(bt, TV_M, 1.f, st);                                                // q = M P^H H Y
       axpby<float>(nq, nk * nb, 1.f, pw, nq, -1.f, pq, nq, pw, nq, st);           // W = D p - q
-      split_block(nq, nk * nb, pq, nq, bt->sb, st);
-      tc_group(bt, TV_GNEG, 1.f, st);                                             // P^H S^{-1} H Y
+      if (!last) {
+        split_block(nq, nk * nb, pq, nq, bt->sb, st);
+        tc_group(bt, TV_GNEG, 1.f, st);                                           // P^H S^{-1} H Y
+      }
     }
     split_block(nq, nk * nb, pw, nq, bt->sb, st);
     tc_group(bt, prev == Yb[0] ? TV_PW0 : TV_PW1, first ? 1.f : 2.f, st);       // Y_{k+1} = T + a P W
-    CHEBFI_LAUNCH("k_bcombine", st, (k_bcombine<float><<<nblk(nk * nq * nb), 256, 0, st>>>(d, nq * nb, nk * nq * nb, pz, pcur, pprev, first)));
+    if (!last)
+      CHEBFI_LAUNCH("k_bcombine", st, (k_bcombine<float><<<nblk(nk * nq * nb), 256, 0, st>>>(d, nq * nb, nk * nq * nb, pz, pcur, pprev, first)));
     std::swap(cur, prev);
     std::swap(pcur, pprev);
   }
