@@ -316,13 +316,15 @@ int chebfi_gemm_fp64(chebfi_ctx* ctx, int conjA, int conjB, int64_t m, int64_t n
                      void* stream);
 
 /* Arithmetic of the FFT passes of the FP64 path (the FP64 form's filter, apply_H and the
- * H application of Rayleigh-Ritz in every form) on the compile-time grids (cubic 24, 32, 48,
- * 64, 72, 96):
- *  CHEBFI_FFT64_DOUBLE_FLOAT (initial): double-float arithmetic on the FP32 units -- each
- *    value the unevaluated sum of two floats (48-bit significand, float's exponent range),
- *    the error-free TwoSum / Fast2Sum / FMA-TwoProd transformations of Knuth and Dekker; a
- *    transform keeps about 2^-44 of its line's norm; GB300's FP64 units run at ~1/64 of the
- *    FP32 rate, so this is several times faster;
+ * H application of Rayleigh-Ritz in every form) on the compile-time grids (cubic 16, 20, 24,
+ * 30, 32, 36, 40, 45, 48, 54, 60, 64, 72, 80, 90, 96, 100, 108):
+ *  CHEBFI_FFT64_DOUBLE_FLOAT (initial): off the FP64 units, which run at ~1/64 of the FP32
+ *    rate, as far as that goes.  On 24, 32, 48, 64, 72 and 96 the z passes in double-float on
+ *    the FP32 units -- each value the unevaluated sum of two floats (48-bit significand,
+ *    float's exponent range), the error-free TwoSum / Fast2Sum / FMA-TwoProd transformations
+ *    of Knuth and Dekker; a transform keeps about 2^-44 of its line's norm -- and the planes
+ *    in 64-bit fixed point, one scale per plane.  On the others but 90 the z passes in FP64
+ *    and the planes in fixed point, which together keep FP64's accuracy;
  *  CHEBFI_FFT64_NATIVE: FP64 arithmetic on the FP64 units.
  * Blocks, V_loc and the results stay FP64 in memory either way.  Other grids use FP64. */
 enum { CHEBFI_FFT64_NATIVE = 0, CHEBFI_FFT64_DOUBLE_FLOAT = 1 };

@@ -340,7 +340,7 @@ class ChebFI:
 
     def set_fft64(self, mode: int):
         """Arithmetic of the FP64 path's FFT passes: FFT64_DOUBLE_FLOAT (initial; pairs of
-        floats on the FP32 units) or FFT64_NATIVE (the FP64 units)."""
+        floats on the FP32 units and 64-bit fixed point) or FFT64_NATIVE (the FP64 units)."""
         self._check(self.lib.chebfi_set_fft64(self.h, mode))
 
     def set_eigensolver(self, mode: int):

@@ -239,9 +239,10 @@ size_t local_workspace_elems(const chebfi_ctx* ctx, int64_t nb) {
   return (size_t)ctx->grid[2] * ncolp * (size_t)nb;
 }
 
-// The FP64 path runs its transforms in double-float on the FP32 units, at the lengths that
-// have them, unless the FP64 units are asked for (chebfi_set_fft64); the column buffer's complex doubles then hold
-// double-float values, 16 bytes each as well.
+// Unless the FP64 units are asked for (chebfi_set_fft64), the FP64 path runs its z passes in
+// double-float on the FP32 units and its planes in fixed point at the lengths that have both
+// (the column buffer's complex doubles then hold double-float values, 16 bytes each as well),
+// and fixed-point planes between FP64 z passes at most others.
 template <typename R>
 bool fast_apply(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx<R>* T, LocalEpi<R> ep,
                 cudaStream_t st, const R* K) {
@@ -279,6 +280,7 @@ bool fixed_fft_size(int n) {
   switch (n) {
 #define CHEBFI_X(n) case n:
     CHEBFI_FFT_DF_SIZES(CHEBFI_X)
+    CHEBFI_FFT_FX_SIZES(CHEBFI_X)
 #undef CHEBFI_X
     return true;
     default: return false;

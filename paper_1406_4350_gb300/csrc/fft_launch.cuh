@@ -23,5 +23,10 @@ template <typename R>
 bool fast_real_space(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx<R>* T, cplx<R>* out, bool planes,
                      cudaStream_t st);
 bool fixed_planes_real(chebfi_ctx* ctx, int64_t nb, const double2* T, double2* out, cudaStream_t st);
+// The plane pass (multiply by V_loc included) of nb <= 65535 bands in fixed point; false where
+// the context's FP64 path does not take it.
+bool fixed_planes(chebfi_ctx* ctx, int64_t nb, cdf* T, cudaStream_t st);
+bool fixed_planes(chebfi_ctx* ctx, int64_t nb, double2* T, cudaStream_t st);
+inline bool fixed_planes(chebfi_ctx*, int64_t, float2*, cudaStream_t) { return false; }
 
 }  // namespace chebfi

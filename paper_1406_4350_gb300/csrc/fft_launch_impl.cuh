@@ -4,9 +4,6 @@
 #pragma once
 
 #include "fft_launch.cuh"
-#ifdef CHEBFI_FFT_DF
-#include "fft_fixed.cuh"
-#endif
 
 namespace chebfi {
 namespace {
@@ -34,19 +31,6 @@ __global__ void __launch_bounds__(kThreads) k_plane_f(cplx<R>* __restrict__ T, c
   fk::plane_body_pruned<R, N, kThreads>(T, Vs, fa, blockIdx.x, blockIdx.y, smem_raw);
 }
 
-#ifdef CHEBFI_FFT_DF
-// The plane pass of the double-float path runs in 64-bit fixed point (16 bytes a point: the
-// 96-point plane fills an SM, whose one block then takes 24 warps; smaller planes run in
-// smaller blocks so that several share an SM and fill each other's barriers).
-template <int N> constexpr int fx_threads() { return N >= 96 ? 768 : N >= 48 ? 256 : 128; }
-template <int N>
-__global__ void __launch_bounds__(fx_threads<N>()) k_plane_fx(cdf* __restrict__ T, const int2* __restrict__ Vs, int ve,
-                                                              FastArgs fa) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  fx::plane_body<N, fx_threads<N>()>(T, Vs, ve, fa, blockIdx.x, blockIdx.y, smem_raw);
-}
-#endif
-
 #ifndef CHEBFI_FFT_DF
 template <typename R, int N>
 __global__ void __launch_bounds__(kThreads) k_plane_real_f(const cplx<R>* __restrict__ T, cplx<R>* __restrict__ out,
@@ -54,14 +38,6 @@ __global__ void __launch_bounds__(kThreads) k_plane_real_f(const cplx<R>* __rest
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fk::plane_real_body<R, N, kThreads>(T, out + ((int64_t)blockIdx.y * N + blockIdx.x) * N * N, fa, blockIdx.x, blockIdx.y,
                                       smem_raw);
-}
-#else
-template <int N>
-__global__ void __launch_bounds__(fx_threads<N>()) k_plane_real_fx(const double2* __restrict__ T, double2* __restrict__ out,
-                                                                   FastArgs fa) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  fx::plane_real_body<N, fx_threads<N>()>(T, out + ((int64_t)blockIdx.y * N + blockIdx.x) * N * N, fa, blockIdx.x, blockIdx.y,
-                                          smem_raw);
 }
 #endif
 
@@ -93,10 +69,7 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
   const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
   fk::init_twiddles();
-#ifdef CHEBFI_FFT_DF
-  fx::init_twiddles();
-  set_smem<R>((const void*)k_plane_fx<N>, pbytes);
-#else
+#ifndef CHEBFI_FFT_DF
   set_smem<R>((const void*)k_plane_f<R, N>, pbytes);
 #endif
   set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
@@ -106,12 +79,13 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
     dim3 gz((s.ncol + kCBF - 1) / kCBF, nbc);
     const double esz = sizeof(cplx<R>), col = (double)N * s.ncol * nbc * esz, sph = (double)ctx->npw * nbc * esz;
     CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
-#ifdef CHEBFI_FFT_DF
-    CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col,
-                    k_plane_fx<N><<<dim3(N, nbc), fx_threads<N>(), pbytes, st>>>(T, ctx->d_vsfx.p, ctx->v_exp, fa));
+    if (!fixed_planes(ctx, nbc, T, st)) {
+#ifndef CHEBFI_FFT_DF
+      CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col, k_plane_f<R, N><<<dim3(N, nbc), kThreads, pbytes, st>>>(T, vtable<R>(ctx), fa));
 #else
-    CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col, k_plane_f<R, N><<<dim3(N, nbc), kThreads, pbytes, st>>>(T, vtable<R>(ctx), fa));
+      CHEBFI_REQUIRE(false, CHEBFI_ERR_STATE, "double-float columns without fixed-point planes");
 #endif
+    }
     LocalEpi<S> e = ep;
     e.Y = ep.Y + b0 * ep.ldy;
     if (e.Z) e.Z = ep.Z + b0 * ep.ldz;
@@ -145,14 +119,6 @@ void real_launch(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cpl
   set_smem<R>((const void*)k_plane_real_f<R, N>, pbytes);
   CHEBFI_LAUNCH("k_plane_real", st, k_plane_real_f<R, N><<<dim3(N, (unsigned)nb), kThreads, pbytes, st>>>(T, out, fa));
 }
-#else
-template <int N> void real_launch_fx(chebfi_ctx* ctx, int64_t nb, const double2* T, double2* out, cudaStream_t st) {
-  const size_t pbytes = (size_t)(N * ctx->sph.pitch) * sizeof(double2);
-  fx::init_twiddles();
-  set_smem<dfl>((const void*)k_plane_real_fx<N>, pbytes);
-  CHEBFI_LAUNCH("k_plane_real", st,
-                k_plane_real_fx<N><<<dim3(N, (unsigned)nb), fx_threads<N>(), pbytes, st>>>(T, out, fk::fast_args(ctx)));
-}
 #endif
 
 }  // namespace
@@ -183,16 +149,6 @@ bool fast_real_space(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb,
 #define CHEBFI_X(n) \
   case n: real_launch<R, n>(ctx, Y, ldy, nb, T, out, planes, st); return true;
     CHEBFI_FFT_SIZES(CHEBFI_X)
-#undef CHEBFI_X
-    default: return false;
-  }
-}
-#else
-bool fixed_planes_real(chebfi_ctx* ctx, int64_t nb, const double2* T, double2* out, cudaStream_t st) {
-  switch (ctx->grid[0]) {
-#define CHEBFI_X(n) \
-  case n: real_launch_fx<n>(ctx, nb, T, out, st); return true;
-    CHEBFI_FFT_DF_SIZES(CHEBFI_X)
 #undef CHEBFI_X
     default: return false;
   }

@@ -231,3 +231,51 @@ def test_vloc_gradient_on_every_kind_of_grid(n):
     # two transforms of log2(n^3) levels and the product, each about 2^-52 of its norm
     bound = 64.0 * 2.0 ** -52 * sum(np.linalg.norm(G[:, j]) * np.linalg.norm(Y[:, j]) for j in range(5)) / n ** 1.5
     assert np.linalg.norm(_np(gV) - ref) <= bound
+
+
+# fixed-point planes between FP64 z passes (the compiled lengths without double-float passes)
+# against the oracle and against the FP64 units, over FP64's range of scales
+@pytest.mark.parametrize("n", [16, 20, 30, 36, 40, 45, 54, 60, 80, 90, 100, 108])
+@pytest.mark.parametrize("kind", ["plain", "tiny", "huge", "spike"])
+def test_fixed_point_planes_between_fp64_passes(n, kind):
+    L = 0.42 * n
+    ecut = 0.5 * (2.0 * np.pi / L * 0.23 * n) ** 2
+    cell = make_cell(L, n, ecut, 1, 8, 6, False, 40, kpt=(0.02, -0.05, 0.03))
+    cell.D = np.zeros_like(cell.D)
+    V = cell.vloc * {"plain": 1.0, "tiny": 1e-12, "huge": 1e9, "spike": 0.0}[kind]
+    if kind == "spike":
+        V[n // 3, n // 5, n // 2] = -7.0
+    cell.vloc = V
+    Y = cell.Y0.copy()
+    Y[:, 1] *= 1e150
+    Y[:, 2] *= 1e-150
+    Y[:, 3] = 0.0
+    Y[:, 4] = 0.0
+    Y[cell.npw // 2, 4] = 1.0
+    Y[:, 5] = 1.0
+    ref = PWOperator.from_cell(cell).apply_H(Y)
+    g = _ctx(cell)
+    got = _np(g.apply_H(_F(Y)))
+    g.set_fft64(0)
+    native = _np(g.apply_H(_F(Y)))
+    # two transforms of log2(n^3) <= 21 levels and the product, each about 2^-52 of its norm;
+    # norms by the largest component first, as 1e-150 squared is zero
+    size = np.abs(Y).max(axis=0)
+    size[3] = 1.0
+    norm = np.linalg.norm(Y / size, axis=0)
+    tol = 64.0 * 2.0 ** -52 * (np.abs(V).max() + ecut) * norm
+    assert np.all(np.linalg.norm((got - ref) / size, axis=0) <= tol)
+    assert np.all(np.linalg.norm((got - native) / size, axis=0) <= tol)
+    assert np.all(got[:, 3] == 0.0)
+
+
+def test_non_finite_bands_stay_apart_between_fp64_passes():
+    cell = make_cell(10.0, 30, 6.0, 1, 8, 4, False, 37)
+    Y = cell.Y0.copy()
+    Y[5, 1] = np.nan
+    Y[7, 2] = np.inf
+    g = _ctx(cell)
+    got = _np(g.apply_H(_F(Y)))
+    good = _np(g.apply_H(_F(cell.Y0)))
+    assert np.isnan(got[:, 1]).all() and np.isnan(got[:, 2]).all()
+    assert np.array_equal(got[:, [0, 3]], good[:, [0, 3]])
