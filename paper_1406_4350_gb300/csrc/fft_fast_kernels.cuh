@@ -150,6 +150,19 @@ __device__ __forceinline__ void zinv_body(const cplx<typename SphT<R>::type>* __
 // rows of a plane are an odd pitch apart: the row-wise passes meet no bank conflicts
 constexpr int plane_pitch(int n) { return n % 2 ? n : n + 1; }
 
+// The row of the i-th group of NB items in the y passes A, whose thread items (group, nb) touch
+// row P + nb.  Rows are an odd number of elements long, so with consecutive rows the banks of
+// neighbouring groups overlap, two to four wavefronts an access; rows chosen so that row P =
+// NB i (mod G), G elements covering the banks once, make a warp's addresses consecutive modulo
+// G.  A permutation of each full G rows; the rest keep their order.  FP32, 512 bands, before
+// and now: 32^3 0.0825 -> 0.0758 ms, 48^3 0.2076 -> 0.2009, 64^3 0.453 -> 0.438; 256 bands at
+// 96^3 0.802 -> 0.783 (at 24^3 and 90^3 no difference).
+template <int N, int G> __device__ __forceinline__ int row_of_group(int i, int full) {
+  constexpr int NB = fast::Plan<N>::NB, g = fast::gcd(NB, G), c = NB * fast::inv_mod(plane_pitch(N) % G, G) % G;
+  constexpr int per = G / g;  // distinct values of c i mod G, all multiples of g
+  return i < full ? i / G * G + (c * i % G + (i / per) % g) : i;
+}
+
 // Plane z of block b: inverse y and x transforms, multiply by V_loc, forward x and y, its
 // zero rows pruned and its scatter / gather fused:
 // the first y pass reads the sphere columns straight from the column buffer (no zeroed
@@ -163,11 +176,11 @@ constexpr int plane_pitch(int n) { return n % 2 ? n : n + 1; }
 template <typename R, int N, int NT>
 __device__ __forceinline__ void inverse_passes(const cplx<R>* __restrict__ t, const FastArgs& fa, cplx<R>* plane) {
   using C = cplx<R>;
-  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N), W = NT / 32;
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N), W = NT / 32, G = 128 / (int)sizeof(C);
   constexpr bool kWarpNb = N % 32 == 0 && W % NB == 0;
   const ConstTw<R, N> tw;
   const C zero = cmake<C>(0.0, 0.0);
-  const int nl = fa.nact, lo = fa.act_lo;
+  const int nl = fa.nact, lo = fa.act_lo, full = nl / G * G;
   C* rows = plane + lo * P;  // row a of the active range
   // y, inverse: F's pass A on the active rows, its inputs read from the column buffer;
   // consecutive threads take consecutive y of one row, so they read consecutive columns
@@ -179,7 +192,7 @@ __device__ __forceinline__ void inverse_passes(const cplx<R>* __restrict__ t, co
 #pragma unroll
     for (int ka = 1; ka < NA; ++ka) w[ka] = fast::twN<+1>(tw, nb * ka);
     for (int it = threadIdx.x; it < nl * NB; it += blockDim.x) {
-      const int a = it / NB;
+      const int a = row_of_group<N, G>(it / NB, full);
       C* row = rows + a * P + nb;
       const int32_t* rc = fa.row_col + a * N + nb;
       C v[NA];
@@ -196,7 +209,7 @@ __device__ __forceinline__ void inverse_passes(const cplx<R>* __restrict__ t, co
   } else {
     // NB = 6 with a 256-thread block: an item's nb and twiddles are its own
     for (int it = threadIdx.x; it < nl * NB; it += blockDim.x) {
-      const int a = it / NB, nb = it - a * NB;
+      const int i = it / NB, nb = it - i * NB, a = row_of_group<N, G>(i, full);
       C* row = rows + a * P + nb;
       const int32_t* rc = fa.row_col + a * N + nb;
       C v[NA];
@@ -261,12 +274,12 @@ template <typename R, int N, int NT = kThreadsF>
 __device__ __forceinline__ void plane_body_pruned(cplx<R>* __restrict__ T, const R* __restrict__ Vs,
                                                   const FastArgs& fa, int z, int64_t b, unsigned char* smem_raw) {
   using C = cplx<R>;
-  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N), W = NT / 32;
+  constexpr int NA = fast::Plan<N>::NA, NB = fast::Plan<N>::NB, P = plane_pitch(N), W = NT / 32, G = 128 / (int)sizeof(C);
   constexpr bool kWarpNb = N % 32 == 0 && W % NB == 0;
   const ConstTw<R, N> tw;
   C* plane = reinterpret_cast<C*>(smem_raw);
   C* t = T + b * fa.ldt + (int64_t)z * fa.ncolp;
-  const int nl = fa.nact, lo = fa.act_lo;
+  const int nl = fa.nact, lo = fa.act_lo, full = nl / G * G;
   C* rows = plane + lo * P;  // row a of the active range
   inverse_passes<R, N, NT>(t, fa, plane);
   {
@@ -333,7 +346,7 @@ __device__ __forceinline__ void plane_body_pruned(cplx<R>* __restrict__ T, const
   }
   __syncthreads();
   for (int it = threadIdx.x; it < nl * NB; it += blockDim.x) {
-    const int a = it / NB, nb = it - a * NB;  // consecutive columns per warp, as above
+    const int i = it / NB, nb = it - i * NB, a = row_of_group<N, G>(i, full);  // consecutive columns, as above
     const C* row = rows + a * P + nb;
     const int32_t* rc = fa.row_col + a * N + nb;
     C v[NA];

@@ -25,10 +25,19 @@ __global__ void __launch_bounds__(kThreads) k_zinv_f(const cplx<typename SphT<R>
   fk::zinv_body<R, N3>(Y, ldy, T, fa, twz, blockIdx.x * kCBF, blockIdx.y, smem_raw);
 }
 
+// Threads of an FP32 plane's block, measured over 64 to 768 per length: small planes run in
+// small blocks, whose barriers more of their neighbours fill (32^3, 512 bands: 128 threads
+// 0.070 ms, 256 0.076; 64^3: 0.425 and 0.438); above 96 only two planes fit an SM, and it
+// takes 512 threads each to fill it (100^3, 256 bands: 1.02 and 1.13 ms).  At 48 to 96 other
+// counts are slower (48^3: 128 0.205, 256 0.201, 384 0.246 ms; 96^3: 192-384 0.79-0.81, 256
+// 0.783, 512 0.89).
+template <typename R, int N> constexpr int plane_threads() {
+  return sizeof(R) != 4 ? kThreads : N < 48 || N == 64 ? 128 : N > 96 ? 512 : 256;
+}
 template <typename R, int N>
-__global__ void __launch_bounds__(kThreads) k_plane_f(cplx<R>* __restrict__ T, const R* __restrict__ Vs, FastArgs fa) {
+__global__ void __launch_bounds__(plane_threads<R, N>()) k_plane_f(cplx<R>* __restrict__ T, const R* __restrict__ Vs, FastArgs fa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fk::plane_body_pruned<R, N, kThreads>(T, Vs, fa, blockIdx.x, blockIdx.y, smem_raw);
+  fk::plane_body_pruned<R, N, plane_threads<R, N>()>(T, Vs, fa, blockIdx.x, blockIdx.y, smem_raw);
 }
 
 #ifndef CHEBFI_FFT_DF
@@ -81,7 +90,7 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
     CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
     if (!fixed_planes(ctx, nbc, T, st)) {
 #ifndef CHEBFI_FFT_DF
-      CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col, k_plane_f<R, N><<<dim3(N, nbc), kThreads, pbytes, st>>>(T, vtable<R>(ctx), fa));
+      CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col, k_plane_f<R, N><<<dim3(N, nbc), plane_threads<R, N>(), pbytes, st>>>(T, vtable<R>(ctx), fa));
 #else
       CHEBFI_REQUIRE(false, CHEBFI_ERR_STATE, "double-float columns without fixed-point planes");
 #endif
