@@ -3,6 +3,8 @@
 // arithmetic R.
 #pragma once
 
+#include <type_traits>
+
 #include "fft_launch.cuh"
 
 namespace chebfi {
@@ -15,11 +17,25 @@ constexpr int kThreads = 256;
 using fk::FastArgs;
 using fk::kCBF;
 
+// Threads of a z pass's block (kCBF lines): its two transform passes have kCBF NB and kCBF NA
+// items, mostly fewer than 256, so smaller blocks leave fewer threads idle at their barriers;
+// measured with 64, 128, 192 and 256 (ms for 512 bands; 256 threads and the choice).  Inverse:
+// FP32 60^3 0.070 and 0.065, 80^3 0.164 and 0.145, double-float 72^3 0.424 and 0.356, 96^3 0.974
+// and 0.907.  Forward, whose epilogue wants more loads in flight: FP32 60^3 0.089 and 0.079,
+// double-float 72^3 0.493 and 0.431, but FP32 64^3 0.080 with 256 and 0.088 with 128.
+// The FP64 units bind theirs whatever the block (36^3: 0.152 ms with 256, 0.157 with 128).
+template <typename R, int N> constexpr int zinv_threads() {
+  return std::is_same<R, double>::value ? kThreads : N < 96 ? 128 : 192;
+}
+template <typename R, int N> constexpr int zfwd_threads() {
+  return std::is_same<R, dfl>::value ? (N < 96 ? 128 : 192) : std::is_same<R, float>::value && N < 64 ? 128 : kThreads;
+}
+
 // R: the arithmetic of the transforms (float, double, or dfl, the double-float form of the
 // FP64 path); blocks, the kinetic diagonal and the epilogue's operands are stored in
 // SphT<R> (double for dfl), the column buffer and the planes in cplx<R>.
 template <typename R, int N3>
-__global__ void __launch_bounds__(kThreads) k_zinv_f(const cplx<typename SphT<R>::type>* __restrict__ Y, int64_t ldy,
+__global__ void __launch_bounds__(zinv_threads<R, N3>()) k_zinv_f(const cplx<typename SphT<R>::type>* __restrict__ Y, int64_t ldy,
                                                      cplx<R>* __restrict__ T, FastArgs fa, const cplx<R>* __restrict__ twz) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fk::zinv_body<R, N3>(Y, ldy, T, fa, twz, blockIdx.x * kCBF, blockIdx.y, smem_raw);
@@ -51,7 +67,7 @@ __global__ void __launch_bounds__(kThreads) k_plane_real_f(const cplx<R>* __rest
 #endif
 
 template <typename R, int N3>
-__global__ void __launch_bounds__(kThreads) k_zfwd_f(const cplx<R>* __restrict__ T, FastArgs fa,
+__global__ void __launch_bounds__(zfwd_threads<R, N3>()) k_zfwd_f(const cplx<R>* __restrict__ T, FastArgs fa,
                                                      const cplx<R>* __restrict__ twz,
                                                      const typename SphT<R>::type* __restrict__ K,
                                                      LocalEpi<typename SphT<R>::type> ep) {
@@ -87,7 +103,7 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
     const int nbc = (int)std::min<int64_t>(65535, nb - b0);
     dim3 gz((s.ncol + kCBF - 1) / kCBF, nbc);
     const double esz = sizeof(cplx<R>), col = (double)N * s.ncol * nbc * esz, sph = (double)ctx->npw * nbc * esz;
-    CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
+    CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, zinv_threads<R, N>(), zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
     if (!fixed_planes(ctx, nbc, T, st)) {
 #ifndef CHEBFI_FFT_DF
       CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col, k_plane_f<R, N><<<dim3(N, nbc), plane_threads<R, N>(), pbytes, st>>>(T, vtable<R>(ctx), fa));
@@ -107,7 +123,7 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
     e.inv_n3 = (S)(1.0 / ((double)N * N * N));
     const double epi = sph * (1.0 + (e.Z ? 1.0 : 0.0) + (e.T ? 1.0 : 0.0) + (e.Yprev ? 1.0 : 0.0)) +
                        (e.Zhi ? (double)ctx->npw * nbc * (e.zplane ? 12.0 : 8.0) : 0.0);
-    CHEBFI_LAUNCH_W("k_zfwd", st, col + epi, k_zfwd_f<R, N><<<gz, kThreads, zbytes, st>>>(T, fa, tw, K, e));
+    CHEBFI_LAUNCH_W("k_zfwd", st, col + epi, k_zfwd_f<R, N><<<gz, zfwd_threads<R, N>(), zbytes, st>>>(T, fa, tw, K, e));
   }
 }
 
@@ -123,7 +139,7 @@ void real_launch(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cpl
   fk::init_twiddles();
   set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
   const dim3 gz((s.ncol + kCBF - 1) / kCBF, (unsigned)nb);
-  CHEBFI_LAUNCH("k_zinv", st, k_zinv_f<R, N><<<gz, kThreads, zbytes, st>>>(Y, ldy, T, fa, tw));
+  CHEBFI_LAUNCH("k_zinv", st, k_zinv_f<R, N><<<gz, zinv_threads<R, N>(), zbytes, st>>>(Y, ldy, T, fa, tw));
   if (!planes) return;
   set_smem<R>((const void*)k_plane_real_f<R, N>, pbytes);
   CHEBFI_LAUNCH("k_plane_real", st, k_plane_real_f<R, N><<<dim3(N, (unsigned)nb), kThreads, pbytes, st>>>(T, out, fa));
