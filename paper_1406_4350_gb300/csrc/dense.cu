@@ -30,8 +30,10 @@ __device__ __forceinline__ void flag_error(int* status, int code) {
 // Unblocked Cholesky of one nb x nb diagonal block (nb <= NB) in shared memory.  One block:
 // the pivots are a serial chain, and GB300's FP64 unit (about two FMAs per clock) makes each
 // square root and division ~10 dependent slow instructions.  Only 1 / sqrt(d) is on the
-// chain (the column is scaled by it); the diagonal's sqrt(d) is another warp's work
-// (32 x 32: 66 us with sqrt and a division per entry on the chain, now 39 us).
+// chain (the column is scaled by it), and one warp forms the next column's while the others
+// update the trailing triangle; the diagonal's square roots are taken together at the end
+// (32 x 32: 66 us with sqrt and a division per entry on the chain, 39 us with the reciprocal
+// root between barriers, now 31 us).
 __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int nb, int* status) {
   __shared__ double2 a[NB][NB + 1];
   __shared__ double rpiv;
@@ -41,17 +43,19 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
     a[i][j] = A[i + j * lda];
   }
   __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    const double d0 = a[j][j].x;
-    const double d = d0 > 0.0 ? d0 : 1.0;  // also catches NaN
-    if (tid == 0) {
-      if (!(d0 > 0.0)) flag_error(status, CHEBFI_ERR_NOT_SPD);
-      rpiv = rsqrt(d);
+  auto pivot = [&](int j) {  // by one thread; a pivot that is not positive (or NaN) counts as 1
+    const double d = a[j][j].x;
+    if (!(d > 0.0)) {
+      flag_error(status, CHEBFI_ERR_NOT_SPD);
+      a[j][j].x = 1.0;
     }
-    const double piv = tid == 32 ? sqrt(d) : 0.0;
-    __syncthreads();
-    if (tid == 32) a[j][j] = make_double2(piv, 0.0);
-    for (int i = j + 1 + tid; i < nb; i += blockDim.x) {
+    rpiv = rsqrt(a[j][j].x);
+  };
+  if (tid == 0) pivot(0);
+  __syncthreads();
+  for (int j = 0; j < nb; ++j) {
+    const int i = j + 1 + tid;
+    if (i < nb) {
       a[i][j].x *= rpiv;
       a[i][j].y *= rpiv;
     }
@@ -60,11 +64,7 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
     // Its m columns are folded in pairs (q, m - 1 - q) of m + 1 entries together, so that no
     // lane of the slow FP64 instructions is spent above the diagonal.
     const int m = nb - j - 1;
-    for (int e = tid; e < (m + 1) * ((m + 1) / 2); e += blockDim.x) {
-      const int q = e / (m + 1), c = e - q * (m + 1);
-      const bool first = c < m - q;
-      if (!first && m - 1 - q == q) continue;  // the middle column of an odd m has no partner
-      const int k = j + 1 + (first ? q : m - 1 - q), i = first ? k + c : k + c - (m - q);
+    auto update = [&](int i, int k) {
       const double2 li = a[i][j], lk = a[k][j];
       double2 v = a[i][k];
       v.x = fma(-li.x, lk.x, v.x);
@@ -72,12 +72,27 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
       v.x = fma(-li.y, lk.y, v.x);
       v.y = fma(li.x, lk.y, v.y);
       a[i][k] = v;
+    };
+    if (tid < 32) {
+      if (tid == 0 && m > 0) {
+        const double2 l = a[j + 1][j];  // the diagonal is real
+        a[j + 1][j + 1].x = fma(-l.y, l.y, fma(-l.x, l.x, a[j + 1][j + 1].x));
+        pivot(j + 1);
+      }
+    } else {
+      for (int e = tid - 32; e < (m + 1) * ((m + 1) / 2); e += blockDim.x - 32) {
+        const int q = e / (m + 1), c = e - q * (m + 1);
+        const bool first = c < m - q;
+        if (!first && m - 1 - q == q) continue;  // the middle column of an odd m has no partner
+        const int k = j + 1 + (first ? q : m - 1 - q), i = first ? k + c : k + c - (m - q);
+        if (i != j + 1) update(i, k);  // (j + 1, j + 1) is the next pivot
+      }
     }
     __syncthreads();
   }
   for (int e = tid; e < nb * nb; e += blockDim.x) {
     const int i = e % nb, j = e / nb;
-    A[i + j * lda] = i >= j ? a[i][j] : make_double2(0.0, 0.0);
+    A[i + j * lda] = i > j ? a[i][j] : make_double2(i == j ? sqrt(a[i][j].x) : 0.0, 0.0);
   }
 }
 
