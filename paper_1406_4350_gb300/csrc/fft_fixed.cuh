@@ -319,7 +319,7 @@ __device__ __forceinline__ double to_double(ll v, int s) {
   const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
   const int lz = __clzll((ll)u), e = 63 - lz - s;
   if (u == 0 || e < -1022) return 0.0;
-  if (e > 1022) return v < 0 ? -INFINITY : INFINITY;  // (the last binade goes with it)
+  if (e > 1023) return v < 0 ? -INFINITY : INFINITY;
   const unsigned long long m = u << lz;  // leading one at bit 63
   // the implicit bit and the rounding carry add into the exponent field
   const ll bits = ((ll)(e + 1022) << 52) + (ll)((m >> 11) + ((m >> 10) & 1));
