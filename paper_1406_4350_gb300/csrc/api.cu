@@ -1423,6 +1423,7 @@ int chebfi_set_vloc(chebfi_ctx* ctx, const double* vloc, int on_device) {
   ctx->d_vtf.upload(tf.data(), n);
   ctx->fast_fft = fast_fft_supported(n1, n2, n3);
   if (ctx->fast_fft) {
+    fill_fft_tables();
     // position (z', x', y') of the two-pass kernels holds real-space point
     // (split_index(x'), split_index(y'), split_index(z'))
     std::vector<double> vs(n);

@@ -834,6 +834,9 @@ void autotune(chebfi_batch* bt, cudaStream_t st) {
   cudaEventDestroy(b);
 }
 
+// the passes' twiddles, for the batches of every context of a device
+fk::OncePerDevice g_tables;
+
 // mixed: the FP32 form with the projector products on the tensor cores (R = float only)
 template <typename R>
 void batch_filter(chebfi_batch* bt, void* const* Y, const int64_t* ld, int degree, const double* lo, const double* hi,
@@ -843,7 +846,6 @@ void batch_filter(chebfi_batch* bt, void* const* Y, const int64_t* ld, int degre
   else autotune<R>(bt, st);
   ensure_ws<R>(bt);
   set_fft_smem_n<R>(bt);
-  fk::init_twiddles();
   // per-call descriptor fields
   auto& h = BatchOps<R>::hdesc(bt);
   for (int k = 0; k < bt->nk; ++k) {
@@ -1015,6 +1017,7 @@ int chebfi_batch_create(chebfi_batch** out, chebfi_ctx* const* kctx, int nk, int
     bt->d64.upload(bt->h64.data(), nk);
     bt->d32.upload(bt->h32.data(), nk);
     bt->counters.alloc(8 * 1001 + 8);
+    g_tables(fk::fill_twiddles);
     int dev = 0;
     CHEBFI_CUDA(cudaGetDevice(&dev));
     CHEBFI_CUDA(cudaDeviceGetAttribute(&bt->nsm, cudaDevAttrMultiProcessorCount, dev));

@@ -253,6 +253,13 @@ bool fast_apply(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx
   return fast_dispatch<R>(ctx, Y, ldy, nb, T, ep, st, K);
 }
 
+void fill_fft_tables() {
+  fft_tables<float>();
+  fft_tables<double>();
+  fft_tables<dfl>();
+  fixed_tables();
+}
+
 bool fast_fft_supported(int n1, int n2, int n3) {
   if (n1 != n2 || n1 != n3) return false;
   switch (n1) {

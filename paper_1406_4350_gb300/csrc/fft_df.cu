@@ -3,6 +3,7 @@
 #include "fft_launch_impl.cuh"
 
 namespace chebfi {
+template void fft_tables<dfl>();
 template bool fast_dispatch<dfl>(chebfi_ctx*, const cplx<double>*, int64_t, int64_t, cplx<dfl>*, LocalEpi<double>, cudaStream_t,
                                 const double*);
 }  // namespace chebfi

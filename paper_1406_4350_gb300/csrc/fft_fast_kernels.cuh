@@ -12,6 +12,8 @@
 #include <cuda_bf16.h>
 
 #include <cmath>
+#include <mutex>
+#include <set>
 #include <vector>
 
 #include "dfloat.cuh"
@@ -60,7 +62,8 @@ inline FastArgs fast_args(const chebfi_ctx* ctx) {
 // Twiddle tables tw[e] = exp(-2 pi i e / N) of the compiled line lengths, in constant memory:
 // a warp of a pass reads one entry (two where it straddles two sub-transforms), which the
 // constant cache broadcasts without using the shared-memory pipe that bounds these kernels.
-// Each translation unit has its own copy, filled by init_twiddles before its first launch.
+// Each translation unit has its own copy, filled by fft_tables (fft_launch.cuh) when a context
+// takes a potential on a compiled grid, before any launch.
 #define CHEBFI_X(n) n,
 constexpr int kTwLens[] = {CHEBFI_FFT_SIZES(CHEBFI_X)};
 #undef CHEBFI_X
@@ -92,13 +95,27 @@ template <int N> struct ConstTw<dfl, N> {
   }
 };
 
-// Fill this translation unit's tables on the current device (once per device; not inside a
-// stream capture).
-static inline void init_twiddles() {
-  static bool done[64] = {false};
-  int dev = 0;
-  CHEBFI_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64 || done[dev]) return;
+// Runs fill once per device and waits for the copies that it starts: the tables are read on any
+// stream, also on one that is not ordered after the stream of the copies, and a copy from
+// pageable memory may return before it has arrived.  One per set of tables.
+class OncePerDevice {
+  std::mutex mu;
+  std::set<int> done;
+
+ public:
+  template <typename F> void operator()(F fill) {
+    int dev = 0;
+    CHEBFI_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count(dev)) return;
+    fill();
+    CHEBFI_CUDA(cudaDeviceSynchronize());
+    done.insert(dev);
+  }
+};
+
+// Copies this translation unit's tables to the current device.
+static inline void fill_twiddles() {
   std::vector<float2> f;
   std::vector<double2> d;
   std::vector<float4> df;
@@ -113,7 +130,6 @@ static inline void init_twiddles() {
   CHEBFI_CUDA(cudaMemcpyToSymbol(c_twf, f.data(), sizeof(float2) * f.size()));
   CHEBFI_CUDA(cudaMemcpyToSymbol(c_twd, d.data(), sizeof(double2) * d.size()));
   CHEBFI_CUDA(cudaMemcpyToSymbol(c_twdf, df.data(), sizeof(float4) * df.size()));
-  done[dev] = true;
 }
 
 // sphere block b, columns [c0, c0 + kCBF) -> inverse z transform -> column buffer T

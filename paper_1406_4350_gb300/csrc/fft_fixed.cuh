@@ -229,19 +229,15 @@ constexpr int pre_shift(int b8, int n) {
 constexpr int pass_bits(int n) { return (kTop8 - grow8(n)) / 8; }
 constexpr int after(int b8, int n) { return b8 - 8 * pre_shift(b8, n) + grow8(n); }
 
-// Twiddles (cos, -sin)(2 pi e / N) of the compiled lengths as (c.h, c.l, s.h, s.l); filled by
-// init_twiddles before a translation unit's first launch.
+// Twiddles (cos, -sin)(2 pi e / N) of the compiled lengths as (c.h, c.l, s.h, s.l); filled as
+// the other passes' tables are (fft_fast_kernels.cuh).
 static __constant__ int4 c_twfx[fk::kTwTotal];
 template <int N, int SIGN> __device__ __forceinline__ void twiddle(int e, Cst& c, Cst& s) {
   const int4 w = c_twfx[fk::TwOff<N>::v + e];
   c = Cst{w.x, w.y};
   s = SIGN > 0 ? Cst{-w.z, -w.w} : Cst{w.z, w.w};
 }
-static inline void init_twiddles() {
-  static bool done[64] = {false};
-  int dev = 0;
-  CHEBFI_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64 || done[dev]) return;
+static inline void fill_twiddles() {
   std::vector<int4> t;
   for (int n : fk::kTwLens)
     for (int k = 0; k < n; ++k) {
@@ -259,7 +255,6 @@ static inline void init_twiddles() {
       t.push_back(make_int4(c.first, c.second, s.first, s.second));
     }
   CHEBFI_CUDA(cudaMemcpyToSymbol(c_twfx, t.data(), sizeof(int4) * t.size()));
-  done[dev] = true;
 }
 
 // 2^e as a float, |e| <= 126

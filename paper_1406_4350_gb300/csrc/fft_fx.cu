@@ -28,7 +28,6 @@ __global__ void __launch_bounds__(fx_threads<N>()) k_plane_real_fx(const double2
 template <int N> size_t prepare(const chebfi_ctx* ctx, const void* kernel) {
   CHEBFI_REQUIRE(ctx->sph.pitch == fk::plane_pitch(N), CHEBFI_ERR_STATE, "plane pitch of the compile-time path");
   const size_t bytes = (size_t)(N * fk::plane_pitch(N)) * sizeof(fx::cfx);
-  fx::init_twiddles();
   CHEBFI_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
   return bytes;
 }
@@ -47,6 +46,11 @@ template <int N> void launch_real(chebfi_ctx* ctx, int64_t nb, const double2* T,
 }
 
 }  // namespace
+
+void fixed_tables() {
+  static fk::OncePerDevice once;
+  once(fx::fill_twiddles);
+}
 
 bool fixed_planes(chebfi_ctx* ctx, int64_t nb, cdf* T, cudaStream_t st) {
   switch (ctx->grid[0]) {

@@ -10,6 +10,12 @@
 
 namespace chebfi {
 
+// The constant tables of the compiled passes on the current device: filled once per device and
+// complete on return.  A context fills them when it takes a potential on a compiled grid, so
+// that its launches, which may be inside a stream capture, have nothing to set up.
+template <typename R> void fft_tables();
+void fixed_tables();
+
 // (K + V_loc) with the compiled kernels of the context's grid; false if its size has none
 template <typename R>
 bool fast_dispatch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t ldy, int64_t nb, cplx<R>* T,

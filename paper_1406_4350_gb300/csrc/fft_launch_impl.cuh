@@ -93,7 +93,6 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
   const cplx<R>* tw = nullptr;  // the passes read their twiddles from constant tables
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
   const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
-  fk::init_twiddles();
 #ifndef CHEBFI_FFT_DF
   set_smem<R>((const void*)k_plane_f<R, N>, pbytes);
 #endif
@@ -136,7 +135,6 @@ void real_launch(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cpl
   CHEBFI_REQUIRE(nb <= 65535, CHEBFI_ERR_ARG, "too many bands in a chunk");
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>), pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
   const cplx<R>* tw = nullptr;
-  fk::init_twiddles();
   set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
   const dim3 gz((s.ncol + kCBF - 1) / kCBF, (unsigned)nb);
   CHEBFI_LAUNCH("k_zinv", st, k_zinv_f<R, N><<<gz, zinv_threads<R, N>(), zbytes, st>>>(Y, ldy, T, fa, tw));
@@ -147,6 +145,11 @@ void real_launch(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cpl
 #endif
 
 }  // namespace
+
+template <typename R> void fft_tables() {
+  static fk::OncePerDevice once;
+  once(fk::fill_twiddles);
+}
 
 // Compile-time-length path for cubic grids of the compiled sizes; false = not taken.
 template <typename R>

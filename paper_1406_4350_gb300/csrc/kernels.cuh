@@ -68,6 +68,8 @@ void block_outer_grad(const chebfi_ctx* ctx, const C* q, const C* p, int64_t ldp
 // the two-pass FFT kernels cover cubic grids of a few compiled sizes; split_index(n, p) is
 // the natural index held at position p of their split order
 bool fast_fft_supported(int n1, int n2, int n3);
+// the constant tables of those passes on the current device (once; complete on return)
+void fill_fft_tables();
 int split_index(int n, int p);
 template <typename R>
 void local_apply(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cplx<R>* T, LocalEpi<R> ep,
