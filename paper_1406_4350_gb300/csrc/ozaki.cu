@@ -762,14 +762,17 @@ int oz_precision_bits(int nmod) {
 void oz_prepare(const double2* X, int64_t ldx, int64_t nrows, int64_t K, bool rows_are_columns, bool conj, int nmod,
                 OzOperand& out, cudaStream_t st) {
   const oz::ModSet& ms = oz::modset(nmod);
-  out.nmod = nmod;
+  out.nmod = 0;  // not prepared until the last launch: a failed allocation must not leave it marked
   out.rows = nrows;
   out.K = K;
   out.ld = (K + 7) / 8 * 8;
   out.pstride = out.rows * out.ld;
   out.res.alloc((size_t)3 * nmod * out.pstride);
   out.shift.alloc((size_t)std::max<int64_t>(nrows, 1));
-  if (nrows == 0 || K == 0) return;
+  if (nrows == 0 || K == 0) {
+    out.nmod = nmod;
+    return;
+  }
   if (rows_are_columns && K <= 2048) {
     const int nt = (int)std::min<int64_t>(256, (K + 127) / 128 * 32);
     auto prep = [&](auto kernel) {
@@ -792,6 +795,7 @@ void oz_prepare(const double2* X, int64_t ldx, int64_t nrows, int64_t K, bool ro
                   oz::k_oz_res_rows<<<dim3((unsigned)((nrows + 31) / 32), (unsigned)((K + 63) / 64)), 256, 0, st>>>(
                       nrows, K, X, ldx, out.shift.p, conj ? 1 : 0, nmod, out.res.p, out.pstride, out.ld));
   }
+  out.nmod = nmod;
 }
 
 namespace {
