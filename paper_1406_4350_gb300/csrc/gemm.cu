@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256, TN == 4 ? 3 : 4)
 #pragma unroll
     for (int a = 0; a < TM; ++a) {
       const int64_t gi = i0 + gt::row_of<float>(tx, a);
-      if (gi >= M) continue;
+      if (gi >= M || (lower && gi < gj)) continue;
       float2 r = make_float2(alpha * accr[a][b], alpha * acci[a][b]);
       if (ws) {
         ws[(int64_t)blockIdx.z * M * N + gi + gj * M] = r;
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(256) k_gemm_d(int64_t M, int64_t N, int64_t K,
     __syncthreads();
   }
   const int64_t gi = i0 + tx, gj = j0 + ty;
-  if (gi >= M || gj >= N) return;
+  if (gi >= M || gj >= N || (lower && gi < gj)) return;
   double2 r = make_double2(alpha * re, alpha * im);
   if (ws) {
     ws[(int64_t)blockIdx.z * M * N + gi + gj * M] = r;
@@ -132,17 +132,19 @@ __global__ void __launch_bounds__(256) k_gemm_d(int64_t M, int64_t N, int64_t K,
   Cm[gi + gj * ldc] = r;
 }
 
-// C = sum_z ws[z] + beta C.  32 outputs per block; eight threads per output each add every
+// C = sum_z ws[z] + beta C (lower: of the entries on and below the diagonal, the only ones that
+// the products left in ws).  32 outputs per block; eight threads per output each add every
 // eighth split, their partial sums are added in a fixed order: one thread per output is a
 // chain of up to 64 dependent loads and slow FP64 additions (16 us at 64 splits of 8 x 32, now 8 us).
 template <typename R>
 __global__ void __launch_bounds__(256) k_splitk_reduce(int64_t M, int64_t N, int splits, const cplx<R>* __restrict__ ws,
-                                                       R beta, cplx<R>* __restrict__ Cm, int64_t ldc) {
+                                                       R beta, cplx<R>* __restrict__ Cm, int64_t ldc, int lower) {
   __shared__ cplx<R> part[8][33];
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   const int64_t idx = (int64_t)blockIdx.x * 32 + tx;
+  const bool in = idx < M * N && !(lower && idx % M < idx / M);
   cplx<R> r = cmake<cplx<R>>(0.0, 0.0);
-  if (idx < M * N) {
+  if (in) {
 #pragma unroll 4
     for (int z = ty; z < splits; z += 8) {
       const cplx<R> v = ws[(int64_t)z * M * N + idx];
@@ -152,7 +154,7 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(int64_t M, int64_t N, int
   }
   part[ty][tx] = r;
   __syncthreads();
-  if (ty != 0 || idx >= M * N) return;
+  if (ty != 0 || !in) return;
 #pragma unroll
   for (int z = 1; z < 8; ++z) {
     r.x += part[z][tx].x;
@@ -207,7 +209,7 @@ void launch_f(int64_t M, int64_t N, int64_t K, double alpha, const float2* A, in
   if (splits > 1) {
     const int64_t tot = M * N;
     CHEBFI_LAUNCH("k_splitk_reduce", st,
-                  k_splitk_reduce<float><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, (int)splits, wsp, (float)beta, Cm, ldc));
+                  k_splitk_reduce<float><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, (int)splits, wsp, (float)beta, Cm, ldc, lower ? 1 : 0));
   }
 }
 
@@ -246,7 +248,7 @@ void launch_d(int64_t M, int64_t N, int64_t K, double alpha, const double2* A, i
   if (splits > 1) {
     const int64_t tot = M * N;
     CHEBFI_LAUNCH("k_splitk_reduce", st,
-                  k_splitk_reduce<double><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, (int)splits, wsp, beta, Cm, ldc));
+                  k_splitk_reduce<double><<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(M, N, (int)splits, wsp, beta, Cm, ldc, lower ? 1 : 0));
   }
 }
 

@@ -79,7 +79,7 @@ void local_apply(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cpl
 // C = alpha op(A) op(B) + beta C, op = identity or conjugate transpose; real alpha, beta.
 // M x N result, inner dimension K.  ws: optional split-K workspace (nullptr = no split).
 // tag: the name the launch is timed under when profiling is on.  lower: square result,
-// only tiles touching the lower triangle are computed (the rest of C is left undefined).
+// only its lower triangle is computed and written.
 template <typename R>
 void gemm(bool conjA, bool conjB, int64_t M, int64_t N, int64_t K, double alpha, const cplx<R>* A,
           int64_t lda, const cplx<R>* B, int64_t ldb, double beta, cplx<R>* C, int64_t ldc, cudaStream_t st,

@@ -14,3 +14,13 @@ needs_nvcc = pytest.mark.skipif(shutil.which("nvcc") is None and not os.path.exi
 def test_operand_without_planes_is_not_marked_prepared(tmp_path):
     [(code, nmod)] = run("operand_alloc_check", tmp_path)
     assert code != 0 and nmod == 0
+
+
+@pytest.mark.gpu
+def test_lower_product_with_split_keeps_the_upper_triangle(tmp_path):
+    rows = run("lower_split_check", tmp_path)
+    assert len(rows) == 8
+    for size, n, k, changed, err in rows:
+        assert changed == 0, (size, n, k)
+        # 2 k + 8 roundings of terms of magnitude one
+        assert err <= (2 * k + 8) * (2.0 ** -53 if size == 8 else 2.0 ** -24), (size, n, k)
