@@ -166,15 +166,14 @@ __device__ __forceinline__ double df_to(dfl a) {
     if (a.h == 0.f) return 0.0;
     return df_to_slow(a);
   }
-  // l in units of h's double ulp, added to h's significand
-  int r = __float2int_rn(a.l * __uint_as_float((unsigned)(127 + 52 - (e - 127)) << 23));
+  // l in units of the sum's double ulp, added to h's significand: h's ulp, or half of it where h
+  // is a power of two and l points to zero (the sum lies below that power; should it round back
+  // to it, the significand's carry moves into the exponent)
+  const int below = (b & 0x7FFFFF) == 0 && (int)(b ^ __float_as_uint(a.l)) < 0 ? 1 : 0;
+  int r = __float2int_rn(a.l * __uint_as_float((unsigned)(127 + 52 + below - (e - 127)) << 23));
   if (b >> 31) r = -r;
-  long long m = ((long long)(b & 0x7FFFFF | 0x800000) << 29) + r;
-  int d = e - 127 + 1022;
-  if (m < (1ll << 52)) {  // below a power of two: one more bit
-    m <<= 1;
-    --d;
-  }
+  const long long m = ((long long)(b & 0x7FFFFF | 0x800000) << (29 + below)) + r;
+  const int d = e - 127 + 1022 - below;
   const long long bits = ((long long)d << 52) + m;  // the implicit bit adds into the exponent
   return __longlong_as_double(bits | (long long)(b & 0x80000000u) << 32);
 }

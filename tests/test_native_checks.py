@@ -24,3 +24,10 @@ def test_lower_product_with_split_keeps_the_upper_triangle(tmp_path):
         assert changed == 0, (size, n, k)
         # 2 k + 8 roundings of terms of magnitude one
         assert err <= (2 * k + 8) * (2.0 ** -53 if size == 8 else 2.0 ** -24), (size, n, k)
+
+
+@pytest.mark.gpu
+def test_double_float_conversions_round_as_the_fp64_unit(tmp_path):
+    [(n, nv, bad, badv)] = run("df_store_check", tmp_path)
+    assert n > 100000 and nv > 100000
+    assert bad == 0 and badv == 0
