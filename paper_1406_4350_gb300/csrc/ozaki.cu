@@ -295,9 +295,47 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // 2-norm of each row of op(X) -> scale exponent s with ||row|| 2^s in [2^(E-1), 2^E);
 // 0 for a zero row, kOzBadShift for a non-finite one (its products come out NaN).
 __device__ __forceinline__ int shift_for(double sumsq, int E) {
-  if (!(sumsq < INFINITY)) return kOzBadShift;  // inf or NaN
-  if (sumsq == 0.0) return 0;
   return E - 1 - (ilogb(sumsq) >> 1);  // floor(log2 sqrt(x)) = floor(floor(log2 x) / 2)
+}
+// Whether the plain sum of squares is as good as it looks: squares below FP64's range have not
+// mattered, none has overflowed.  Other rows (zero, beyond 2^-450 or 2^511, or not finite) are
+// summed again, scaled by their largest component.
+__device__ __forceinline__ bool sum_in_range(double sumsq) { return sumsq >= 0x1p-900 && sumsq < INFINITY; }
+constexpr int kAgain = 0x40000000;  // no shift yet
+__device__ __forceinline__ int exponent_of(double2 v) {
+  return max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF);
+}
+// the power of two that brings components of largest biased exponent e to [1, 2)
+__device__ __forceinline__ double scale_of(int e) { return ldexp(1.0, 1023 - e); }
+__device__ __forceinline__ double add_scaled(double s, double2 v, double f) {
+  const double x = v.x * f, y = v.y * f;
+  return fma(x, x, fma(y, y, s));
+}
+// shift of a row of largest biased exponent e whose scaled squares sum to s
+__device__ __forceinline__ int shift_scaled(int e, double s, int E) {
+  return e == 0x7FF ? kOzBadShift : e == 0 ? 0 : shift_for(s, E) + (1023 - e);  // e = 0: zero or dropped (scaled_int)
+}
+// the scaled sum of a column x of X by the whole block; the result in every thread
+__device__ __noinline__ int column_shift_scaled(const double2* __restrict__ x, int64_t K, int E) {
+  __shared__ int se[32];
+  __shared__ double ss[32];
+  const int tid = threadIdx.x, nw = blockDim.x / 32;
+  int e = 0;
+  for (int64_t k = tid; k < K; k += blockDim.x) e = max(e, exponent_of(x[k]));
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (tid % 32 == 0) se[tid / 32] = e;
+  __syncthreads();
+  for (int i = 0; i < nw; ++i) e = max(e, se[i]);
+  double s = 0.0;
+  const double f = scale_of(e);
+  for (int64_t k = tid; k < K; k += blockDim.x) s = add_scaled(s, x[k], f);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (tid % 32 == 0) ss[tid / 32] = s;
+  __syncthreads();
+  s = 0.0;
+  for (int i = 0; i < nw; ++i) s += ss[i];
+  return shift_scaled(e, s, E);
 }
 
 // rows of op(X) are the columns of X (contiguous): one block per row
@@ -317,7 +355,12 @@ __global__ void k_oz_norm_cols(int64_t nrows, int64_t K, const double2* __restri
     if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
     __syncthreads();
   }
-  if (threadIdx.x == 0) shift[r] = shift_for(red[0], E);
+  if (sum_in_range(red[0])) {
+    if (threadIdx.x == 0) shift[r] = shift_for(red[0], E);
+    return;
+  }
+  const int sh = column_shift_scaled(x, K, E);
+  if (threadIdx.x == 0) shift[r] = sh;
 }
 
 // rows of op(X) are the rows of X (strided): 32 rows per block, eight threads per row
@@ -336,11 +379,34 @@ __global__ void __launch_bounds__(256) k_oz_norm_rows(int64_t nrows, int64_t K, 
   }
   part[ty][tx] = s;
   __syncthreads();
+  bool again = false;
   if (ty == 0 && r < nrows) {
     double t = part[0][tx];
 #pragma unroll
     for (int j = 1; j < 8; ++j) t += part[j][tx];
-    shift[r] = shift_for(t, E);
+    if (sum_in_range(t)) shift[r] = shift_for(t, E);
+    else again = true;
+  }
+  if (!__syncthreads_or(again)) return;
+  // a row of this block is out of range: all of them again
+  __shared__ int pe[8][33];
+  int e = 0;
+  if (r < nrows)
+    for (int64_t k = ty; k < K; k += 8) e = max(e, exponent_of(X[r + k * ldx]));
+  pe[ty][tx] = e;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 8; ++j) e = max(e, pe[j][tx]);
+  const double f = scale_of(e);
+  s = 0.0;
+  if (r < nrows)
+    for (int64_t k = ty; k < K; k += 8) s = add_scaled(s, X[r + k * ldx], f);
+  part[ty][tx] = s;
+  __syncthreads();
+  if (ty == 0 && r < nrows) {
+#pragma unroll
+    for (int j = 1; j < 8; ++j) s += part[j][tx];
+    shift[r] = shift_scaled(e, s, E);
   }
 }
 
@@ -483,13 +549,16 @@ __global__ void __launch_bounds__(256) k_oz_prep_cols(int64_t K, const double2* 
   __syncthreads();
   if (tid == 0) {
     for (int i = 1; i < nt / 32; ++i) s += red[i];
-    shift[r] = s_shift = shift_for(s, E);
+    s_shift = sum_in_range(s) ? shift_for(s, E) : kAgain;
   }
   __syncthreads();
+  int sh = s_shift;
+  if (sh == kAgain) sh = column_shift_scaled(x, K, E);
+  if (tid == 0) shift[r] = sh;
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     const int64_t k = 4 * ((int64_t)g * nt + tid);
-    if (k < K) put_entries(a[g], conj != 0, s_shift, nmod, out, pstride, ld, r, k);
+    if (k < K) put_entries(a[g], conj != 0, sh, nmod, out, pstride, ld, r, k);
   }
 }
 

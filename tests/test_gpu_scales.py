@@ -1,0 +1,65 @@
+"""Results over the range of scales that FP64 has.  Tolerances are the a-priori rounding bounds."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import chebyshev as ch
+from oracle.planewave import PWOperator
+from synth import make_cell
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1406_4350_gb300 import build
+    build.build()
+
+
+def _F(x):
+    from paper_1406_4350_gb300.chebfi import fortran
+    return fortran(x)
+
+
+def _np(t):
+    torch.cuda.synchronize()
+    return t.cpu().numpy()
+
+
+def _ctx(cell=None):
+    from paper_1406_4350_gb300.chebfi import ChebFI
+    return ChebFI.from_cell(cell) if cell is not None else ChebFI(0)
+
+# products that take the modular engine by their size: rows and columns of any scale whose
+# products are representable come out exact (integers times powers of two); every way the
+# operands are read (columns up to 1024 and 2048, longer columns, rows)
+@pytest.mark.parametrize("m,n,k", [(192, 200, 300), (96, 97, 1500), (97, 96, 2100)])
+@pytest.mark.parametrize("conjA,conjB", [(False, False), (True, False), (False, True), (True, True)])
+def test_modular_gemm_at_every_scale(m, n, k, conjA, conjB):
+    rng = np.random.default_rng(m + k)
+    a = rng.integers(-1000, 1001, (2, m, k))
+    b = rng.integers(-1000, 1001, (2, k, n))
+    re, im = a[0] @ b[0] - a[1] @ b[1], a[0] @ b[1] + a[1] @ b[0]
+    ei = rng.integers(-900, 901, m)[:, None]
+    ei[:4, 0] = [-1010, 1000, 505, -505]
+    # columns of the opposite scale, so that products of both signs of exponent are in range
+    fj = rng.integers(-60, 61, n)[None, :]
+    A = (np.ldexp(1.0, ei) * a[0]) + 1j * (np.ldexp(1.0, ei) * a[1])
+    B = (np.ldexp(1.0, fj) * b[0]) + 1j * (np.ldexp(1.0, fj) * b[1])
+    with np.errstate(over="ignore", under="ignore"):
+        ref_re, ref_im = np.ldexp(re.astype(float), ei + fj), np.ldexp(im.astype(float), ei + fj)
+    for flip in (False, True):  # the wide scales on op(A)'s rows, then on op(B)'s columns
+        g = _ctx()
+        if not flip:
+            X, Z, cx, cz = A, B, conjA, conjB
+        else:
+            X, Z, cx, cz = B.T, A.T, conjA, conjB
+        g.profile(True)
+        C = _np(g.gemm_fp64(_F(X.conj().T if cx else X), _F(Z.conj().T if cz else Z), cx, cz))
+        assert "k_oz_gemm" in g.profile_totals()
+        C = C.T if flip else C
+        inside = (ei + fj > -1000) & (ei + fj < 950)  # in FP64's normal range
+        assert np.array_equal(np.where(inside, C.real, 0), np.where(inside, ref_re, 0))
+        assert np.array_equal(np.where(inside, C.imag, 0), np.where(inside, ref_im, 0))
