@@ -720,8 +720,8 @@ void eigh_rr(chebfi_ctx* ctx, int64_t n, double2* A, double* w, double2* X, cuda
     }
   }
   if (!conv) {
-    // stage 1: FP32 Jacobi on a copy; stage 2: refinement from its vectors
-    convert(n, n, A, n, wk.e32a.p, n, st);
+    // stage 1: FP32 Jacobi on a scaled copy; stage 2: refinement from its vectors
+    scaled_to_f32(n, A, wk.e32a.p, reinterpret_cast<int*>(wk.estats.p), st);
     if (jacobi_eigh_f32(n, wk.e32a.p, n, wk.e32b.p, n, st, &wk.small5)) {
       convert(n, n, wk.e32b.p, n, X, n, st);
       Xc = X;

@@ -987,6 +987,26 @@ __global__ void __launch_bounds__(SolveThreads<SS>::v) k_bj_small(int n, const f
   for (int e = threadIdx.x; e < n * n; e += SolveThreads<SS>::v) V[e % n + (e / n) * ldv] = W[e % n + (SS + 1) * (e / n)];
 }
 
+// The largest biased exponent of A's components (A dense, n2 entries), and A times the power of
+// two that brings them below 2 in FP32: the rotations square entries, and a matrix in other units
+// of energy must not lose them to float's range.  A non-finite A stays so.
+__global__ void __launch_bounds__(256) k_bj_exponent(int64_t n2, const double2* __restrict__ A, int* __restrict__ emax) {
+  int e = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x) {
+    const double2 v = A[i];
+    e = max(e, max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF));
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (threadIdx.x % 32 == 0) atomicMax(emax, e);
+}
+__global__ void __launch_bounds__(256) k_bj_scale(int64_t n2, const double2* __restrict__ A, const int* __restrict__ emax,
+                                                  float2* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n2) return;
+  const double f = ldexp(1.0, 1023 - *emax);
+  out[i] = make_float2((float)(A[i].x * f), (float)(A[i].y * f));
+}
+
 // zero-padded copy
 __global__ void k_bj_pad(int64_t n0, int64_t np, const float2* __restrict__ A, int64_t lda, float2* __restrict__ Ap) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1058,7 +1078,14 @@ void jacobi_eigh(int64_t n0, double2* A, int64_t lda, double* w, double2* V, int
   jacobi_eigh_t<double>(n0, A, lda, w, V, ldv, status, st, ws, 1e-15, 1e-12, true);
 }
 
-// The FP32 Jacobi (bj:: kernels) on A (n0 x n0): approximate eigenvectors in V (ld ldv), in
+void scaled_to_f32(int64_t n, const double2* A, float2* out, int* emax, cudaStream_t st) {
+  const int64_t n2 = n * n;
+  CHEBFI_CUDA(cudaMemsetAsync(emax, 0, sizeof(int), st));
+  CHEBFI_LAUNCH("k_bj_scale", st, bj::k_bj_exponent<<<(unsigned)std::min<int64_t>(nblk(n2), 1024), 256, 0, st>>>(n2, A, emax));
+  CHEBFI_LAUNCH("k_bj_scale", st, bj::k_bj_scale<<<nblk(n2), 256, 0, st>>>(n2, A, emax, out));
+}
+
+// The FP32 Jacobi (bj:: kernels) on A (n0 x n0), components below about 2 (scaled_to_f32): approximate eigenvectors in V (ld ldv), in
 // no particular order.  One block for n0 <= 64, the block tournament above.  The matrix is
 // padded with decoupled zero rows and columns, which no rotation touches (a rotation needs a
 // non-zero off-diagonal entry).  False if A is not finite in FP32 (V is not written).

@@ -209,6 +209,9 @@ void trsm_lower(int64_t n, int64_t m, const double2* L, int64_t ldl, double2* B,
 // CHEBFI_ERR_NO_CONVERGENCE on the sweep limit.  Synchronises the stream (sweep test).
 void jacobi_eigh(int64_t n, double2* A, int64_t lda, double* w, double2* V, int64_t ldv, int* status,
                  cudaStream_t st, DevBuf<double2>* ws);
+// A in FP32, scaled by the power of two that brings its largest component to [1, 2) (emax: a device
+// word), as jacobi_eigh_f32 takes it: the eigenvectors do not depend on the scale.
+void scaled_to_f32(int64_t n, const double2* A, float2* out, int* emax, cudaStream_t st);
 // Approximate eigenvectors V of a finite Hermitian A by Jacobi in FP32, to its rounding level
 // and in no particular order (first stage of the refined solver).  False if A is not finite.
 // Synchronises the stream; ws holds its copies and rotations.

@@ -32,6 +32,39 @@ def _ctx(cell=None):
     from paper_1406_4350_gb300.chebfi import ChebFI
     return ChebFI.from_cell(cell) if cell is not None else ChebFI(0)
 
+def _scaled(cell, e):
+    """The cell with its potentials and, for e < 0, its kinetic energies 2^e times as large (e
+    even; for e > 0 a lattice that small is refused, and H is V and D alone)."""
+    f = 2.0 ** (-min(e, 0) // 2)
+    cell.lattice = cell.lattice * f
+    cell.kpt = cell.kpt / f
+    cell.vloc = cell.vloc * 2.0 ** e
+    cell.D = cell.D * 2.0 ** e
+    return cell
+
+
+# one block and the block tournament of the FP32 stage; scales whose squares, and that
+# themselves, pass float's range.  The refinement must converge from that stage.
+@pytest.mark.parametrize("nb", [40, 100])
+@pytest.mark.parametrize("e", [-200, -70, 0, 70, 200])
+def test_rayleigh_ritz_at_every_scale(nb, e):
+    cell = _scaled(make_cell(8.0, 20, 6.0, 2, 8, nb, True, 42), e)
+    op = PWOperator.from_cell(cell)
+    g = _ctx(cell)
+    Y = _F(cell.Y0)
+    ev, rs = g.rayleigh_ritz(Y)
+    w, Yg = _np(ev), _np(Y)
+    assert g.eigensolver_steps >= 1
+    w_ref, _ = ch.rayleigh_ritz(op, cell.Y0)
+    scale = np.abs(w_ref).max()
+    # the Gram matrix's condition number multiplies the rounding of every entry
+    tol = 200.0 * nb * U * np.linalg.cond(cell.Y0.conj().T @ op.apply_S(cell.Y0))
+    np.testing.assert_allclose(w / scale, w_ref / scale, atol=tol)
+    np.testing.assert_allclose(Yg.conj().T @ op.apply_S(Yg), np.eye(nb), atol=tol)
+    np.testing.assert_allclose(Yg.conj().T @ op.apply_H(Yg) / scale, np.diag(w) / scale, atol=tol)
+    np.testing.assert_allclose(_np(rs) / scale, ch.residuals(op, Yg, w) / scale, atol=tol)
+
+
 # products that take the modular engine by their size: rows and columns of any scale whose
 # products are representable come out exact (integers times powers of two); every way the
 # operands are read (columns up to 1024 and 2048, longer columns, rows)
