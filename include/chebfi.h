@@ -323,8 +323,10 @@ int chebfi_gemm_fp64(chebfi_ctx* ctx, int conjA, int conjB, int64_t m, int64_t n
  *    the FP32 units -- each value the unevaluated sum of two floats (48-bit significand,
  *    float's exponent range), the error-free TwoSum / Fast2Sum / FMA-TwoProd transformations
  *    of Knuth and Dekker; a transform keeps about 2^-44 of its line's norm -- and the planes
- *    in 64-bit fixed point, one scale per plane.  On the others but 90 the z passes in FP64
- *    and the planes in fixed point, which together keep FP64's accuracy;
+ *    in 64-bit fixed point, one scale per plane of a band and one per plane of V_loc.  On the
+ *    others but 90 the z passes in FP64 and the planes in fixed point, which together round
+ *    like FP64 relative to a plane's norm (single values far below their plane's largest keep
+ *    fewer bits than FP64 gives them);
  *  CHEBFI_FFT64_NATIVE: FP64 arithmetic on the FP64 units.
  * Blocks, V_loc and the results stay FP64 in memory either way.  Other grids use FP64. */
 enum { CHEBFI_FFT64_NATIVE = 0, CHEBFI_FFT64_DOUBLE_FLOAT = 1 };

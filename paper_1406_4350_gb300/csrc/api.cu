@@ -1436,20 +1436,33 @@ int chebfi_set_vloc(chebfi_ctx* ctx, const double* vloc, int on_device) {
           vs[((size_t)pz * n1 + px) * n2 + py] = v;
           vsf[((size_t)pz * n1 + px) * n2 + py] = (float)v;
         }
-    // |V_loc| < 2^e (1 - 2^-31); both parts are exact roundings of the scaled double
-    double top = 0.0;
-    for (size_t i = 0; i < n; ++i) top = std::max(top, std::fabs(vs[i]));
-    int e = 0;
-    if (top > 0.0) {
-      std::frexp(top, &e);
-      if (top > std::ldexp(1.0 - 1e-9, e)) ++e;
-    }
+    // fixed point, one exponent per plane: |V_loc| < 2^e (1 - 2^-31) on the plane, and the two
+    // parts hold it to 2^(e - 62), so values below 2^-9 of their plane's largest keep fewer than
+    // 53 bits.  One exponent for the grid was not enough: a core 2^6 times the potential in one
+    // plane took bits from all the others (H without its kinetic part, rms error in 2^-53 of
+    // ||V psi|| + ||V|| rms(psi), one exponent / one per plane / FP64 planes: 60^3 2.9 / 1.4 / 0.5,
+    // 108^3 4.8 / 0.6 / 0.7, 96^3 77 / 4.5 with 16 from the z passes when there is no core).
+    // An exponent for every value gives the same errors (60^3 1.3, 96^3 4.5) and costs the FP64
+    // filter 2 %: within a plane the transform rounds relative to the plane's largest anyway.
+    const size_t plane = (size_t)n1 * n2;
     std::vector<int2> vsfx(n);
-    for (size_t i = 0; i < n; ++i) {
-      const double s = std::ldexp(vs[i], 31 - e), h = std::nearbyint(s);
-      vsfx[i] = make_int2((int)h, (int)std::nearbyint((s - h) * 2147483648.0));
+    std::vector<int> vexp(n3);
+    for (int pz = 0; pz < n3; ++pz) {
+      const double* v = vs.data() + pz * plane;
+      double top = 0.0;
+      for (size_t i = 0; i < plane; ++i) top = std::max(top, std::fabs(v[i]));
+      int e = 0;
+      if (top > 0.0) {
+        std::frexp(top, &e);
+        if (top > std::ldexp(1.0 - 1e-9, e)) ++e;
+      }
+      for (size_t i = 0; i < plane; ++i) {
+        const double s = std::ldexp(v[i], 31 - e), h = std::nearbyint(s);
+        vsfx[pz * plane + i] = make_int2((int)h, (int)std::nearbyint((s - h) * 2147483648.0));
+      }
+      vexp[pz] = e;
     }
-    ctx->v_exp = e;
+    ctx->d_vexp.upload(vexp.data(), n3);
     ctx->d_vs.upload(vs.data(), n);
     ctx->d_vsf.upload(vsf.data(), n);
     ctx->d_vsfx.upload(vsfx.data(), n);

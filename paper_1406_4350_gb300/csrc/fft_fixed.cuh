@@ -533,7 +533,7 @@ __device__ __forceinline__ void inverse_passes(Load load, const fk::FastArgs& fa
 }
 
 // Plane z of band b (fk::plane_body_pruned in fixed point): inverse y and x transforms,
-// multiply by V_loc (Vs: (h, l) of V_loc / 2^ve in split order), forward x and y.  C: the
+// multiply by V_loc (Vs: (h, l) of V_loc / 2^ve in split order, ve the plane's exponent), forward x and y.  C: the
 // column buffer's elements, double-float pairs or FP64.  NT threads; the plane (16 bytes a
 // point) fills the SM's shared memory, so one block runs per SM at N = 96.
 template <int N, int NT, typename C>

@@ -11,10 +11,10 @@ namespace {
 template <int N> constexpr int fx_threads() { return N >= 90 ? 768 : N >= 48 ? 256 : 128; }
 
 template <int N, typename C>
-__global__ void __launch_bounds__(fx_threads<N>()) k_plane_fx(C* __restrict__ T, const int2* __restrict__ Vs, int ve,
-                                                              fk::FastArgs fa) {
+__global__ void __launch_bounds__(fx_threads<N>()) k_plane_fx(C* __restrict__ T, const int2* __restrict__ Vs,
+                                                              const int* __restrict__ ve, fk::FastArgs fa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fx::plane_body<N, fx_threads<N>()>(T, Vs, ve, fa, blockIdx.x, blockIdx.y, smem_raw);
+  fx::plane_body<N, fx_threads<N>()>(T, Vs, ve[blockIdx.x], fa, blockIdx.x, blockIdx.y, smem_raw);
 }
 
 template <int N>
@@ -36,7 +36,7 @@ template <int N, typename C> void launch(chebfi_ctx* ctx, int64_t nb, C* T, cuda
   const size_t bytes = prepare<N>(ctx, (const void*)k_plane_fx<N, C>);
   const double col = (double)N * ctx->sph.ncol * (double)nb * sizeof(C);
   CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col,
-                  k_plane_fx<N, C><<<dim3(N, (unsigned)nb), fx_threads<N>(), bytes, st>>>(T, ctx->d_vsfx.p, ctx->v_exp,
+                  k_plane_fx<N, C><<<dim3(N, (unsigned)nb), fx_threads<N>(), bytes, st>>>(T, ctx->d_vsfx.p, ctx->d_vexp.p,
                                                                                       fk::fast_args(ctx)));
 }
 template <int N> void launch_real(chebfi_ctx* ctx, int64_t nb, const double2* T, double2* out, cudaStream_t st) {

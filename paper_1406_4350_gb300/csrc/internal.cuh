@@ -303,8 +303,8 @@ struct chebfi_ctx {
   bool fast_fft = false;         // cubic grid of a compiled size: two-pass FFT kernels
   chebfi::DevBuf<double> d_vs;   // V_loc in split order [z'][x'][y'] for those kernels
   chebfi::DevBuf<float> d_vsf;
-  chebfi::DevBuf<int2> d_vsfx;   // the same table in fixed point: V_loc = (h 2^31 + l) 2^(v_exp - 62)
-  int v_exp = 0;
+  chebfi::DevBuf<int2> d_vsfx;   // the same table in fixed point: V_loc = (h 2^31 + l) 2^(vexp[z'] - 62)
+  chebfi::DevBuf<int> d_vexp;
   int fft64 = CHEBFI_FFT64_DOUBLE_FLOAT;       // arithmetic of the FP64 path's transforms
   double vmax = 0.0;
 

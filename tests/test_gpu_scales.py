@@ -96,3 +96,54 @@ def test_modular_gemm_at_every_scale(m, n, k, conjA, conjB):
         inside = (ei + fj > -1000) & (ei + fj < 950)  # in FP64's normal range
         assert np.array_equal(np.where(inside, C.real, 0), np.where(inside, ref_re, 0))
         assert np.array_equal(np.where(inside, C.imag, 0), np.where(inside, ref_im, 0))
+
+
+def _vpart(cell, Y):
+    """The sphere's coefficients of V psi in extended precision, and ||V psi|| + ||V|| rms(psi), what
+    an FP64 transform's rounding is relative to."""
+    n = int(cell.grid[0])
+    m = np.asarray(cell.miller) % n
+    out, size = np.empty(Y.shape, np.clongdouble), np.empty(Y.shape[1])
+    V = cell.vloc.astype(np.longdouble)
+    for j in range(Y.shape[1]):
+        box = np.zeros((n, n, n), np.clongdouble)
+        box[m[:, 0], m[:, 1], m[:, 2]] = Y[:, j]
+        psi = np.fft.ifftn(box) * np.longdouble(n) ** 3
+        f = V * psi
+        out[:, j] = (np.fft.fftn(f) / np.longdouble(n) ** 3)[m[:, 0], m[:, 1], m[:, 2]]
+        size[j] = (np.linalg.norm(f.astype(complex)) +
+                   np.linalg.norm(cell.vloc) * np.linalg.norm(Y[:, j])) / n ** 1.5
+    return out, size
+
+
+def _without_kinetic(n, core=0.0, scale=1.0):
+    """A cell so large that its kinetic energies are 2^-120 of their size, and no projectors' part."""
+    L = 0.42 * n
+    cell = make_cell(L, n, 0.5 * (2.0 * np.pi / L * 0.23 * n) ** 2, 1, 8, 3, False, 43, kpt=(0.02, -0.05, 0.03))
+    cell.D = np.zeros_like(cell.D)
+    cell.vloc = cell.vloc * scale
+    if core:
+        cell.vloc[n // 3, n // 5, n // 2] = core
+    cell.lattice = cell.lattice * 2.0 ** 60
+    cell.kpt = cell.kpt * 2.0 ** -60
+    return cell
+
+
+def _vpart_error(cell):
+    """Errors of V psi, relative to what an FP64 transform's rounding is relative to."""
+    ref, size = _vpart(cell, cell.Y0)
+    got = _np(_ctx(cell).apply_H(_F(cell.Y0)))
+    return np.linalg.norm((got - ref).astype(complex), axis=0) / size
+
+
+# V psi alone, for an ordinary potential, and one with a core at one point.  3 log2 n levels
+# each way that round half a unit each, adding up as their root; on the lengths with
+# double-float z passes, twice what those round without the core
+@pytest.mark.parametrize("n", [36, 60, 64, 80])
+def test_a_core_takes_no_bits_from_the_other_planes(n):
+    plain = _vpart_error(_without_kinetic(n))
+    cored = _vpart_error(_without_kinetic(n, 64.0))
+    if n == 64:
+        assert cored.max() <= 2.0 * plain.max()
+    else:
+        assert max(plain.max(), cored.max()) <= 0.5 * np.sqrt(6.0 * np.log2(n)) * U, (plain / U, cored / U)
