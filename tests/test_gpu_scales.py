@@ -147,3 +147,17 @@ def test_a_core_takes_no_bits_from_the_other_planes(n):
         assert cored.max() <= 2.0 * plain.max()
     else:
         assert max(plain.max(), cored.max()) <= 0.5 * np.sqrt(6.0 * np.log2(n)) * U, (plain / U, cored / U)
+
+
+# Potentials far from one, whose planes' exponents are far from zero.  A power of two changes no
+# digit of V psi: the results differ by it and no more than the rounding of the kinetic part's
+# 2^-80 beside it (on the double-float lengths a unit of the pairs)
+@pytest.mark.parametrize("n", [16, 24, 48, 60, 90, 96])
+@pytest.mark.parametrize("e", [-40, -3, 3, 30])
+def test_local_potential_of_any_size(n, e):
+    cell = _without_kinetic(n)
+    one = _np(_ctx(cell).apply_H(_F(cell.Y0)))
+    ref = PWOperator.from_cell(cell).apply_H(cell.Y0)
+    assert np.abs(one - ref).max() <= 1e-11 * np.abs(ref).max()  # the FP64 form's parity tolerance
+    got = _np(_ctx(_without_kinetic(n, scale=2.0 ** e)).apply_H(_F(cell.Y0))) * 2.0 ** -e
+    assert np.abs(got - one).max() <= 2.0 ** -46 * np.abs(one).max()
