@@ -30,13 +30,16 @@ __device__ __forceinline__ void flag_error(int* status, int code) {
 // Unblocked Cholesky of one nb x nb diagonal block (nb <= NB) in shared memory.  One block:
 // the pivots are a serial chain, and GB300's FP64 unit (about two FMAs per clock) makes each
 // square root and division ~10 dependent slow instructions.  Only 1 / sqrt(d) is on the
-// chain (the column is scaled by it), and one warp forms the next column's while the others
-// update the trailing triangle; the diagonal's square roots are taken together at the end
-// (32 x 32: 66 us with sqrt and a division per entry on the chain, 39 us with the reciprocal
-// root between barriers, now 31 us).
+// chain, with one Newton step for the root itself; one warp forms the next column's while the
+// others update the trailing triangle.  32 x 32: 66 us with sqrt and a division per entry on the
+// chain, now 36.
+// Each operation rounds once, as those did: an entry times the reciprocal is corrected by its
+// residual to a / s, and a product of two complex entries is formed before it is subtracted.
+// Without these (the reciprocal alone, two multiply-adds into the entry: 31 us) the rms of
+// |A - L L^H| is 0.86-0.89 units of 2^-53 |L| |L|^H where it is 0.64.
 __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int nb, int* status) {
   __shared__ double2 a[NB][NB + 1];
-  __shared__ double rpiv;
+  __shared__ double2 piv;  // (sqrt(d), 1 / sqrt(d))
   const int tid = threadIdx.x;
   for (int e = tid; e < nb * nb; e += blockDim.x) {
     const int i = e % nb, j = e / nb;
@@ -49,16 +52,20 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
       flag_error(status, CHEBFI_ERR_NOT_SPD);
       a[j][j].x = 1.0;
     }
-    rpiv = rsqrt(a[j][j].x);
+    // the root of the pivot, rounded to nearest but for rare ties: one Newton step on d rsqrt(d)
+    const double p = a[j][j].x, r = rsqrt(p), s = p * r;
+    piv = make_double2(fma(0.5 * r, fma(-s, s, p), s), r);
   };
   if (tid == 0) pivot(0);
   __syncthreads();
   for (int j = 0; j < nb; ++j) {
-    const int i = j + 1 + tid;
-    if (i < nb) {
-      a[i][j].x *= rpiv;
-      a[i][j].y *= rpiv;
+    const int i = j + 1 + tid % 32;
+    if (tid < 64 && i < nb) {  // one warp a part: a / s rounded once
+      double* v = &a[i][j].x + tid / 32;
+      const double q = *v * piv.y;
+      *v = fma(fma(-q, piv.x, *v), piv.y, q);
     }
+    if (tid == 64) a[j][j] = make_double2(piv.x, 0.0);
     __syncthreads();
     // trailing update of the lower triangle: a[i][k] -= L[i][j] conj(L[k][j]) for i >= k > j.
     // Its m columns are folded in pairs (q, m - 1 - q) of m + 1 entries together, so that no
@@ -67,16 +74,14 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
     auto update = [&](int i, int k) {
       const double2 li = a[i][j], lk = a[k][j];
       double2 v = a[i][k];
-      v.x = fma(-li.x, lk.x, v.x);
-      v.y = fma(-li.y, lk.x, v.y);
-      v.x = fma(-li.y, lk.y, v.x);
-      v.y = fma(li.x, lk.y, v.y);
+      v.x -= fma(li.y, lk.y, li.x * lk.x);
+      v.y -= fma(li.y, lk.x, -(li.x * lk.y));
       a[i][k] = v;
     };
     if (tid < 32) {
       if (tid == 0 && m > 0) {
         const double2 l = a[j + 1][j];  // the diagonal is real
-        a[j + 1][j + 1].x = fma(-l.y, l.y, fma(-l.x, l.x, a[j + 1][j + 1].x));
+        a[j + 1][j + 1].x -= fma(l.y, l.y, l.x * l.x);
         pivot(j + 1);
       }
     } else {
@@ -92,7 +97,7 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
   }
   for (int e = tid; e < nb * nb; e += blockDim.x) {
     const int i = e % nb, j = e / nb;
-    A[i + j * lda] = i > j ? a[i][j] : make_double2(i == j ? sqrt(a[i][j].x) : 0.0, 0.0);
+    A[i + j * lda] = i >= j ? a[i][j] : make_double2(0.0, 0.0);
   }
 }
 
@@ -100,31 +105,38 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
 // lanes hold its unknowns, and step k broadcasts x_k = s_k / L_kk to the lanes that still
 // need it.  A system is a serial chain of nb slow FP64 steps, so systems are spread over the
 // SMs (four warps a block) instead of one per thread, which kept 128 of them on one SM
-// (224 x 32: 131 and 172 us with a thread per system, now 18 us).
+// (224 x 32: 131 and 172 us with a thread per system, now 22 us).  The reciprocal is a pair of
+// twice the precision and a complex product is formed before it is subtracted, so that each
+// operation rounds once, as with a division (rms residual 0.50 units of 2^-53 |L| |x|; with the
+// reciprocal alone and two multiply-adds 0.66, and 18 us).
 constexpr int kTrsmWarps = 4;
 // x_l <- x_l - sum_{k < l} c_lk x_k solved forward; c_lk = L[l][k], or its conjugate
 template <bool CONJ>
-__device__ __forceinline__ double2 warp_forward(const double2 (*l)[NB + 1], const double* rd, double2 x, int nb) {
+__device__ __forceinline__ double2 warp_forward(const double2 (*l)[NB + 1], const double2* rd, double2 x, int nb) {
   const int lane = threadIdx.x % 32;
   for (int k = 0; k < nb; ++k) {
-    const double r = rd[k];
-    const double2 xk = make_double2(__shfl_sync(0xffffffffu, x.x, k) * r, __shfl_sync(0xffffffffu, x.y, k) * r);
+    const double2 r = rd[k];
+    const double sx = __shfl_sync(0xffffffffu, x.x, k), sy = __shfl_sync(0xffffffffu, x.y, k);
+    const double2 xk = make_double2(fma(sx, r.x, sx * r.y), fma(sy, r.x, sy * r.y));
     double2 c = l[lane][k];  // L is lower triangular: zero above, and rows >= nb are zero
     if (CONJ) c.y = -c.y;
     if (lane == k) x = xk;
     else if (lane > k) {
-      x.x = fma(-c.x, xk.x, fma(c.y, xk.y, x.x));
-      x.y = fma(-c.x, xk.y, fma(-c.y, xk.x, x.y));
+      x.x -= fma(c.x, xk.x, -(c.y * xk.y));
+      x.y -= fma(c.x, xk.y, c.y * xk.x);
     }
   }
   return x;
 }
 __device__ __forceinline__ void load_tri(const double2* __restrict__ L, int64_t ldl, int nb, double2 (*l)[NB + 1],
-                                         double* rd) {
+                                         double2* rd) {
   for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
     const int i = e % NB, j = e / NB;
     l[i][j] = i < nb && j < nb ? L[i + j * ldl] : make_double2(0.0, 0.0);
-    if (i == j) rd[i] = i < nb ? 1.0 / L[i + j * ldl].x : 0.0;
+    if (i == j) {
+      const double d = i < nb ? L[i + j * ldl].x : 1.0, r = 1.0 / d;
+      rd[i] = make_double2(r, r * fma(-r, d, 1.0));
+    }
   }
   __syncthreads();
 }
@@ -133,7 +145,7 @@ __device__ __forceinline__ void load_tri(const double2* __restrict__ L, int64_t 
 __global__ void __launch_bounds__(32 * kTrsmWarps) k_trsm_right_lh(const double2* __restrict__ L, int64_t ldl, double2* B, int64_t ldb, int64_t m,
                                                                   int nb) {
   __shared__ double2 l[NB][NB + 1];
-  __shared__ double rd[NB];
+  __shared__ double2 rd[NB];
   load_tri(L, ldl, nb, l, rd);
   const int lane = threadIdx.x % 32;
   const int64_t r = (int64_t)blockIdx.x * kTrsmWarps + threadIdx.x / 32;
@@ -147,7 +159,7 @@ __global__ void __launch_bounds__(32 * kTrsmWarps) k_trsm_right_lh(const double2
 __global__ void __launch_bounds__(32 * kTrsmWarps) k_trsm_left_l(const double2* __restrict__ L, int64_t ldl, double2* B, int64_t ldb, int64_t m,
                                                                 int nb) {
   __shared__ double2 l[NB][NB + 1];
-  __shared__ double rd[NB];
+  __shared__ double2 rd[NB];
   load_tri(L, ldl, nb, l, rd);
   const int lane = threadIdx.x % 32;
   const int64_t c = (int64_t)blockIdx.x * kTrsmWarps + threadIdx.x / 32;

@@ -31,3 +31,12 @@ def test_double_float_conversions_round_as_the_fp64_unit(tmp_path):
     [(n, nv, bad, badv)] = run("df_store_check", tmp_path)
     assert n > 100000 and nv > 100000
     assert bad == 0 and badv == 0
+
+
+@pytest.mark.gpu
+def test_cholesky_and_triangular_solve_round_once_per_operation(tmp_path):
+    [(nq, bad, nt, badt)] = run("quotient_check", tmp_path)
+    assert nq > 15000 and nt > 400000
+    # a product of relative size 2^-24 moves a rounding in about one of 2^20 values, the
+    # reciprocals' own errors in fewer
+    assert bad <= 1e-4 * nq and badt <= 1e-4 * nt
