@@ -892,18 +892,18 @@ __device__ void solve_shared(float2* S, float2* W, int sweeps, float tol) {
   }
 }
 
-// Blocks [0, npairs): gather the pair's subproblem, one sweep, write its rotation W (64 x 64,
-// column-major) to Wout[pair].  The others: V <- V W of the round before (Wprev), a block per
-// 128 rows and pair, 64 rows for each half of its threads.
+// Blocks [0, nsolve) (all pairs, or none): gather the pair's subproblem, one sweep, write its
+// rotation W (64 x 64, column-major) to Wout[pair].  The others: V <- V W of the round before
+// (Wprev), a block per 128 rows and pair, 64 rows for each half of its threads.
 __global__ void __launch_bounds__(512) k_bj_solve(const float2* __restrict__ A, float2* __restrict__ V, int64_t ld,
-                                                  int nbk, int round, int round_prev, float2* __restrict__ Wout,
+                                                  int nbk, int nsolve, int round, int round_prev, float2* __restrict__ Wout,
                                                   const float2* __restrict__ Wprev, float tol) {
   extern __shared__ __align__(16) unsigned char smem[];
   float2* W = reinterpret_cast<float2*>(smem);
   float2* S = W + S2 * PS;
   const int tid = threadIdx.x, npairs = nbk / 2;
   int I, J;
-  if ((int)blockIdx.x < npairs) {
+  if ((int)blockIdx.x < nsolve) {
     blocks_of(blockIdx.x, round, nbk, I, J);
     for (int e = tid; e < S2 * S2; e += 512) {
       const int i = e % S2, j = e / S2;
@@ -918,7 +918,7 @@ __global__ void __launch_bounds__(512) k_bj_solve(const float2* __restrict__ A, 
     for (int e = tid; e < S2 * S2; e += 512) wo[e] = W[(e % S2) + PS * (e / S2)];
     return;
   }
-  const int u = blockIdx.x - npairs, pair = u % npairs, half = tid / 256, t = tid % 256;
+  const int u = blockIdx.x - nsolve, pair = u % npairs, half = tid / 256, t = tid % 256;
   const int64_t r0 = (int64_t)(u / npairs) * 2 * S2 + half * S2;
   const bool rows = r0 < ld;  // an odd number of 64-row tiles leaves the last half idle
   blocks_of(pair, round_prev, nbk, I, J);
@@ -1163,17 +1163,17 @@ bool jacobi_eigh_f32(int64_t n0, const float2* A, int64_t lda, float2* V, int64_
     for (int round = 0; round < nbk - 1; ++round) {
       const unsigned extra = last_round >= 0 ? vtiles : 0;
       CHEBFI_LAUNCH_W("k_bj_solve", st, prod * 2.0 * extra,
-                      bj::k_bj_solve<<<npairs + extra, 512, sbytes, st>>>(Ap, Vp, np, nbk, round, last_round, Wb[w], Wb[w ^ 1],
-                                                                         1e-7f));
+                      bj::k_bj_solve<<<npairs + extra, 512, sbytes, st>>>(Ap, Vp, np, nbk, npairs, round, last_round, Wb[w],
+                                                                         Wb[w ^ 1], 1e-7f));
       CHEBFI_LAUNCH_W("k_bj_update", st, prod * 2.0 * atiles,
                       bj::k_bj_update<<<atiles, 256, bytes, st>>>(Ap, np, nbk, round, Wb[w]));
       last_round = round;
       w ^= 1;
     }
   }
-  if (last_round >= 0) {  // the last W (the block's own subproblem is solved again, into the free W)
+  if (last_round >= 0) {  // the last W: nothing is left to solve
     CHEBFI_LAUNCH_W("k_bj_solve", st, prod * 2.0 * vtiles,
-                    bj::k_bj_solve<<<npairs + vtiles, 512, sbytes, st>>>(Ap, Vp, np, nbk, 0, last_round, Wb[w], Wb[w ^ 1], 1e-7f));
+                    bj::k_bj_solve<<<vtiles, 512, sbytes, st>>>(Ap, Vp, np, nbk, 0, 0, last_round, Wb[w], Wb[w ^ 1], 1e-7f));
   }
   CHEBFI_CUDA(cudaMemcpy2DAsync(V, ldv * sizeof(float2), Vp, np * sizeof(float2), n0 * sizeof(float2), n0,
                                 cudaMemcpyDeviceToDevice, st));
