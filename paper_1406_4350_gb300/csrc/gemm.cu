@@ -4,7 +4,7 @@
 // (Algorithm 1, Section 5.1), the Woodbury core products, and the subspace matrices and
 // rotations of Algorithm 2.  FP32: 64 x 64 output tiles, 256 threads, 4 x 4 complex outputs
 // per thread (gemm_tile.cuh).  FP64: 256 outputs per tile, one per thread (k_gemm_d).  Both split K, with a
-// deterministic second pass, when the output has too few tiles to fill the 152 SMs.
+// deterministic second pass, when the output has too few tiles to fill the SMs.
 #include <algorithm>
 
 #include "gemm_tile.cuh"
@@ -169,6 +169,13 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(int64_t M, int64_t N, int
   Cm[i + j * ldc] = r;
 }
 
+int sm_count() {
+  int dev = 0, sms = 0;
+  CHEBFI_CUDA(cudaGetDevice(&dev));
+  CHEBFI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  return sms;
+}
+
 template <bool CA, bool CB>
 void launch_f(int64_t M, int64_t N, int64_t K, double alpha, const float2* A, int64_t lda, const float2* B, int64_t ldb,
               double beta, float2* Cm, int64_t ldc, cudaStream_t st, DevBuf<float2>* ws, const char* tag, bool lower) {
@@ -185,9 +192,9 @@ void launch_f(int64_t M, int64_t N, int64_t K, double alpha, const float2* A, in
     splits = std::max<int64_t>(1, (K + kchunk - 1) / kchunk);
     return (double)((tiles * splits + per_round - 1) / per_round) * (double)kchunk;
   };
-  constexpr int64_t kSMs = 152;
+  const int64_t sms = sm_count();
   int64_t s4, c4, s2, c2;
-  const double cost4 = 3.0 * plan((N + 63) / 64, 3 * kSMs, s4, c4), cost2 = 4.0 * 0.5 * 1.1 * plan((N + 31) / 32, 4 * kSMs, s2, c2);
+  const double cost4 = 3.0 * plan((N + 63) / 64, 3 * sms, s4, c4), cost2 = 4.0 * 0.5 * 1.1 * plan((N + 31) / 32, 4 * sms, s2, c2);
   const bool narrow = cost2 < cost4;
   const int64_t tn = narrow ? (N + 31) / 32 : (N + 63) / 64, tiles = tm * tn, splits = narrow ? s2 : s4, kchunk = narrow ? c2 : c4;
   float2* wsp = nullptr;
@@ -224,8 +231,9 @@ void launch_d(int64_t M, int64_t N, int64_t K, double alpha, const double2* A, i
   if (padded(32, 8) < padded(TM, TN)) { TM = 32; TN = 8; }
   const int64_t tm = (M + TM - 1) / TM, tn = (N + TN - 1) / TN, tiles = tm * tn;
   // two blocks per SM; a split is at least one k tile
+  const int64_t blocks = 2 * sm_count();
   int64_t splits = 1;
-  if (ws && tiles < 304) splits = std::max<int64_t>(1, std::min<int64_t>((304 + tiles - 1) / tiles, (K + KD - 1) / KD));
+  if (ws && tiles < blocks) splits = std::max<int64_t>(1, std::min<int64_t>((blocks + tiles - 1) / tiles, (K + KD - 1) / KD));
   int64_t kchunk = std::max<int64_t>(KD, ((K + splits - 1) / splits + KD - 1) / KD * KD);
   splits = std::max<int64_t>(1, (K + kchunk - 1) / kchunk);
   double2* wsp = nullptr;
