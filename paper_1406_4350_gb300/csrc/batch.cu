@@ -77,13 +77,13 @@ __global__ void k_bscatter(const KDesc<R>* __restrict__ ks, int64_t nb, const cp
 // ---------------------------------------------------------------- FFT passes
 template <typename R, int N>
 __global__ void __launch_bounds__(kT) k_bzinv(const KDesc<R>* __restrict__ ks, const cplx<R>* __restrict__ Y,
-                                              cplx<R>* __restrict__ T, const cplx<R>* __restrict__ tw,
-                                              const int32_t* __restrict__ cb_k, const int32_t* __restrict__ cb_c0) {
+                                              cplx<R>* __restrict__ T, const int32_t* __restrict__ cb_k,
+                                              const int32_t* __restrict__ cb_c0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int k = cb_k[blockIdx.x];
   const KDesc<R>& d = ks[k];
   const FastArgs fa = d.fa;
-  fk::zinv_body<R, N>(Y + d.y_off, d.npw, T + d.t_off, fa, tw, cb_c0[blockIdx.x], blockIdx.y, smem_raw);
+  fk::zinv_body<R, N>(Y + d.y_off, d.npw, T + d.t_off, fa, cb_c0[blockIdx.x], blockIdx.y, smem_raw);
 }
 
 template <typename R, int N>
@@ -100,9 +100,8 @@ __global__ void __launch_bounds__(kT) k_bplane(const KDesc<R>* __restrict__ ks, 
 // Z_k = (K + V_loc) Y_k and T_k = a_k (Z_k - c_k Y_k) - b Yprev_k written over Yprev_k
 template <typename R, int N>
 __global__ void __launch_bounds__(kT) k_bzfwd(const KDesc<R>* __restrict__ ks, const cplx<R>* __restrict__ T,
-                                              const cplx<R>* __restrict__ tw, const int32_t* __restrict__ cb_k,
-                                              const int32_t* __restrict__ cb_c0, const cplx<R>* Ycur, cplx<R>* Z,
-                                              cplx<R>* Yprev, int first) {
+                                              const int32_t* __restrict__ cb_k, const int32_t* __restrict__ cb_c0,
+                                              const cplx<R>* Ycur, cplx<R>* Z, cplx<R>* Yprev, int first) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int k = cb_k[blockIdx.x];
   const KDesc<R>& d = ks[k];
@@ -119,7 +118,7 @@ __global__ void __launch_bounds__(kT) k_bzfwd(const KDesc<R>* __restrict__ ks, c
   ep.c = d.c;
   ep.bprev = first ? (R)0 : (R)1;
   ep.inv_n3 = (R)(1.0 / ((double)N * N * N));
-  fk::zfwd_body<R, N>(T + d.t_off, fa, tw, d.K, ep, cb_c0[blockIdx.x], blockIdx.y, smem_raw);
+  fk::zfwd_body<R, N>(T + d.t_off, fa, d.K, ep, cb_c0[blockIdx.x], blockIdx.y, smem_raw);
 }
 
 // ---------------------------------------------------------------- projection-space combination
@@ -384,7 +383,6 @@ template <> struct BatchOps<double> {
   static const double2* M(chebfi_ctx* c) { return c->d_M.p; }
   static const double* D(chebfi_ctx* c) { return c->d_Dblk.p; }
   static const double* Vs(chebfi_ctx* c) { return c->d_vs.p; }
-  static const double2* tw(chebfi_ctx* c) { return c->ax[0].tw64.p; }
 };
 template <> struct BatchOps<float> {
   static constexpr int form = 1;
@@ -401,7 +399,6 @@ template <> struct BatchOps<float> {
   static const float2* M(chebfi_ctx* c) { return c->d_Mf.p; }
   static const float* D(chebfi_ctx* c) { return c->d_Dblkf.p; }
   static const float* Vs(chebfi_ctx* c) { return c->d_vsf.p; }
-  static const float2* tw(chebfi_ctx* c) { return c->ax[0].tw32.p; }
 };
 
 // (k, tile[, chunk]) items of a GEMM class for tile shape `shape` and split factor
@@ -480,12 +477,11 @@ void blocal(chebfi_batch* bt, const cplx<R>* cur, cplx<R>* Z, cplx<R>* prev, int
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
   const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
   const KDesc<R>* d = BatchOps<R>::desc(bt).p;
-  const cplx<R>* tw = BatchOps<R>::tw(c0);
   cplx<R>* T = BatchOps<R>::T(bt).p;
   const dim3 gz((unsigned)bt->ncb, (unsigned)bt->nb);
-  CHEBFI_LAUNCH("k_bzinv", st, (k_bzinv<R, N><<<gz, kT, zbytes, st>>>(d, cur, T, tw, bt->cb_k.p, bt->cb_c0.p)));
+  CHEBFI_LAUNCH("k_bzinv", st, (k_bzinv<R, N><<<gz, kT, zbytes, st>>>(d, cur, T, bt->cb_k.p, bt->cb_c0.p)));
   CHEBFI_LAUNCH("k_bplane", st, (k_bplane<R, N><<<dim3(N, (unsigned)(bt->nk * bt->nb)), kT, pbytes, st>>>(d, bt->nb, T, BatchOps<R>::Vs(c0))));
-  CHEBFI_LAUNCH("k_bzfwd", st, (k_bzfwd<R, N><<<gz, kT, zbytes, st>>>(d, T, tw, bt->cb_k.p, bt->cb_c0.p, cur, Z, prev, first)));
+  CHEBFI_LAUNCH("k_bzfwd", st, (k_bzfwd<R, N><<<gz, kT, zbytes, st>>>(d, T, bt->cb_k.p, bt->cb_c0.p, cur, Z, prev, first)));
 }
 
 // the grouped kernels are compiled for these lengths

@@ -177,32 +177,22 @@ __global__ void k_zero_upper(int64_t n, double2* A, int64_t lda) {
 }
 
 // ------------------------------------------------------------------ Jacobi
-// Templated on the real type: FP64 for the eigensolver itself, FP32 for the first stage of
-// the refined eigensolver (whose vectors are then refined to FP64 accuracy).
-template <typename R> struct JacEps;
-template <> struct JacEps<double> {
-  static constexpr double v = 1.1102230246251565e-16, tiny = 1e-300;
-};
-template <> struct JacEps<float> {
-  static constexpr float v = 5.9604645e-8f, tiny = 1e-37f;
-};
+// In FP64; the refined eigensolver's first stage has its own FP32 form (blocked Jacobi, below).
+constexpr double kEpsD = 1.1102230246251565e-16, kTinyD = 1e-300;
+constexpr float kEpsF = 5.9604645e-8f;
 
 __device__ __forceinline__ int64_t rr_player(int64_t pos, int64_t round, int64_t n) {
   return pos == 0 ? 0 : 1 + (pos - 1 + round) % (n - 1);
 }
 
-template <typename R> struct RotT {
-  R c, s;
-  cplx<R> ph;  // e^{i phi}
+struct Rot {
+  double c, s;
+  double2 ph;  // e^{i phi}
 };
 
-__device__ __forceinline__ double hyp(double a, double b) { return hypot(a, b); }
-__device__ __forceinline__ float hyp(float a, float b) { return hypotf(a, b); }
-
 // rotation parameters of pair t of the given round (p < q; q = -1 for the padding player)
-template <typename R>
 __device__ __forceinline__ void jac_params_item(int64_t t, int64_t n0, int64_t n, int64_t round,
-                                                const cplx<R>* __restrict__ A, int64_t lda, RotT<R>* __restrict__ rot,
+                                                const double2* __restrict__ A, int64_t lda, Rot* __restrict__ rot,
                                                 int* __restrict__ pairs) {
   int64_t p = rr_player(t, round, n), q = rr_player(n - 1 - t, round, n);
   if (p > q) {
@@ -210,20 +200,20 @@ __device__ __forceinline__ void jac_params_item(int64_t t, int64_t n0, int64_t n
     p = q;
     q = tmp;
   }
-  RotT<R> r;
-  r.c = (R)1;
-  r.s = (R)0;
-  r.ph = cmake<cplx<R>>(1.0, 0.0);
+  Rot r;
+  r.c = 1.0;
+  r.s = 0.0;
+  r.ph = make_double2(1.0, 0.0);
   if (q < n0) {
-    const cplx<R> h = A[p + q * lda];
-    const R g = hyp(h.x, h.y);
-    const R app = A[p + p * lda].x, aqq = A[q + q * lda].x;
-    if (g > JacEps<R>::tiny && g > JacEps<R>::v * sqrt(fabs(app * aqq))) {
-      const R zeta = (aqq - app) / ((R)2 * g);
-      const R t_ = (zeta >= (R)0 ? (R)1 : (R)-1) / (fabs(zeta) + hyp((R)1, zeta));
-      r.c = (R)1 / sqrt((R)1 + t_ * t_);
+    const double2 h = A[p + q * lda];
+    const double g = hypot(h.x, h.y);
+    const double app = A[p + p * lda].x, aqq = A[q + q * lda].x;
+    if (g > kTinyD && g > kEpsD * sqrt(fabs(app * aqq))) {
+      const double zeta = (aqq - app) / (2.0 * g);
+      const double t_ = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + hypot(1.0, zeta));
+      r.c = 1.0 / sqrt(1.0 + t_ * t_);
       r.s = t_ * r.c;
-      r.ph = cmake<cplx<R>>(h.x / g, h.y / g);
+      r.ph = make_double2(h.x / g, h.y / g);
     }
   } else {
     q = -1;
@@ -233,18 +223,16 @@ __device__ __forceinline__ void jac_params_item(int64_t t, int64_t n0, int64_t n
   pairs[2 * t + 1] = (int)q;
 }
 
-template <typename R>
-__global__ void k_jac_params(int64_t n0, int64_t n, int64_t round, const cplx<R>* __restrict__ A, int64_t lda,
-                             RotT<R>* __restrict__ rot, int* __restrict__ pairs) {
+__global__ void k_jac_params(int64_t n0, int64_t n, int64_t round, const double2* __restrict__ A, int64_t lda,
+                             Rot* __restrict__ rot, int* __restrict__ pairs) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n / 2) jac_params_item<R>(t, n0, n, round, A, lda, rot, pairs);
+  if (t < n / 2) jac_params_item(t, n0, n, round, A, lda, rot, pairs);
 }
 
 // [a, b] <- [c a - s e^{i phi} b, s a + c e^{i phi} b] (rows, U^H from the left) and
 // [a, b] <- [c a - s e^{-i phi} b, s a + c e^{-i phi} b] (columns, U from the right)
-template <typename C, typename R>
-__device__ __forceinline__ void rot2(C& a, C& b, R c, R s, C ph) {
-  C na, nb;
+__device__ __forceinline__ void rot2(double2& a, double2& b, double c, double s, double2 ph) {
+  double2 na, nb;
   na.x = c * a.x - s * (ph.x * b.x - ph.y * b.y);
   na.y = c * a.y - s * (ph.x * b.y + ph.y * b.x);
   nb.x = s * a.x + c * (ph.x * b.x - ph.y * b.y);
@@ -259,38 +247,36 @@ __host__ __device__ inline int64_t jac_items(int64_t h, int64_t n) { return h * 
 // One round of rotations in one pass: item (t1, t2) maps the 2 x 2 block of A on rows
 // {p1, q1} and columns {p2, q2} to U1^H A U2 (the pairs are disjoint, so every element of A
 // belongs to exactly one block); the remaining items apply V <- V U2 on columns {p2, q2}.
-template <typename R>
-__device__ __forceinline__ void jac_apply_item(int64_t idx, int64_t h, int64_t n, cplx<R>* A, int64_t lda,
-                                               cplx<R>* V, int64_t ldv, const RotT<R>* __restrict__ rot,
+__device__ __forceinline__ void jac_apply_item(int64_t idx, int64_t h, int64_t n, double2* A, int64_t lda,
+                                               double2* V, int64_t ldv, const Rot* __restrict__ rot,
                                                const int* __restrict__ pairs) {
-  using C = cplx<R>;
   const int64_t nblk_a = h * h;
   if (idx < nblk_a) {
     const int64_t t1 = idx % h, t2 = idx / h;
     const int q1 = pairs[2 * t1 + 1], q2 = pairs[2 * t2 + 1];
     const int p1 = pairs[2 * t1], p2 = pairs[2 * t2];
-    const RotT<R> r1 = rot[t1], r2 = rot[t2];
-    const bool act1 = q1 >= 0 && r1.s != (R)0, act2 = q2 >= 0 && r2.s != (R)0;
+    const Rot r1 = rot[t1], r2 = rot[t2];
+    const bool act1 = q1 >= 0 && r1.s != 0.0, act2 = q2 >= 0 && r2.s != 0.0;
     if (!act1 && !act2) return;
-    const C cph2 = conjg(r2.ph);
+    const double2 cph2 = conjg(r2.ph);
     // the padding player (q < 0) owns no row or column of A: 1 x 2 or 2 x 1 blocks
     if (q1 < 0 || q2 < 0) {
       if (q1 < 0 && q2 < 0) return;
       if (q1 < 0) {  // row p1 alone, columns {p2, q2} rotate by U2
-        C a = A[p1 + (int64_t)p2 * lda], b = A[p1 + (int64_t)q2 * lda];
+        double2 a = A[p1 + (int64_t)p2 * lda], b = A[p1 + (int64_t)q2 * lda];
         rot2(a, b, r2.c, r2.s, cph2);
         A[p1 + (int64_t)p2 * lda] = a;
         A[p1 + (int64_t)q2 * lda] = b;
       } else {  // column p2 alone, rows {p1, q1} rotate by U1^H
-        C a = A[p1 + (int64_t)p2 * lda], b = A[q1 + (int64_t)p2 * lda];
+        double2 a = A[p1 + (int64_t)p2 * lda], b = A[q1 + (int64_t)p2 * lda];
         rot2(a, b, r1.c, r1.s, r1.ph);
         A[p1 + (int64_t)p2 * lda] = a;
         A[q1 + (int64_t)p2 * lda] = b;
       }
       return;
     }
-    C m00 = A[p1 + (int64_t)p2 * lda], m10 = A[q1 + (int64_t)p2 * lda];
-    C m01 = A[p1 + (int64_t)q2 * lda], m11 = A[q1 + (int64_t)q2 * lda];
+    double2 m00 = A[p1 + (int64_t)p2 * lda], m10 = A[q1 + (int64_t)p2 * lda];
+    double2 m01 = A[p1 + (int64_t)q2 * lda], m11 = A[q1 + (int64_t)q2 * lda];
     if (act1) {  // rows: [m0*; m1*] <- U1^H [m0*; m1*]
       rot2(m00, m10, r1.c, r1.s, r1.ph);
       rot2(m01, m11, r1.c, r1.s, r1.ph);
@@ -310,34 +296,32 @@ __device__ __forceinline__ void jac_apply_item(int64_t idx, int64_t h, int64_t n
   const int64_t i = vidx % n, t = vidx / n;
   const int q = pairs[2 * t + 1];
   if (q < 0) return;
-  const RotT<R> r = rot[t];
-  if (r.s == (R)0) return;
+  const Rot r = rot[t];
+  if (r.s == 0.0) return;
   const int p = pairs[2 * t];
-  C ap = V[i + (int64_t)p * ldv], aq = V[i + (int64_t)q * ldv];
+  double2 ap = V[i + (int64_t)p * ldv], aq = V[i + (int64_t)q * ldv];
   rot2(ap, aq, r.c, r.s, conjg(r.ph));
   V[i + (int64_t)p * ldv] = ap;
   V[i + (int64_t)q * ldv] = aq;
 }
 
-template <typename R>
-__global__ void k_jac_apply(int64_t h, int64_t n, cplx<R>* A, int64_t lda, cplx<R>* V, int64_t ldv,
-                            const RotT<R>* __restrict__ rot, const int* __restrict__ pairs) {
+__global__ void k_jac_apply(int64_t h, int64_t n, double2* A, int64_t lda, double2* V, int64_t ldv,
+                            const Rot* __restrict__ rot, const int* __restrict__ pairs) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  jac_apply_item<R>(idx, h, n, A, lda, V, ldv, rot, pairs);
+  jac_apply_item(idx, h, n, A, lda, V, ldv, rot, pairs);
 }
 
 // All n-1 rounds of one Jacobi sweep in one cooperative launch: per round, the rotation
 // parameters of the n/2 pairs, a grid barrier, the one-pass update of A and V, a barrier.
-template <typename R>
-__global__ void k_jac_sweep(int64_t n0, int64_t n, cplx<R>* A, int64_t lda, cplx<R>* V, int64_t ldv, RotT<R>* rot,
+__global__ void k_jac_sweep(int64_t n0, int64_t n, double2* A, int64_t lda, double2* V, int64_t ldv, Rot* rot,
                             int* pairs, unsigned* bar, int* status) {
   const int64_t h = n / 2;
   const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (int64_t round = 0; round < n - 1; ++round) {
-    for (int64_t t = tid; t < h; t += nthreads) jac_params_item<R>(t, n0, n, round, A, lda, rot, pairs);
+    for (int64_t t = tid; t < h; t += nthreads) jac_params_item(t, n0, n, round, A, lda, rot, pairs);
     grid_barrier(bar, bar + 1, gridDim.x, status);
-    for (int64_t i = tid; i < jac_items(h, n0); i += nthreads) jac_apply_item<R>(i, h, n0, A, lda, V, ldv, rot, pairs);
+    for (int64_t i = tid; i < jac_items(h, n0); i += nthreads) jac_apply_item(i, h, n0, A, lda, V, ldv, rot, pairs);
     grid_barrier(bar, bar + 1, gridDim.x, status);
   }
 }
@@ -384,17 +368,16 @@ __global__ void k_offnorm_sum(int nparts, const double* part, double* out) {
 }
 
 // Sort eigenpairs ascending (stable): rank by counting, then permute w and the columns of V.
-template <typename R>
-__global__ void k_eig_sort(int64_t n, const cplx<R>* __restrict__ A, int64_t lda, const cplx<R>* __restrict__ Vin,
-                           int64_t ldvi, R* __restrict__ w, cplx<R>* __restrict__ Vout, int64_t ldvo) {
+__global__ void k_eig_sort(int64_t n, const double2* __restrict__ A, int64_t lda, const double2* __restrict__ Vin,
+                           int64_t ldvi, double* __restrict__ w, double2* __restrict__ Vout, int64_t ldvo) {
   const int64_t i = blockIdx.x;
   __shared__ int64_t rank;
-  const R wi = A[i + i * lda].x;
+  const double wi = A[i + i * lda].x;
   if (threadIdx.x == 0) rank = 0;
   __syncthreads();
   int64_t cnt = 0;
   for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-    const R wj = A[j + j * lda].x;
+    const double wj = A[j + j * lda].x;
     if (wj < wi || (wj == wi && j < i)) ++cnt;
   }
   atomicAdd((unsigned long long*)&rank, (unsigned long long)cnt);
@@ -404,38 +387,26 @@ __global__ void k_eig_sort(int64_t n, const cplx<R>* __restrict__ A, int64_t lda
   for (int64_t k = threadIdx.x; k < n; k += blockDim.x) Vout[k + r * ldvo] = Vin[k + i * ldvi];
 }
 
-template <typename C> __global__ void k_identity_t(int64_t n, C* A, int64_t lda) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int64_t i = idx % n, j = idx / n;
-  A[i + j * lda] = cmake<C>(i == j ? 1.0 : 0.0, 0.0);
-}
-template <typename R> void set_identity_t(int64_t n, cplx<R>* A, int64_t lda, cudaStream_t st) {
-  CHEBFI_LAUNCH("k_identity", st, k_identity_t<cplx<R>><<<nblk(n * n), 256, 0, st>>>(n, A, lda));
-}
-
-template <typename R>
-void jacobi_eigh_t(int64_t n0, cplx<R>* A, int64_t lda, R* w, cplx<R>* V, int64_t ldv, int* status, cudaStream_t st,
-                   DevBuf<double2>* ws, double tol_conv, double tol_stall, bool report) {
-  using C = cplx<R>;
+void jacobi_scalar(int64_t n0, double2* A, int64_t lda, double* w, double2* V, int64_t ldv, int* status, cudaStream_t st,
+                   DevBuf<double2>* ws) {
+  constexpr double tol_conv = 1e-15, tol_stall = 1e-12;
   if (n0 <= 0) return;
   const int64_t n = n0 + (n0 & 1);  // a padding player never paired for real
   // workspace (in double2 units): rotations, pair list, norm partials, barrier, a copy of V
   constexpr int kParts = 256;
-  const size_t rot_c = (size_t)(n / 2) * sizeof(RotT<R>) / sizeof(double2) + 1;
+  const size_t rot_c = (size_t)(n / 2) * sizeof(Rot) / sizeof(double2) + 1;
   const size_t pair_c = (size_t)n * sizeof(int) / sizeof(double2) + 1;
   const size_t part_c = kParts + 2;
-  const size_t vtmp = ((size_t)n0 * n0 * sizeof(C) + sizeof(double2) - 1) / sizeof(double2);
-  ws->alloc(rot_c + pair_c + part_c + 1 + vtmp);
-  RotT<R>* rot = reinterpret_cast<RotT<R>*>(ws->p);
+  ws->alloc(rot_c + pair_c + part_c + 1 + (size_t)n0 * n0);
+  Rot* rot = reinterpret_cast<Rot*>(ws->p);
   int* pairs = reinterpret_cast<int*>(ws->p + rot_c);
   double* part = reinterpret_cast<double*>(ws->p + rot_c + pair_c);
   double* nrm = part + 2 * kParts;
   unsigned* bar = reinterpret_cast<unsigned*>(ws->p + rot_c + pair_c + part_c);
-  C* Vtmp = reinterpret_cast<C*>(ws->p + rot_c + pair_c + part_c + 1);
+  double2* Vtmp = reinterpret_cast<double2*>(ws->p + rot_c + pair_c + part_c + 1);
   if (n0 == 1) {
-    set_identity_t<R>(1, Vtmp, 1, st);
-    CHEBFI_LAUNCH("k_eig_sort", st, k_eig_sort<R><<<1, 32, 0, st>>>(1, A, lda, Vtmp, 1, w, V, ldv));
+    set_identity(1, Vtmp, 1, st);
+    CHEBFI_LAUNCH("k_eig_sort", st, k_eig_sort<<<1, 32, 0, st>>>(1, A, lda, Vtmp, 1, w, V, ldv));
     return;
   }
   CHEBFI_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), st));
@@ -444,15 +415,15 @@ void jacobi_eigh_t(int64_t n0, cplx<R>* A, int64_t lda, R* w, cplx<R>* V, int64_
   CHEBFI_CUDA(cudaGetDevice(&dev));
   CHEBFI_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   CHEBFI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  CHEBFI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jac_sweep<R>, 256, 0));
+  CHEBFI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jac_sweep, 256, 0));
   const int coop_blocks = sms * std::min(per_sm, 8);
-  set_identity_t<R>(n0, Vtmp, n0, st);
+  set_identity(n0, Vtmp, n0, st);
   const int max_sweeps = 40;
   const unsigned parts = (unsigned)std::min<int64_t>(kParts, std::max<int64_t>(1, n0 * n0 / 4096));
   double prev_off = INFINITY;
-  bool done = false;
+  bool done = false, report = true;
   for (int sweep = 0; sweep <= max_sweeps && !done; ++sweep) {
-    CHEBFI_LAUNCH("k_offnorm", st, k_offnorm_part<R><<<parts, 256, 0, st>>>(n0, A, lda, part));
+    CHEBFI_LAUNCH("k_offnorm", st, k_offnorm_part<double><<<parts, 256, 0, st>>>(n0, A, lda, part));
     CHEBFI_LAUNCH("k_offnorm", st, k_offnorm_sum<<<1, 32, 0, st>>>((int)parts, part, nrm));
     double hn[2];
     CHEBFI_CUDA(cudaMemcpyAsync(hn, nrm, sizeof(hn), cudaMemcpyDeviceToHost, st));
@@ -474,21 +445,21 @@ void jacobi_eigh_t(int64_t n0, cplx<R>* A, int64_t lda, R* w, cplx<R>* V, int64_
     prev_off = off;
     if (coop && coop_blocks > 0) {
       int64_t n0a = n0, na = n, ldaa = lda, ldva = n0;
-      C* Aa = A;
-      C* Va = Vtmp;
+      double2* Aa = A;
+      double2* Va = Vtmp;
       void* args[] = {&n0a, &na, &Aa, &ldaa, &Va, &ldva, &rot, &pairs, &bar, &status};
       // work: per round every entry of A gets two rotations and every entry of V one, about
       // 11 real flops per complex entry per rotation: 33 n^3 per sweep
       CHEBFI_LAUNCH_W("k_jac_sweep", st, 33.0 * (double)n0 * (double)n0 * (double)n0,
-                      CHEBFI_CUDA(cudaLaunchCooperativeKernel((const void*)k_jac_sweep<R>, dim3(coop_blocks),
+                      CHEBFI_CUDA(cudaLaunchCooperativeKernel((const void*)k_jac_sweep, dim3(coop_blocks),
                                                               dim3(256), args, 0, st)));
     } else {
       for (int64_t round = 0; round < n - 1; ++round) {
         CHEBFI_LAUNCH("k_jac_params", st,
-                      k_jac_params<R><<<nblk(n / 2), 256, 0, st>>>(n0, n, round, A, lda, rot, pairs));
+                      k_jac_params<<<nblk(n / 2), 256, 0, st>>>(n0, n, round, A, lda, rot, pairs));
         const int64_t h = n / 2;
         CHEBFI_LAUNCH("k_jac_apply", st,
-                      k_jac_apply<R><<<nblk(jac_items(h, n0)), 256, 0, st>>>(h, n0, A, lda, Vtmp, n0, rot, pairs));
+                      k_jac_apply<<<nblk(jac_items(h, n0)), 256, 0, st>>>(h, n0, A, lda, Vtmp, n0, rot, pairs));
       }
     }
   }
@@ -498,7 +469,7 @@ void jacobi_eigh_t(int64_t n0, cplx<R>* A, int64_t lda, R* w, cplx<R>* V, int64_
     CHEBFI_CUDA(cudaMemcpyAsync(status, &code, sizeof(int), cudaMemcpyHostToDevice, st));
     CHEBFI_CUDA(cudaStreamSynchronize(st));
   }
-  CHEBFI_LAUNCH("k_eig_sort", st, k_eig_sort<R><<<(unsigned)n0, 128, 0, st>>>(n0, A, lda, Vtmp, n0, w, V, ldv));
+  CHEBFI_LAUNCH("k_eig_sort", st, k_eig_sort<<<(unsigned)n0, 128, 0, st>>>(n0, A, lda, Vtmp, n0, w, V, ldv));
 }
 
 
@@ -627,7 +598,7 @@ __global__ void __launch_bounds__(256) k_cluster_solve(int64_t n, const int* __r
                                                        double2* X, double* __restrict__ lam, int* status) {
   constexpr int P = kMaxCluster + 1;
   __shared__ double2 A[kMaxCluster * P], Z[kMaxCluster * P];
-  __shared__ RotT<double> rot[kMaxCluster / 2];
+  __shared__ Rot rot[kMaxCluster / 2];
   __shared__ int pairs[kMaxCluster];
   __shared__ double norms[2];
   const int* id = idx + off[blockIdx.x];
@@ -678,10 +649,10 @@ __global__ void __launch_bounds__(256) k_cluster_solve(int64_t n, const int* __r
     if (sweep == 40 || !(t < INFINITY)) break;
     prev = o;
     for (int r = 0; r < kp - 1; ++r) {
-      if (tid < kp / 2) jac_params_item<double>(tid, k, kp, r, A, P, rot, pairs);
+      if (tid < kp / 2) jac_params_item(tid, k, kp, r, A, P, rot, pairs);
       __syncthreads();
       for (int i = tid; i < (int)jac_items(kp / 2, k); i += blockDim.x)
-        jac_apply_item<double>(i, kp / 2, k, A, P, Z, P, rot, pairs);
+        jac_apply_item(i, kp / 2, k, A, P, Z, P, rot, pairs);
       __syncthreads();
     }
   }
@@ -842,7 +813,7 @@ __device__ void solve_shared(float2* S, float2* W, int sweeps, float tol) {
       const float app = S[p + P * p].x, aqq = S[q + P * q].x;
       const float g2 = h.x * h.x + h.y * h.y;
       float c = 1.f, s = 0.f, px = 1.f, py = 0.f;
-      if (g2 > 1e-36f && g2 > JacEps<float>::v * JacEps<float>::v * fabsf(app * aqq)) {
+      if (g2 > 1e-36f && g2 > kEpsF * kEpsF * fabsf(app * aqq)) {
         const float rg = rsqrtf(g2), zeta = 0.5f * (aqq - app) * rg;
         const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + __fsqrt_rn(fmaf(zeta, zeta, 1.f)));
         c = rsqrtf(fmaf(tt, tt, 1.f));
@@ -1019,6 +990,11 @@ __global__ void __launch_bounds__(256) k_bj_scale(int64_t n2, const double2* __r
   out[i] = make_float2((float)(A[i].x * f), (float)(A[i].y * f));
 }
 
+__global__ void k_bj_identity(int64_t n, float2* V) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < n * n) V[e] = make_float2(e % (n + 1) == 0 ? 1.f : 0.f, 0.f);
+}
+
 // zero-padded copy
 __global__ void k_bj_pad(int64_t n0, int64_t np, const float2* __restrict__ A, int64_t lda, float2* __restrict__ Ap) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1087,7 +1063,7 @@ void trsm_lower(int64_t n, int64_t m, const double2* L, int64_t ldl, double2* B,
 
 void jacobi_eigh(int64_t n0, double2* A, int64_t lda, double* w, double2* V, int64_t ldv, int* status, cudaStream_t st,
                  DevBuf<double2>* ws) {
-  jacobi_eigh_t<double>(n0, A, lda, w, V, ldv, status, st, ws, 1e-15, 1e-12, true);
+  jacobi_scalar(n0, A, lda, w, V, ldv, status, st, ws);
 }
 
 void scaled_to_f32(int64_t n, const double2* A, float2* out, int* emax, cudaStream_t st) {
@@ -1142,7 +1118,7 @@ bool jacobi_eigh_f32(int64_t n0, const float2* A, int64_t lda, float2* V, int64_
     return true;
   }
   CHEBFI_LAUNCH("k_bj_pad", st, bj::k_bj_pad<<<nblk((int64_t)nn), 256, 0, st>>>(n0, np, A, lda, Ap));
-  set_identity_t<float>(np, Vp, np, st);
+  CHEBFI_LAUNCH("k_identity", st, bj::k_bj_identity<<<nblk((int64_t)nn), 256, 0, st>>>(np, Vp));
   const size_t bytes = (size_t)2 * bj::S2 * bj::PS * sizeof(float2);
   const size_t sbytes = (size_t)3 * bj::S2 * bj::PS * sizeof(float2);
   CHEBFI_CUDA(cudaFuncSetAttribute(bj::k_bj_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbytes));

@@ -136,9 +136,8 @@ static inline void fill_twiddles() {
 template <typename R, int N3>
 __device__ __forceinline__ void zinv_body(const cplx<typename SphT<R>::type>* __restrict__ Y, int64_t ldy,
                                           cplx<R>* __restrict__ T, const FastArgs& fa,
-                                          const cplx<R>* __restrict__ twz, int c0, int64_t b,
+                                          int c0, int64_t b,
                                           unsigned char* smem_raw) {
-  (void)twz;
   const ConstTw<R, N3> tw;
   cplx<R>* lines = reinterpret_cast<cplx<R>*>(smem_raw);
   const int nc = min(kCBF, fa.ncol - c0);
@@ -403,12 +402,10 @@ __device__ __forceinline__ void plane_real_body(const cplx<R>* __restrict__ T, c
 // the epilogue (Z, its bf16 planes, and the Chebyshev combination T = a (Z - c Y) - b Yprev)
 template <typename R, int N3>
 __device__ __forceinline__ void zfwd_body(const cplx<R>* __restrict__ T, const FastArgs& fa,
-                                          const cplx<R>* __restrict__ twz,
                                           const typename SphT<R>::type* __restrict__ K,
                                           const LocalEpi<typename SphT<R>::type>& ep, int c0, int64_t b,
                                           unsigned char* smem_raw) {
   using CS = cplx<typename SphT<R>::type>;
-  (void)twz;
   const ConstTw<R, N3> tw;
   cplx<R>* lines = reinterpret_cast<cplx<R>*>(smem_raw);
   const int nc = min(kCBF, fa.ncol - c0);

@@ -36,9 +36,9 @@ template <typename R, int N> constexpr int zfwd_threads() {
 // SphT<R> (double for dfl), the column buffer and the planes in cplx<R>.
 template <typename R, int N3>
 __global__ void __launch_bounds__(zinv_threads<R, N3>()) k_zinv_f(const cplx<typename SphT<R>::type>* __restrict__ Y, int64_t ldy,
-                                                     cplx<R>* __restrict__ T, FastArgs fa, const cplx<R>* __restrict__ twz) {
+                                                     cplx<R>* __restrict__ T, FastArgs fa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fk::zinv_body<R, N3>(Y, ldy, T, fa, twz, blockIdx.x * kCBF, blockIdx.y, smem_raw);
+  fk::zinv_body<R, N3>(Y, ldy, T, fa, blockIdx.x * kCBF, blockIdx.y, smem_raw);
 }
 
 // Threads of an FP32 plane's block, measured over 64 to 768 per length: small planes run in
@@ -68,11 +68,10 @@ __global__ void __launch_bounds__(kThreads) k_plane_real_f(const cplx<R>* __rest
 
 template <typename R, int N3>
 __global__ void __launch_bounds__(zfwd_threads<R, N3>()) k_zfwd_f(const cplx<R>* __restrict__ T, FastArgs fa,
-                                                     const cplx<R>* __restrict__ twz,
                                                      const typename SphT<R>::type* __restrict__ K,
                                                      LocalEpi<typename SphT<R>::type> ep) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fk::zfwd_body<R, N3>(T, fa, twz, K, ep, blockIdx.x * kCBF, blockIdx.y, smem_raw);
+  fk::zfwd_body<R, N3>(T, fa, K, ep, blockIdx.x * kCBF, blockIdx.y, smem_raw);
 }
 
 template <typename R> void set_smem(const void* f, size_t bytes) {
@@ -90,7 +89,6 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
   const SphereFFT& s = ctx->sph;
   const FastArgs fa = fk::fast_args(ctx);
   CHEBFI_REQUIRE(s.pitch == fk::plane_pitch(N), CHEBFI_ERR_STATE, "plane pitch of the compile-time path");
-  const cplx<R>* tw = nullptr;  // the passes read their twiddles from constant tables
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>);
   const size_t pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
 #ifndef CHEBFI_FFT_DF
@@ -102,7 +100,7 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
     const int nbc = (int)std::min<int64_t>(65535, nb - b0);
     dim3 gz((s.ncol + kCBF - 1) / kCBF, nbc);
     const double esz = sizeof(cplx<R>), col = (double)N * s.ncol * nbc * esz, sph = (double)ctx->npw * nbc * esz;
-    CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, zinv_threads<R, N>(), zbytes, st>>>(Y + b0 * ldy, ldy, T, fa, tw));
+    CHEBFI_LAUNCH_W("k_zinv", st, sph + col, k_zinv_f<R, N><<<gz, zinv_threads<R, N>(), zbytes, st>>>(Y + b0 * ldy, ldy, T, fa));
     if (!fixed_planes(ctx, nbc, T, st)) {
 #ifndef CHEBFI_FFT_DF
       CHEBFI_LAUNCH_W("k_plane", st, 2.0 * col, k_plane_f<R, N><<<dim3(N, nbc), plane_threads<R, N>(), pbytes, st>>>(T, vtable<R>(ctx), fa));
@@ -122,7 +120,7 @@ void fast_launch(chebfi_ctx* ctx, const cplx<typename SphT<R>::type>* Y, int64_t
     e.inv_n3 = (S)(1.0 / ((double)N * N * N));
     const double epi = sph * (1.0 + (e.Z ? 1.0 : 0.0) + (e.T ? 1.0 : 0.0) + (e.Yprev ? 1.0 : 0.0)) +
                        (e.Zhi ? (double)ctx->npw * nbc * (e.zplane ? 12.0 : 8.0) : 0.0);
-    CHEBFI_LAUNCH_W("k_zfwd", st, col + epi, k_zfwd_f<R, N><<<gz, zfwd_threads<R, N>(), zbytes, st>>>(T, fa, tw, K, e));
+    CHEBFI_LAUNCH_W("k_zfwd", st, col + epi, k_zfwd_f<R, N><<<gz, zfwd_threads<R, N>(), zbytes, st>>>(T, fa, K, e));
   }
 }
 
@@ -134,10 +132,9 @@ void real_launch(chebfi_ctx* ctx, const cplx<R>* Y, int64_t ldy, int64_t nb, cpl
   const FastArgs fa = fk::fast_args(ctx);
   CHEBFI_REQUIRE(nb <= 65535, CHEBFI_ERR_ARG, "too many bands in a chunk");
   const size_t zbytes = (size_t)(kCBF * s.zpitch) * sizeof(cplx<R>), pbytes = (size_t)(N * s.pitch) * sizeof(cplx<R>);
-  const cplx<R>* tw = nullptr;
   set_smem<R>((const void*)k_zinv_f<R, N>, zbytes);
   const dim3 gz((s.ncol + kCBF - 1) / kCBF, (unsigned)nb);
-  CHEBFI_LAUNCH("k_zinv", st, k_zinv_f<R, N><<<gz, zinv_threads<R, N>(), zbytes, st>>>(Y, ldy, T, fa, tw));
+  CHEBFI_LAUNCH("k_zinv", st, k_zinv_f<R, N><<<gz, zinv_threads<R, N>(), zbytes, st>>>(Y, ldy, T, fa));
   if (!planes) return;
   set_smem<R>((const void*)k_plane_real_f<R, N>, pbytes);
   CHEBFI_LAUNCH("k_plane_real", st, k_plane_real_f<R, N><<<dim3(N, (unsigned)nb), kThreads, pbytes, st>>>(T, out, fa));
