@@ -294,17 +294,22 @@ int chebfi_apply_H_noalloc(chebfi_ctx* ctx, const void* Y, void* HY, int64_t nb,
  * op(B) is scaled by a power of two to a 2-norm in [2^(E-1), 2^E) and rounded to integers,
  * one tensor-core GEMM per modulus computes the product of their residues exactly, and the
  * Chinese remainder theorem recovers the integer product.  The result's error is about
- * 2^-E ||row of op(A)|| ||column of op(B)|| per entry, E = 53 with the default 14 moduli:
- * no larger than an FP64 dot product's.  The paper (FP64 BLAS on CPUs) has no counterpart. */
+ * 2^-E ||row of op(A)|| ||column of op(B)|| per entry, E = 53 with the default 14 moduli (the
+ * order of an FP64 dot product's) and 57 with 15.  The bound is in norms: an entry keeps E bits of
+ * its row's norm, not of itself, so where large entries of a row meet only small ones of a column
+ * and the reverse, FP64 sums are more exact.  Rows of any scale work; a row with an infinity or a
+ * NaN makes its products NaN.  The paper (FP64 BLAS on CPUs) has no counterpart. */
 enum {
-  CHEBFI_GEMM_AUTO = 0,        /* tensor cores when K >= 64 and 8 M N K >= 6e7, else CUDA cores */
+  CHEBFI_GEMM_AUTO = 0,        /* tensor cores when K >= 64 and 8 M N K >= 6e7 (with 15 moduli below
+                                  1e9), else CUDA cores */
   CHEBFI_GEMM_CUDA_CORES = 1,  /* FP64 FMA on the CUDA cores only */
   CHEBFI_GEMM_TENSOR = 2       /* the modular emulation for every product */
 };
 /* Select the engine (a CHEBFI_GEMM_* value) and the modulus count of the emulation (8..15;
  * 0 keeps the current one, initially 14; fewer moduli run faster with a smaller E: 8 -> 30,
  * 10 -> 38, 12 -> 45, 14 -> 53, 15 -> 57).  *precision_bits (nullable) receives E.  The
- * emulation keeps residues of P (about 2 x nmod x 4 N_pw N_proj bytes) once used. */
+ * emulation keeps residues of P and P^H (6 nmod N_pw N_proj bytes each) and of the projection
+ * space's G and M (6 nmod N_proj^2 bytes each) once used. */
 int chebfi_set_fp64_gemm(chebfi_ctx* ctx, int engine, int nmod, int* precision_bits);
 
 /* Complex FP64 GEMM through the context's engine selection: C = alpha op(A) op(B) + beta C,

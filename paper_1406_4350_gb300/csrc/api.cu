@@ -178,12 +178,21 @@ bool use_tensor_fp64(const chebfi_ctx* ctx, int64_t M, int64_t N, int64_t K) {
   return K >= 64 && 8.0 * (double)M * (double)N * (double)K >= 6e7;
 }
 
-// residues of P^H (conj) or P as the A operand, kept while the modulus count is unchanged
-const OzOperand& oz_P(chebfi_ctx* ctx, bool conj, cudaStream_t st) {
-  OzOperand& o = conj ? ctx->ozPh : ctx->ozP;
-  if (o.nmod != ctx->oz_nmod)
-    oz_prepare(ctx->d_P.p, ctx->npw, conj ? ctx->nproj : ctx->npw, conj ? ctx->npw : ctx->nproj, conj, conj,
-               ctx->oz_nmod, o, st);
+// Modulus count of a product on the tensor cores: the context's from 1e9 flops up.  Smaller ones,
+// which the library would run on the FP64 units but for their speed, take all 15: rounding the
+// operands to 57 bits of their rows' norms keeps them at least as exact as those units, at 1/14
+// more work of a product that its launches bound (rms error in 2^-53 of |a| |b|, FP64 units / 14 /
+// 15 moduli: random 256^3 0.40 / 1.06 / 0.07, 200 x 30 x 6000 0.14 / 0.88 / 0.06; 256 x 256 x 256
+// G p of the 48^3 cell 3.9 / 17.9 / 1.2, Y^H Y 3.9 / 5.6 / 0.4).
+int fp64_moduli(const chebfi_ctx* ctx, int64_t M, int64_t N, int64_t K) {
+  return ctx->fp64_gemm == CHEBFI_GEMM_AUTO && 8.0 * (double)M * (double)N * (double)K < 1e9 ? kOzMaxMod : ctx->oz_nmod;
+}
+
+// residues of P^H (conj) or P as the A operand, kept for each count (the context's, or all)
+const OzOperand& oz_P(chebfi_ctx* ctx, bool conj, int nmod, cudaStream_t st) {
+  OzOperand& o = (conj ? ctx->ozPh : ctx->ozP)[nmod == kOzMaxMod];
+  if (o.nmod != nmod)
+    oz_prepare(ctx->d_P.p, ctx->npw, conj ? ctx->nproj : ctx->npw, conj ? ctx->npw : ctx->nproj, conj, conj, nmod, o, st);
   return o;
 }
 
@@ -197,21 +206,22 @@ void gemm64(chebfi_ctx* ctx, bool conjA, bool conjB, int64_t M, int64_t N, int64
   }
   OzWork& z = ctx->oz;
   const OzOperand* a = &z.A;
+  const int nmod = fp64_moduli(ctx, M, N, K);
   const bool is_P = ctx->has_proj && A == ctx->d_P.p && lda == ctx->npw &&
                     (conjA ? (M == ctx->nproj && K == ctx->npw) : (M == ctx->npw && K == ctx->nproj));
   const bool square = ctx->has_proj && !conjA && lda == ctx->nproj && M == ctx->nproj && K == ctx->nproj;
   if (is_P) {
-    a = &oz_P(ctx, conjA, st);
+    a = &oz_P(ctx, conjA, nmod, st);
   } else if (square && (A == ctx->d_G.p || A == ctx->d_M.p)) {
     // the Woodbury core's constant matrices: three of a filter step's products, whose operand
     // preparation costs as much as the product
-    OzOperand& o = A == ctx->d_G.p ? ctx->ozG : ctx->ozM;
-    if (o.nmod != ctx->oz_nmod) oz_prepare(A, lda, M, K, false, false, ctx->oz_nmod, o, st);
+    OzOperand& o = (A == ctx->d_G.p ? ctx->ozG : ctx->ozM)[nmod == kOzMaxMod];
+    if (o.nmod != nmod) oz_prepare(A, lda, M, K, false, false, nmod, o, st);
     a = &o;
   } else {
-    oz_prepare(A, lda, M, K, conjA, conjA, ctx->oz_nmod, z.A, st);
+    oz_prepare(A, lda, M, K, conjA, conjA, nmod, z.A, st);
   }
-  oz_prepare(B, ldb, N, K, !conjB, conjB, ctx->oz_nmod, z.B, st);
+  oz_prepare(B, ldb, N, K, !conjB, conjB, nmod, z.B, st);
   oz_gemm(*a, z.B, alpha, beta, C, ldc, lower, z.R, ctx->d_status.p, st, tag);
 }
 
@@ -1486,7 +1496,8 @@ int chebfi_set_projectors(chebfi_ctx* ctx, int64_t nproj, const void* P, int64_t
   ctx->paw = false;
   ctx->bound_rigorous = -1.0;
   ctx->has_proj = false;
-  ctx->ozPh.nmod = ctx->ozP.nmod = ctx->ozG.nmod = ctx->ozM.nmod = 0;  // residues of the previous P are stale
+  for (int i = 0; i < 2; ++i)  // residues of the previous P are stale
+    ctx->ozPh[i].nmod = ctx->ozP[i].nmod = ctx->ozG[i].nmod = ctx->ozM[i].nmod = 0;
   ctx->tc_ready = ctx->tcP_ready = ctx->tc3_ready = false;  // and so are its bf16 embeddings
   if (nproj == 0) {
     ctx->has_proj = true;

@@ -338,7 +338,8 @@ struct chebfi_ctx {
   int eig_iters = 0;               // refinement steps of its last call (0: FP64 Jacobi ran)
   int oz_nmod = 14;
   chebfi::OzWork oz;
-  chebfi::OzOperand ozPh, ozP, ozG, ozM;  // residues of P^H, P, G and M as A operands (nmod 0: to be built)
+  // residues of P^H, P, G and M as A operands, by oz_nmod moduli and by all of them (nmod 0: to be built)
+  chebfi::OzOperand ozPh[2], ozP[2], ozG[2], ozM[2];
   double bound_rigorous = -1.0;
   double smin = 1.0;  // lower bound of lambda_min(S), set with bound_rigorous
   // host-block filter: staging buffers, copy streams and their events (created on first use)

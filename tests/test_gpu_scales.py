@@ -161,3 +161,38 @@ def test_local_potential_of_any_size(n, e):
     assert np.abs(one - ref).max() <= 1e-11 * np.abs(ref).max()  # the FP64 form's parity tolerance
     got = _np(_ctx(_without_kinetic(n, scale=2.0 ** e)).apply_H(_F(cell.Y0))) * 2.0 ** -e
     assert np.abs(got - one).max() <= 2.0 ** -46 * np.abs(one).max()
+
+
+# products that the FP64 units would take longer for, and that no caller has asked to round
+# differently: no less exact than on those units, entry by entry and on operands of this library
+@pytest.mark.parametrize("what", ["square", "deep", "PhY", "Gp", "gram"])
+def test_products_of_middle_size_are_as_exact_as_fp64(what):
+    from paper_1406_4350_gb300._lib import GEMM_CUDA_CORES
+    rng = np.random.default_rng(44)
+
+    def rand(*s):
+        return rng.standard_normal(s) + 1j * rng.standard_normal(s)
+    if what == "square":
+        A, B = rand(256, 256), rand(256, 256)
+    elif what == "deep":
+        A, B = rand(6000, 200), rand(6000, 30)
+    else:
+        cell = make_cell(12.0, 30, 8.0, 32, 8, 128, True, 45)
+        p = cell.P.conj().T @ cell.Y0
+        A, B = {"PhY": (cell.P, cell.Y0), "Gp": (cell.P.conj().T @ cell.P, p), "gram": (cell.Y0, cell.Y0)}[what]
+    m, n = A.shape[1], B.shape[1]
+    assert 6e7 <= 8.0 * m * n * A.shape[0] < 1e9
+    i, j = rng.integers(0, m, 200), rng.integers(0, n, 200)
+    ref = np.array([(A[:, a].conj().astype(np.clongdouble) * B[:, b].astype(np.clongdouble)).sum()
+                    for a, b in zip(i, j)])
+    size = np.array([(np.abs(A[:, a]) * np.abs(B[:, b])).sum() for a, b in zip(i, j)])
+    err = []
+    for engine in (None, GEMM_CUDA_CORES):
+        g = _ctx()
+        if engine is not None:
+            g.set_fp64_gemm(engine)
+        g.profile(True)
+        C = _np(g.gemm_fp64(_F(A), _F(B), conjA=True))
+        assert ("k_oz_gemm" in g.profile_totals()) == (engine is None)
+        err.append(np.sqrt(np.mean((np.abs((C[i, j] - ref).astype(complex)) / size) ** 2)))
+    assert err[0] <= err[1], (err[0] / U, err[1] / U)
