@@ -16,6 +16,15 @@ def test_operand_without_planes_is_not_marked_prepared(tmp_path):
     assert code != 0 and nmod == 0
 
 
+@needs_nvcc
+def test_two_pass_fft_code_on_host_at_every_compiled_length(tmp_path):
+    rows = run("fft_lengths_check", tmp_path)
+    assert [int(r[0]) for r in rows] == [16, 20, 24, 30, 32, 36, 40, 45, 48, 54, 60, 64, 72, 80, 90, 96, 100, 108]
+    for n, f64, g64, f32, g32 in rows:  # the tolerances of the check at the other lengths
+        assert f64 < 2e-15 and g64 < 2e-15, n
+        assert f32 < 1e-6 and g32 < 1e-6, n
+
+
 @pytest.mark.gpu
 def test_lower_product_with_split_keeps_the_upper_triangle(tmp_path):
     rows = run("lower_split_check", tmp_path)
