@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <vector>
 
 #include "internal.cuh"
 #include "kernels.cuh"
@@ -793,10 +794,8 @@ struct ModSet {
 };
 
 // moduli, E and the CRT constants of the first n moduli (host, 128-bit arithmetic)
-const ModSet& modset(int n) {
-  static ModSet sets[kOzMaxMod + 1];
-  ModSet& s = sets[n];
-  if (s.n == n) return s;
+ModSet make_modset(int n) {
+  ModSet s{};
   unsigned __int128 M = 1;
   double l2 = 0.0;
   for (int i = 0; i < n; ++i) {
@@ -819,6 +818,15 @@ const ModSet& modset(int n) {
   s.E = std::min(62, (int)std::floor((l2 - 3.0) / 2.0));
   s.n = n;
   return s;
+}
+// built once, whichever thread comes first
+const ModSet& modset(int n) {
+  static const std::vector<ModSet> sets = [] {
+    std::vector<ModSet> v(kOzMaxMod + 1);
+    for (int k = kOzMinMod; k <= kOzMaxMod; ++k) v[k] = make_modset(k);
+    return v;
+  }();
+  return sets[n];
 }
 
 }  // namespace oz
