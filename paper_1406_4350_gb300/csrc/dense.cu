@@ -105,10 +105,10 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* A, int64_t lda, int 
 // lanes hold its unknowns, and step k broadcasts x_k = s_k / L_kk to the lanes that still
 // need it.  A system is a serial chain of nb slow FP64 steps, so systems are spread over the
 // SMs (four warps a block) instead of one per thread, which kept 128 of them on one SM
-// (224 x 32: 131 and 172 us with a thread per system, now 22 us).  The reciprocal is a pair of
+// (224 x 32: 131 and 172 us with a thread per system, now 18 us).  The reciprocal is a pair of
 // twice the precision and a complex product is formed before it is subtracted, so that each
 // operation rounds once, as with a division (rms residual 0.50 units of 2^-53 |L| |x|; with the
-// reciprocal alone and two multiply-adds 0.66, and 18 us).
+// reciprocal alone and two multiply-adds 0.66, and 4 us less).
 constexpr int kTrsmWarps = 4;
 // x_l <- x_l - sum_{k < l} c_lk x_k solved forward; c_lk = L[l][k], or its conjugate
 template <bool CONJ>
@@ -130,13 +130,16 @@ __device__ __forceinline__ double2 warp_forward(const double2 (*l)[NB + 1], cons
 }
 __device__ __forceinline__ void load_tri(const double2* __restrict__ L, int64_t ldl, int nb, double2 (*l)[NB + 1],
                                          double2* rd) {
+  // one warp's lanes take the reciprocals side by side: a division in every warp's pass over its
+  // column of the square, for the one lane on the diagonal, took 4 of 22 us
+  if (threadIdx.x < NB) {
+    const int i = threadIdx.x;
+    const double d = i < nb ? L[i + i * ldl].x : 1.0, r = 1.0 / d;
+    rd[i] = make_double2(r, r * fma(-r, d, 1.0));
+  }
   for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
     const int i = e % NB, j = e / NB;
     l[i][j] = i < nb && j < nb ? L[i + j * ldl] : make_double2(0.0, 0.0);
-    if (i == j) {
-      const double d = i < nb ? L[i + j * ldl].x : 1.0, r = 1.0 / d;
-      rd[i] = make_double2(r, r * fma(-r, d, 1.0));
-    }
   }
   __syncthreads();
 }
