@@ -277,10 +277,9 @@ int chebfi_solve(chebfi_ctx* ctx, void* Y, double* evals, double* resid, int64_t
  *  - Bands are processed in chunks that fit the array.  A problem whose single band needs
  *    more than 32 MiB of scratch (FFT column buffer N3 x columns, plus 2 npw + 2 nproj, in
  *    complex doubles) is rejected with CHEBFI_ERR_ARG and a message naming the sizes.
- *  - The first call on each device does one-time set-up with that device current: it looks
- *    up the array's device address (cudaGetSymbolAddress) and uploads the FFT twiddle tables
- *    to constant memory (a synchronous copy).  Make that first call before any stream
- *    capture.
+ *  - The first call on each device looks up the array's device address with that device
+ *    current (cudaGetSymbolAddress).  It copies nothing (the FFT tables went up with V_loc), so
+ *    it may be inside a stream capture.
  *  - All calls share the one array, which keeps the previous call's contents (nothing in it
  *    needs to start at zero); calls that overlap on the GPU (other streams, other contexts
  *    on the same device, other host threads) race on it. */
@@ -410,7 +409,8 @@ int chebfi_profile_entry(chebfi_ctx* ctx, int i, char* name, int name_len, doubl
  * take (k, tile) items from a device work queue), and the whole degree-n filter is captured
  * in a CUDA graph on first use and replayed afterwards.  Tile shapes of the grouped GEMMs are
  * chosen by timing every candidate on the batch (chebfi_batch_autotune; run implicitly by
- * the first filter call of each form). */
+ * the first filter call of each form).  The FP64 form runs on the FP64 units throughout; one
+ * chebfi_cheb_filter per k-point, which does not, is faster there. */
 typedef struct chebfi_batch chebfi_batch;
 
 /* kctx: nk fully set-up contexts (set_cell/sphere/vloc/projectors) on one device, with the
